@@ -26,20 +26,23 @@ using kmcdev::FULL_WARP;
 using kmcdev::HASH_PRIME;
 using u128 = unsigned __int128;
 
-constexpr int PART_WARPS = 4;        // trajectories per CTA
+constexpr int PART_WARPS = 1;        // trajectories per CTA: few trajectories spread over the SMs
 constexpr int PART_MAX_L = 128;
 constexpr int PART_PHASE_SLOTS = 64; // Philox phase index np = n*64 + p
 constexpr int PART_BLOCKS = 0, PART_STRIPES = 1;
 constexpr uint32_t PART_TAG_PERM = 2u;
-// shared memory per warp (64-bit words): bit rows, the domain order, the
-// class counts of every domain (int [64][10]), the rate sum R' of every
-// domain (u64 [64]), the fixed-point rates (u64 [16]) and, when the lattice
-// has at most PART_RC_ROWS domain rows (N_D x domain height), the class
-// counts of every domain row (u8 [rows][10], in 32-bit words)
-constexpr int PART_RC_ROWS = 512;
-constexpr int PART_OFF_ORDER = 2 * PART_MAX_L, PART_OFF_DCOUNT = PART_OFF_ORDER + 8,
-              PART_OFF_DR = PART_OFF_DCOUNT + 64 * 10 / 2, PART_OFF_ATAB = PART_OFF_DR + 64,
-              PART_OFF_RC = PART_OFF_ATAB + 16;
+// shared memory per warp (64-bit words): bit rows, the domains of the visits
+// (u8: the random orders of the schedules in use, or one colour schedule's
+// visits and after them their phases), each domain's neighbours (u8 [64][4]),
+// the class counts of every domain (u32 [64][12], ten used), the fixed-point
+// rates and their reciprocals (u64 [10][2]) and, when the lattice has at most
+// PART_RC_ROWS domain rows (N_D x domain height, padded to a multiple of 4),
+// the class counts of every domain row (u8 [N_D][10][rows])
+constexpr int PART_RC_ROWS = 768;
+constexpr int PART_ORDER_BYTES = 1024;
+constexpr int PART_OFF_ORDER = 2 * PART_MAX_L, PART_OFF_NBD = PART_OFF_ORDER + PART_ORDER_BYTES / 8,
+              PART_OFF_DCOUNT = PART_OFF_NBD + 64 * 4 / 8, PART_OFF_ATAB = PART_OFF_DCOUNT + 64 * 12 / 2,
+              PART_OFF_RC = PART_OFF_ATAB + 20;
 constexpr int PART_WARP_WORDS = PART_OFF_RC + PART_RC_ROWS * 10 / 8;
 
 struct PartParams {
@@ -139,29 +142,45 @@ __device__ __forceinline__ int select128(u128 m, uint32_t rr)
     return 64 + kmcdev::select_bit((uint64_t)(m >> 64), rr - pl);
 }
 
-// Class 5 up + (number of up neighbours) of site (x, y), from the live rows.
-__device__ __forceinline__ int site_class(const uint64_t *rows, int x, int y, int L)
+// Class 5 up + (number of up neighbours) of site (x, y), from the live rows
+// (32-bit words, four per row).
+__device__ __forceinline__ int site_class(const uint32_t *row32, int x, int y, int L)
 {
     const int xm = (x == 0) ? L - 1 : x - 1, xp = (x == L - 1) ? 0 : x + 1;
     const int ym = (y == 0) ? L - 1 : y - 1, yp = (y == L - 1) ? 0 : y + 1;
-    auto bit = [&](int xx, int yy) { return (int)((rows[2 * yy + (xx >> 6)] >> (xx & 63)) & 1ull); };
+    auto bit = [&](int xx, int yy) { return (int)((row32[4 * yy + (xx >> 5)] >> (xx & 31)) & 1u); };
     return 5 * bit(x, y) + bit(xm, y) + bit(xp, y) + bit(x, ym) + bit(x, yp);
 }
 
+// One warp runs one trajectory's steps in windows of 32 consecutive steps of
+// its sequence (schedule after schedule, visit after visit), whatever visits
+// they belong to: lane i draws step i of the window and holds its domain,
+// its target and that domain's cumulative class rates.  A null step changes
+// nothing, so one ballot of target < R' over the lanes finds the next real
+// event of the whole window, in whichever visit it falls; every lane has
+// formed its own step's class and member index by then, and after the event
+// each lane forms its domain's rates again from the class counts in shared
+// memory.  What a trajectory costs is thus one chain per real event (about
+// one step in eight at T = 2.4) and a fixed part per 32 steps, where a loop
+// over visits paid a fixed part per visit.  Records between the window's
+// steps come from per-lane copies of the bond sum and the magnetisation and
+// from the inclusive products of the clock variates; the lanes at whose
+// steps a pass with a record ends write them side by side.
 template <bool EXPO>
 __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams P)
 {
-    extern __shared__ uint64_t part_smem[];
+    extern __shared__ __align__(16) uint64_t part_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tr = blockIdx.x * PART_WARPS + warp;
     if (tr >= P.n_traj) return; // whole warps only; no CTA-wide barrier below
-    const int L = P.L;
+    const int L = P.L, ND = P.ND;
     uint64_t *rows = part_smem + (size_t)warp * PART_WARP_WORDS;
+    uint32_t *row32 = reinterpret_cast<uint32_t *>(rows);
     uint8_t *order = reinterpret_cast<uint8_t *>(rows + PART_OFF_ORDER);
-    int *dcount = reinterpret_cast<int *>(rows + PART_OFF_DCOUNT);              // [N_D][10] class counts
-    unsigned long long *dR = reinterpret_cast<unsigned long long *>(rows + PART_OFF_DR); // [N_D] R'
-    uint64_t *Atab = rows + PART_OFF_ATAB;                                       // [10] A_c
-    uint8_t *rc = reinterpret_cast<uint8_t *>(rows + PART_OFF_RC);               // [N_D * H][10]
+    uint8_t *nbd = reinterpret_cast<uint8_t *>(rows + PART_OFF_NBD);          // [N_D][4] W, E, N, S domains
+    uint32_t *dcount = reinterpret_cast<uint32_t *>(rows + PART_OFF_DCOUNT);  // [N_D][12] class counts
+    ulonglong2 *atab = reinterpret_cast<ulonglong2 *>(rows + PART_OFF_ATAB);  // [10] A_c, floor((2^64 - 1) / A_c)
+    uint8_t *rc = reinterpret_cast<uint8_t *>(rows + PART_OFF_RC);            // [N_D][10][Hp]
     const u128 Lm = (L == 128) ? ~(u128)0 : (((u128)1 << L) - 1);
     const int8_t *sp = P.spins + (size_t)tr * L * L;
 
@@ -184,234 +203,108 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
     if (__any_sync(FULL_WARP, bad) && lane == 0) atomicOr(P.err, 1);
     __syncwarp();
 
-    uint64_t A = 0;
-    if (lane < 10) A = P.A[(size_t)tr * 10 + lane];
-    // 1/A_c from below (A_c rounded up, its reciprocal rounded down)
-    const float invAf = (lane < 10) ? __frcp_rd(kmcdev::u64_to_float_ru(A)) : 0.0f;
+    uint64_t A[10];
+#pragma unroll
+    for (int c = 0; c < 10; ++c) A[c] = P.A[(size_t)tr * 10 + c];
     const uint64_t seed = P.seed[tr];
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     const double hr = P.h[tr];
     uint64_t H = P.hash[tr], clkM = P.clkM[tr];
-    int64_t clkE = P.clkE[tr], flips = P.flips[tr], steps = P.steps[tr];
-    const int W = P.W, Hd = P.H, RPL = (Hd + 31) / 32, k = P.k;
+    int64_t clkE = P.clkE[tr], flips = P.flips[tr];
+    const int64_t steps0 = P.steps[tr];
+    // lane l holds domain rows l*RPL .. l*RPL+RPL-1, RPL a power of two
+    const int W = P.W, Hd = P.H, RPL = Hd <= 32 ? 1 : Hd <= 64 ? 2 : 4, k = P.k;
+    const int Hp = (Hd + 3) & ~3;
     const u128 DM0 = (W == 128) ? ~(u128)0 : (((u128)1 << W) - 1);
     const uint64_t M = P.M;
+    const bool stripes = P.kind == PART_STRIPES;
+    const int nbx = stripes ? ND : P.Dx, nby = stripes ? 1 : P.Dx; // domains per row and column
 
-    auto domain_origin = [&](int d, int &x0, int &y0) {
-        if (P.kind == PART_STRIPES) {
-            x0 = d * W;
-            y0 = 0;
-        } else {
-            x0 = (d % P.Dx) * W;
-            y0 = (d / P.Dx) * W;
-        }
-    };
+    const bool use_rc = ND * Hp <= PART_RC_ROWS;
+    if (lane < 10) {
+        const uint64_t Al = P.A[(size_t)tr * 10 + lane];
+        atab[lane] = make_ulonglong2(Al, Al ? ~0ull / Al : 0ull);
+    }
+    for (int d = lane; d < ND; d += 32) {
+        const int bx = d % nbx, by = d / nbx;
+        nbd[4 * d + 0] = (uint8_t)(by * nbx + (bx == 0 ? nbx - 1 : bx - 1));
+        nbd[4 * d + 1] = (uint8_t)(by * nbx + (bx == nbx - 1 ? 0 : bx + 1));
+        nbd[4 * d + 2] = (uint8_t)((by == 0 ? nby - 1 : by - 1) * nbx + bx);
+        nbd[4 * d + 3] = (uint8_t)((by == nby - 1 ? 0 : by + 1) * nbx + bx);
+    }
     // class counts of every domain (and of every domain row, when they
-    // fit) and every domain's rate sum, kept up to date flip by flip
-    const bool use_rc = P.ND * Hd <= PART_RC_ROWS;
-    if (lane < 10) Atab[lane] = A;
-    for (int d = 0; d < P.ND; ++d) {
-        int x0, y0;
-        domain_origin(d, x0, y0);
-        const uint32_t n = part_counts(rows, lane, y0, Hd, RPL, L, Lm, DM0 << x0);
-        if (lane < 10) dcount[d * 10 + lane] = (int)n;
-        const uint64_t R0 = __shfl_sync(FULL_WARP, kmcdev::prefix16((uint64_t)n * A, lane), 9);
-        if (lane == 0) dR[d] = R0;
+    // fit), kept up to date flip by flip
+    for (int d = 0; d < ND; ++d) {
+        const int x0 = (d % nbx) * W, y0 = (d / nbx) * Hd;
+        const uint32_t n = part_counts(rows, lane, y0, Hd, (Hd + 31) / 32, L, Lm, DM0 << x0);
+        if (lane < 12) dcount[d * 12 + lane] = n;
         if (use_rc) {
-            for (int yy = lane; yy < Hd; yy += 32) {
-                const RowPlanes pr = row_planes(rows, y0 + yy, L, Lm, DM0 << x0);
-                for (int c = 0; c < 10; ++c) rc[(d * Hd + yy) * 10 + c] = (uint8_t)popc128(class_mask(pr, c));
+            for (int yy = lane; yy < Hp; yy += 32) {
+                const RowPlanes pr = row_planes(rows, y0 + min(yy, Hd - 1), L, Lm, DM0 << x0);
+                for (int c = 0; c < 10; ++c)
+                    rc[(d * 10 + c) * Hp + yy] = (yy < Hd) ? (uint8_t)popc128(class_mask(pr, c)) : (uint8_t)0;
             }
         }
     }
-    __syncwarp();
-    // a domain row's count byte: the 32-bit word holding it and its shift
-    auto rc_word = [&](int d, int yy, int c, int &sh) {
-        const int b = (d * Hd + yy) * 10 + c;
-        sh = 8 * (b & 3);
-        return reinterpret_cast<unsigned *>(rc) + (b >> 2);
-    };
-
-    // The real events among the steps held by lanes [lo, hi): lane i holds
-    // step j = i - lo + jbase of the visit (target tgt, ~0 for no step).
-    // Null runs are skipped by one ballot; each real event selects its class
-    // and member, flips, and updates the class counts of the domains the five
-    // touched sites belong to.
-    auto events = [&](int d, uint64_t np, int x0, int y0, u128 DM, uint64_t tgt, int lo, int hi, int jbase) {
-        // a visit without real events needs only the domain's rate sum
-        uint64_t R = dR[d];
-        if (!__any_sync(FULL_WARP, lane >= lo && lane < hi && tgt < R)) return;
-        uint32_t n_c = (lane < 10) ? (uint32_t)dcount[d * 10 + lane] : 0u;
-        uint64_t Wc = (uint64_t)n_c * A;
-        uint64_t Cinc = kmcdev::prefix16(Wc, lane);
-        int pos = lo;
-        while (true) {
-            const unsigned real = __ballot_sync(FULL_WARP, lane >= pos && lane < hi && tgt < R);
-            if (!real) break;
-            const int jx = __ffs(real) - 1;
-            const uint64_t t = __shfl_sync(FULL_WARP, tgt, jx);
-            const unsigned sel = __ballot_sync(FULL_WARP, lane < 10 && t < Cinc);
-            const int c = __ffs(sel) - 1;
-            // exact q = floor((t - C_{c-1}) / A_c) < n_c <= 16384 from an FP32
-            // estimate with every rounding toward the lower side (so it is q or
-            // q - 1) and one integer comparison, instead of a 64-bit division
-            const uint64_t xq = t - (Cinc - Wc);
-            uint32_t q = (uint32_t)__fmul_rz(kmcdev::u64_to_float_rz(xq), invAf);
-            q = (xq - (uint64_t)q * A >= A) ? q + 1u : q;
-            const uint32_t jj = __shfl_sync(FULL_WARP, q, c);
-            // jj-th member of class c in row-major order
-            uint32_t cl = 0;
-            for (int tt = 0; tt < RPL; ++tt) {
-                const int yy = lane * RPL + tt;
-                if (yy >= Hd) break;
-                cl += use_rc ? (uint32_t)rc[(d * Hd + yy) * 10 + c]
-                             : (uint32_t)popc128(class_mask(row_planes(rows, y0 + yy, L, Lm, DM), c));
-            }
-            uint32_t incl = cl;
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint32_t v = __shfl_up_sync(FULL_WARP, incl, off);
-                if (lane >= off) incl += v;
-            }
-            const uint32_t excl = incl - cl;
-            const unsigned win = __ballot_sync(FULL_WARP, jj >= excl && jj < incl);
-            if (!win) {
-                if (lane == 0) atomicOr(P.err, 2);
-                break;
-            }
-            const int wl = __ffs(win) - 1;
-            uint32_t yx = 0;
-            if (lane == wl) {
-                uint32_t rr = jj - excl;
-                for (int tt = 0; tt < RPL; ++tt) {
-                    const int yy = lane * RPL + tt;
-                    if (use_rc) {
-                        // the row from its count, then that row's class mask alone
-                        const uint32_t pc = rc[(d * Hd + yy) * 10 + c];
-                        if (rr < pc) {
-                            const u128 mk = class_mask(row_planes(rows, y0 + yy, L, Lm, DM), c);
-                            yx = ((uint32_t)yy << 8) | (uint32_t)select128(mk, rr);
-                            break;
-                        }
-                        rr -= pc;
-                        continue;
-                    }
-                    const u128 mk = class_mask(row_planes(rows, y0 + yy, L, Lm, DM), c);
-                    const uint32_t pc = (uint32_t)popc128(mk);
-                    if (rr < pc) {
-                        yx = ((uint32_t)yy << 8) | (uint32_t)select128(mk, rr);
-                        break;
-                    }
-                    rr -= pc;
-                }
-            }
-            yx = __shfl_sync(FULL_WARP, yx, wl);
-            const int yy = (int)(yx >> 8), x = (int)(yx & 255u);
-            // the flip changes the classes of the site and its four
-            // neighbours (lanes 0..4); their domains' counts follow
-            const int y = y0 + yy;
-            int sx = x, sy = y;
-            if (lane == 1) sx = (x == 0) ? L - 1 : x - 1;
-            if (lane == 2) sx = (x == L - 1) ? 0 : x + 1;
-            if (lane == 3) sy = (y == 0) ? L - 1 : y - 1;
-            if (lane == 4) sy = (y == L - 1) ? 0 : y + 1;
-            const bool mine = lane < 5 && !(L == 2 && (lane == 2 || lane == 4)); // L = 2: x-1 = x+1
-            const int sd = (P.kind == PART_STRIPES) ? sx / W : (sy / W) * P.Dx + sx / W;
-            __syncwarp();
-            const int old_c = mine ? site_class(rows, sx, sy, L) : 0;
-            __syncwarp();
-            if (lane == 0) rows[2 * y + (x >> 6)] ^= 1ull << (x & 63);
-            __syncwarp();
-            if (mine) {
-                const int new_c = site_class(rows, sx, sy, L);
-                if (new_c != old_c) {
-                    atomicAdd(&dcount[sd * 10 + old_c], -1);
-                    atomicAdd(&dcount[sd * 10 + new_c], 1);
-                    atomicAdd(&dR[sd], (unsigned long long)(Atab[new_c] - Atab[old_c])); // mod 2^64
-                    if (use_rc) {
-                        const int syy = (P.kind == PART_STRIPES) ? sy : sy - (sd / P.Dx) * W;
-                        int sh0, sh1;
-                        unsigned *w0 = rc_word(sd, syy, old_c, sh0);
-                        unsigned *w1 = rc_word(sd, syy, new_c, sh1);
-                        atomicSub(w0, 1u << sh0); // the byte holds at least this site
-                        atomicAdd(w1, 1u << sh1);
-                    }
-                }
-            }
-            __syncwarp();
-            const uint64_t ev = (np << 32) | ((uint64_t)(jx - lo + jbase) << 16) | (uint64_t)(yy * W + (x - x0));
-            H = (H ^ ev) * HASH_PRIME;
-            ++flips;
-            pos = jx + 1;
-            // the classes are needed again only if a step of this visit remains
-            if (pos >= hi) break;
-            n_c = (lane < 10) ? (uint32_t)dcount[d * 10 + lane] : 0u;
-            Wc = (uint64_t)n_c * A;
-            Cinc = kmcdev::prefix16(Wc, lane);
-            R = dR[d];
-        }
-    };
-
-    // Step draw of lane `lane` for step j of domain d in phase np:
-    // target = floor(X M / 2^64) (tgt) and the clock variate (V).
-    auto draw = [&](uint32_t j, uint32_t d, uint64_t np, uint64_t &tgt, uint64_t &V) {
-        const uint4 w = kmcdev::philox4x32_10(make_uint4(j, d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu), key);
-        tgt = __umul64hi(((uint64_t)w.y << 32) | w.x, M);
-        V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
-    };
-    // Product of the variates of aligned groups of `span` lanes (a power of
-    // two; lanes without a step hold 1): lane 0 of each group receives it.
-    auto variate_product = [&](uint64_t V, int span, uint64_t &m, int &e) {
-        const int z = __clzll((long long)V);
-        m = V << z;
-        e = 10 - z;
-        for (int off = 1; off < span; off <<= 1) {
-            const uint64_t m2 = __shfl_xor_sync(FULL_WARP, m, off);
-            const int e2 = __shfl_xor_sync(FULL_WARP, e, off);
-            kmcdev::mant_mul32(m, e, m2, e2);
-        }
-    };
-
-    // One visit with its own draws, 32 steps at a time.
-    auto visit = [&](int d, uint64_t np) {
-        int x0, y0;
-        domain_origin(d, x0, y0);
-        const u128 DM = DM0 << x0;
-        for (int base = 0; base < k; base += 32) {
-            uint64_t tgt = ~0ull, V = 1ull << 53;
-            if (base + lane < k) draw((uint32_t)(base + lane), (uint32_t)d, np, tgt, V);
-            const int chunk_end = min(32, k - base);
-            if (EXPO) {
-                uint64_t m;
-                int e;
-                variate_product(V, 32, m, e);
-                kmcdev::mant_mul(clkM, clkE, __shfl_sync(FULL_WARP, m, 0), (int64_t)__shfl_sync(FULL_WARP, e, 0));
-            }
-            steps += chunk_end;
-            events(d, np, x0, y0, DM, tgt, 0, chunk_end, base);
-        }
-    };
 
     const bool perm = P.schedule == kmcdev::SCHED_RANDOM_PERM;
-    const int nph = perm ? P.ND : (P.schedule == kmcdev::SCHED_PALINDROME ? 2 * P.ncol : P.ncol);
-    const int dpp = (perm || P.ND == 1) ? 1 : P.ND / P.ncol; // visits per phase
-    const int Vs = nph * dpp;                                // visits per schedule
+    const int nph = perm ? ND : (P.schedule == kmcdev::SCHED_PALINDROME ? 2 * P.ncol : P.ncol);
+    const int dpp = (perm || ND == 1) ? 1 : ND / P.ncol; // visits per phase
+    const int Vs = nph * dpp;                             // visits per schedule
     const double N = (double)L * (double)L;
-    int64_t passes = 0;
+    uint8_t *phase_of = order + 128; // colour schedules: the phase of visit v (Vs <= 128)
+    if (!perm) {
+        // colour of phase p: 0 1 .. [.. 1 0]; the i-th domain of colour col in
+        // ascending order (blocks: by = col>>1 + 2 (i / (Dx/2)), bx = col&1 + 2 (i % (Dx/2)))
+        for (int v = lane; v < Vs; v += 32) {
+            const int p = v / dpp, i = v - p * dpp;
+            const int col = (p < P.ncol) ? p : (2 * P.ncol - 1 - p);
+            int d = 0;
+            if (ND > 1) {
+                const int half = P.Dx / 2;
+                d = stripes ? col + 2 * i : ((col >> 1) + 2 * (i / half)) * P.Dx + (col & 1) + 2 * (i % half);
+            }
+            order[v] = (uint8_t)d;
+            phase_of[v] = (uint8_t)p;
+        }
+    }
+    __syncwarp();
 
-    // colour of phase p: 0 1 .. [.. 1 0]; the i-th domain of colour col in
-    // ascending order (blocks: by = col>>1 + 2 (i / (Dx/2)), bx = col&1 + 2 (i % (Dx/2)))
-    auto phase_colour = [&](int p) { return (p < P.ncol) ? p : (2 * P.ncol - 1 - p); };
-    auto domain_of_colour = [&](int col, int i) {
-        if (P.ND == 1) return 0;
-        if (P.kind == PART_STRIPES) return col + 2 * i;
-        const int half = P.Dx / 2;
-        return ((col >> 1) + 2 * (i / half)) * P.Dx + (col & 1) + 2 * (i % half);
+    // bond sum = 2 L^2 - 2 (unlike neighbour pairs), magnetisation = 2 (up spins) - L^2
+    const bool want = P.obs != nullptr && P.obs_every > 0;
+    int bonds = 0, mag = 0;
+    if (want) {
+        int unlike = 0, up = 0;
+        for (int y = lane; y < L; y += 32) {
+            const u128 c = row_ld(rows, y);
+            const u128 s = row_ld(rows, (y == L - 1) ? 0 : y + 1);
+            unlike += popc128((c ^ rot_e(c, L)) & Lm) + popc128(c ^ s);
+            up += popc128(c);
+        }
+        bonds = 2 * L * L - 2 * __reduce_add_sync(FULL_WARP, unlike);
+        mag = 2 * __reduce_add_sync(FULL_WARP, up) - L * L;
+    }
+    auto write_record = [&](int64_t rec, int b, int mg, uint64_t cm, int64_t ce, int64_t st) {
+        const double e = __ddiv_rn(__dsub_rn(__dmul_rn(-P.J, (double)b), __dmul_rn(hr, (double)mg)), N);
+        const double m = __ddiv_rn((double)mg, N);
+        double4_32a v;
+        v.x = e;
+        v.y = m;
+        v.z = __dmul_rn(e, m);
+        v.w = kmcdev::domain_time(EXPO, cm, ce, st, __dmul_rn(N, P.nu));
+        reinterpret_cast<double4_32a *>(P.obs)[(size_t)rec * P.n_traj + tr] = v;
     };
-    // the paper's random order of all domains of schedule n (Fisher-Yates over Philox)
-    auto shuffle = [&](uint8_t *ord, uint64_t n) {
-        for (int i = 0; i < P.ND; ++i) ord[i] = (uint8_t)i;
-        for (int i = P.ND - 1; i >= 1; --i) {
+
+    // The paper's random order of all domains of a schedule (Fisher-Yates over
+    // Philox), one schedule per lane, into a ring of n_ord schedules.
+    int n_ord = 64;
+    while (n_ord * ND > PART_ORDER_BYTES) n_ord >>= 1; // a power of two, >= 16
+    int64_t ord_end = 0; // schedules shuffled so far
+    auto shuffle = [&](int64_t nl) {
+        uint8_t *ord = order + (int)(nl & (n_ord - 1)) * ND;
+        const uint64_t n = (uint64_t)(P.sched_begin + nl);
+        for (int i = 0; i < ND; ++i) ord[i] = (uint8_t)i;
+        for (int i = ND - 1; i >= 1; --i) {
             const uint4 w = kmcdev::philox4x32_10(
                 make_uint4((uint32_t)i, 0u, (uint32_t)n, ((uint32_t)(n >> 32) & 0xFFFFFFu) | (PART_TAG_PERM << 24)),
                 key);
@@ -421,99 +314,237 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             ord[jx] = tmp;
         }
     };
-    auto pass_done = [&]() {
-        ++passes;
-        if (P.obs != nullptr && P.obs_every > 0 && passes % P.obs_every == 0) {
-            // bonds = 2 L^2 - 2 (unlike neighbour pairs), mag = 2 (up spins) - L^2
-            int unlike = 0, up = 0;
-            for (int y = lane; y < L; y += 32) {
-                const u128 c = row_ld(rows, y);
-                const u128 s = row_ld(rows, (y == L - 1) ? 0 : y + 1);
-                unlike += popc128((c ^ rot_e(c, L)) & Lm) + popc128(c ^ s);
-                up += popc128(c);
-            }
-            unlike = __reduce_add_sync(FULL_WARP, unlike);
-            up = __reduce_add_sync(FULL_WARP, up);
-            if (lane == 0) {
-                const int64_t bonds = 2ll * L * L - 2ll * unlike;
-                const int64_t mag = 2ll * up - (int64_t)L * L;
-                const double e = __ddiv_rn(__dsub_rn(__dmul_rn(-P.J, (double)bonds), __dmul_rn(hr, (double)mag)), N);
-                const double m = __ddiv_rn((double)mag, N);
-                double4_32a v;
-                v.x = e;
-                v.y = m;
-                v.z = __dmul_rn(e, m);
-                v.w = kmcdev::domain_time(EXPO, clkM, clkE, steps, __dmul_rn(N, P.nu));
-                const int64_t rec = passes / P.obs_every - 1;
-                reinterpret_cast<double4_32a *>(P.obs)[(size_t)rec * P.n_traj + tr] = v;
-            }
-        }
-    };
 
-    // Short visits: the steps of the visits of Sw consecutive schedules are
-    // drawn together, lane i holding step i % kp of visit i / kp (kp = k
-    // rounded up to a power of two), when Sw Vs kp <= 32; the schedules'
-    // domain orders are shuffled one per lane first.
-    int kp = 1;
-    while (kp < k) kp <<= 1;
-    const int Sw = (k >= 1 && kp * Vs <= 32) ? 32 / (kp * Vs) : 0;
-    if (Sw > 0) {
-        for (int64_t nl = 0; nl < P.n_sched; nl += Sw) {
-            const int sw = (int)((P.n_sched - nl < Sw) ? (P.n_sched - nl) : Sw);
-            const uint64_t n0 = (uint64_t)(P.sched_begin + nl);
-            if (perm) {
+    const int64_t total = P.n_sched * (int64_t)Vs * k;
+    // this lane's step: schedule nl (of this launch), visit v, step j of it;
+    // 32 steps on are 32 / k visits and 32 % k steps on
+    int64_t nl = 0;
+    int v = 0, j = 0;
+    if (k > 0) {
+        const int q = lane / k;
+        j = lane - q * k;
+        nl = q / Vs;
+        v = q - (int)nl * Vs;
+    }
+    const int jump_j = k > 0 ? 32 % k : 0, jump_v = k > 0 ? (32 / k) % Vs : 0, jump_n = k > 0 ? (32 / k) / Vs : 0;
+    for (int64_t s0 = 0; s0 < total; s0 += 32) {
+        const bool act = s0 + lane < total;
+        if (perm) {
+            // a window spans at most n_ord / 2 schedules, so the half of the
+            // ring that is filled here holds none of its orders
+            const int64_t last = __shfl_sync(FULL_WARP, (long long)nl, 31);
+            while (ord_end <= last && ord_end < P.n_sched) {
                 __syncwarp();
-                if (lane < sw) shuffle(order + lane * P.ND, n0 + lane);
+                if (lane < n_ord / 2 && ord_end + lane < P.n_sched) shuffle(ord_end + lane);
+                ord_end += n_ord / 2;
                 __syncwarp();
             }
-            uint64_t tgt = ~0ull, V = 1ull << 53;
+        }
+        int d = 0, p = 0;
+        uint64_t tgt = ~0ull, ebase = 0, pm = 1ull << 63;
+        int pe = 0;
+        if (act) {
+            d = perm ? order[(int)(nl & (n_ord - 1)) * ND + v] : order[v];
+            p = perm ? v : phase_of[v];
+            const uint64_t np = (uint64_t)(P.sched_begin + nl) * PART_PHASE_SLOTS + (uint64_t)p;
+            ebase = (np << 32) | ((uint64_t)j << 16);
+            // target = floor(X M / 2^64), clock variate V 2^-53 as a
+            // normalised mantissa pm / 2^63 times 2^pe
+            const uint4 w = kmcdev::philox4x32_10(
+                make_uint4((uint32_t)j, (uint32_t)d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu), key);
+            tgt = __umul64hi(((uint64_t)w.y << 32) | w.x, M);
+            const uint64_t V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
+            const int z = __clzll((long long)V);
+            pm = V << z;
+            pe = 10 - z;
+        }
+        if (EXPO) {
+            // inclusive products over the lanes
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint64_t m2 = __shfl_up_sync(FULL_WARP, pm, off);
+                const int e2 = __shfl_up_sync(FULL_WARP, pe, off);
+                if (lane >= off) kmcdev::mant_mul32(pm, pe, m2, e2);
+            }
+        }
+        // the real events of the window, in step order
+        int pos = 0;
+        while (true) {
+            // the cumulative class rates of this lane's domain
+            uint64_t C[10];
             {
-                const int t = lane / kp, j = lane % kp;
-                if (t < sw * Vs && j < k) {
-                    const int sv = t / Vs, r = t % Vs;
-                    const int p = perm ? r : r / dpp;
-                    const int d = perm ? order[sv * P.ND + r] : domain_of_colour(phase_colour(p), r % dpp);
-                    draw((uint32_t)j, (uint32_t)d, (n0 + sv) * PART_PHASE_SLOTS + (uint64_t)p, tgt, V);
+                const uint4 n0 = *reinterpret_cast<const uint4 *>(dcount + d * 12);
+                const uint4 n1 = *reinterpret_cast<const uint4 *>(dcount + d * 12 + 4);
+                const uint2 n2 = *reinterpret_cast<const uint2 *>(dcount + d * 12 + 8);
+                const uint32_t n[10] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w, n2.x, n2.y};
+                uint64_t acc = 0;
+#pragma unroll
+                for (int c = 0; c < 10; ++c) {
+                    acc += (uint64_t)n[c] * A[c];
+                    C[c] = acc;
                 }
             }
-            uint64_t pm = 0;
-            int pe = 0;
-            if (EXPO) variate_product(V, kp, pm, pe);
+            const unsigned real = __ballot_sync(FULL_WARP, lane >= pos && tgt < C[9]);
+            if (!real) break;
+            const int jx = __ffs(real) - 1;
+            // each lane's class (the first c with target < C_c) and member index
+            // jj = floor((target - C_{c-1}) / A_c) < n_c: the high word of
+            // (target - C_{c-1}) floor((2^64 - 1) / A_c) is jj or jj - 1
+            int c = 0;
+            uint64_t Cprev = 0;
+#pragma unroll
+            for (int cc = 0; cc < 9; ++cc) {
+                const bool past = tgt >= C[cc];
+                c += past ? 1 : 0;
+                Cprev = past ? C[cc] : Cprev;
+            }
+            const ulonglong2 am = atab[c];
+            const uint64_t xq = tgt - Cprev;
+            uint32_t jj = (uint32_t)__umul64hi(xq, am.y);
+            jj = (xq - (uint64_t)jj * am.x >= am.x) ? jj + 1u : jj;
+            const uint32_t pick = __shfl_sync(FULL_WARP, (uint32_t)c | ((uint32_t)d << 4) | (jj << 10), jx);
+            const uint64_t ev = __shfl_sync(FULL_WARP, ebase, jx);
+            const int ec = (int)(pick & 15u), ed = (int)((pick >> 4) & 63u);
+            const uint32_t ejj = pick >> 10;
+            const int by = stripes ? 0 : ed / P.Dx;
+            const int x0 = (ed - by * nbx) * W, y0 = by * Hd;
+            // the row of the jj-th member of class c in row-major order
+            uint32_t rw = 0, cl = 0; // counts of this lane's rows, a byte each; their sum
+            u128 DM = 0;
+            if (use_rc) {
+                const uint8_t *rp = rc + (ed * 10 + ec) * Hp + lane * RPL;
+                if (lane * RPL < Hd)
+                    rw = RPL == 1 ? *rp
+                                  : RPL == 2 ? *reinterpret_cast<const uint16_t *>(rp)
+                                             : *reinterpret_cast<const uint32_t *>(rp);
+            } else {
+                DM = DM0 << x0;
+                for (int t = 0; t < RPL; ++t) {
+                    const int yy = lane * RPL + t;
+                    if (yy < Hd)
+                        rw |= (uint32_t)popc128(class_mask(row_planes(rows, y0 + yy, L, Lm, DM), ec)) << (8 * t);
+                }
+            }
+            cl = __dp4a(rw, 0x01010101u, 0u);
+            uint32_t incl = cl;
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                const uint32_t u = __shfl_up_sync(FULL_WARP, incl, off);
+                if (lane >= off) incl += u;
+            }
+            uint32_t rr = ejj - (incl - cl);
+            const unsigned win = __ballot_sync(FULL_WARP, ejj < incl && rr < cl);
+            if (!win) {
+                if (lane == 0) atomicOr(P.err, 2);
+                pos = jx + 1;
+                continue;
+            }
             int t = 0;
-            for (int sv = 0; sv < sw; ++sv) {
-                for (int p = 0; p < nph; ++p) {
-                    const uint64_t np = (n0 + sv) * PART_PHASE_SLOTS + (uint64_t)p;
-                    for (int i = 0; i < dpp; ++i, ++t) {
-                        const int d = perm ? order[sv * P.ND + p] : domain_of_colour(phase_colour(p), i);
-                        int x0, y0;
-                        domain_origin(d, x0, y0);
-                        if (EXPO)
-                            kmcdev::mant_mul(clkM, clkE, __shfl_sync(FULL_WARP, pm, t * kp),
-                                             (int64_t)__shfl_sync(FULL_WARP, pe, t * kp));
-                        steps += k;
-                        events(d, np, x0, y0, DM0 << x0, tgt, t * kp, t * kp + k, 0);
-                    }
-                    pass_done();
+            {
+                const uint32_t b0 = rw & 255u, b1 = b0 + ((rw >> 8) & 255u), b2 = b1 + ((rw >> 16) & 255u);
+                uint32_t before = 0;
+                if (rr >= b0) { t = 1; before = b0; }
+                if (rr >= b1) { t = 2; before = b1; }
+                if (rr >= b2) { t = 3; before = b2; }
+                rr -= before;
+            }
+            const uint32_t yr = __shfl_sync(FULL_WARP, (uint32_t)(lane * RPL + t) | (rr << 8), __ffs(win) - 1);
+            const int yy = (int)(yr & 255u), y = y0 + yy;
+            rr = yr >> 8;
+            // its column: one lane per column, 32 at a time
+            int x = x0;
+            for (int t0 = 0; t0 < W; t0 += 32) {
+                const int xx = x0 + t0 + lane;
+                const bool member = t0 + lane < W && site_class(row32, xx, y, L) == ec;
+                const unsigned mk = __ballot_sync(FULL_WARP, member);
+                const uint32_t pc = (uint32_t)__popc(mk);
+                if (rr < pc) {
+                    const unsigned it = __ballot_sync(FULL_WARP, member && (uint32_t)__popc(mk & ((1u << lane) - 1u)) == rr);
+                    x = x0 + t0 + __ffs(it) - 1;
+                    break;
+                }
+                rr -= pc;
+            }
+            // the flip changes the classes of the site and its four
+            // neighbours (lanes 0..4: site, W, E, N, S): the site's spin, and
+            // every neighbour's count by one (by two on a 2 x 2 lattice, whose
+            // opposite neighbours are the same site)
+            int sx = x, sy = y, sd = ed;
+            if (lane == 1) {
+                sx = (x == 0) ? L - 1 : x - 1;
+                if (x == x0) sd = nbd[4 * ed];
+            } else if (lane == 2) {
+                sx = (x == L - 1) ? 0 : x + 1;
+                if (x == x0 + W - 1) sd = nbd[4 * ed + 1];
+            } else if (lane == 3) {
+                sy = (y == 0) ? L - 1 : y - 1;
+                if (yy == 0) sd = nbd[4 * ed + 2];
+            } else if (lane == 4) {
+                sy = (y == L - 1) ? 0 : y + 1;
+                if (yy == Hd - 1) sd = nbd[4 * ed + 3];
+            }
+            const bool mine = lane < 5 && !(L == 2 && (lane == 2 || lane == 4));
+            const int gain = (ec < 5) ? 1 : -1;
+            const int old_c = mine ? site_class(row32, sx, sy, L) : 0;
+            const int new_c = (lane == 0) ? old_c + 5 * gain : old_c + (L == 2 ? 2 : 1) * gain;
+            __syncwarp();
+            if (lane == 0) row32[4 * y + (x >> 5)] ^= 1u << (x & 31);
+            if (mine) {
+                atomicSub(&dcount[sd * 12 + old_c], 1u);
+                atomicAdd(&dcount[sd * 12 + new_c], 1u);
+                if (use_rc) {
+                    const int syy = stripes ? sy : sy - (sd / P.Dx) * Hd;
+                    const int i0 = (sd * 10 + old_c) * Hp + syy, i1 = (sd * 10 + new_c) * Hp + syy;
+                    atomicSub(reinterpret_cast<unsigned *>(rc) + (i0 >> 2), 1u << (8 * (i0 & 3))); // the byte holds this site
+                    atomicAdd(reinterpret_cast<unsigned *>(rc) + (i1 >> 2), 1u << (8 * (i1 & 3)));
                 }
             }
-        }
-    } else {
-        for (int64_t nl = 0; nl < P.n_sched; ++nl) {
-            const uint64_t n = (uint64_t)(P.sched_begin + nl);
-            if (perm) {
-                __syncwarp();
-                if (lane == 0) shuffle(order, n);
-                __syncwarp();
+            __syncwarp();
+            H = (H ^ (ev | (uint64_t)(yy * W + (x - x0)))) * HASH_PRIME;
+            ++flips;
+            // flipping spin s with neighbour sum 2 q - 4 changes the bond sum by
+            // -2 s (2 q - 4) and the magnetisation by -2 s, for every record from
+            // this step on
+            if (lane >= jx) {
+                bonds += 2 * gain * (2 * (ec < 5 ? ec : ec - 5) - 4);
+                mag += 2 * gain;
             }
-            for (int p = 0; p < nph; ++p) {
-                const uint64_t np = n * PART_PHASE_SLOTS + (uint64_t)p;
-                for (int i = 0; i < dpp; ++i) visit(perm ? order[p] : domain_of_colour(phase_colour(p), i), np);
-                pass_done();
+            pos = jx + 1;
+        }
+        if (want && act && j == k - 1) {
+            // the last step of a visit; a pass ends with its last visit
+            const int64_t pass = nl * nph + p + 1;
+            if (v - p * dpp == dpp - 1 && pass % P.obs_every == 0) {
+                uint64_t cm = clkM;
+                int64_t ce = clkE;
+                if (EXPO) kmcdev::mant_mul(cm, ce, pm, (int64_t)pe);
+                write_record(pass / P.obs_every - 1, bonds, mag, cm, ce, steps0 + s0 + lane + 1);
             }
         }
+        if (want) {
+            bonds = __shfl_sync(FULL_WARP, bonds, 31);
+            mag = __shfl_sync(FULL_WARP, mag, 31);
+        }
+        if (EXPO)
+            kmcdev::mant_mul(clkM, clkE, __shfl_sync(FULL_WARP, pm, 31), (int64_t)__shfl_sync(FULL_WARP, pe, 31));
+        j += jump_j;
+        const int carry = (j >= k) ? 1 : 0;
+        j -= carry ? k : 0;
+        v += jump_v + carry;
+        nl += jump_n;
+        if (v >= Vs) {
+            v -= Vs;
+            ++nl;
+        }
+    }
+    if (k == 0 && want) {
+        // visits without steps: every record holds the state as it is
+        for (int64_t rec = lane; rec < P.n_sched * nph / P.obs_every; rec += 32)
+            write_record(rec, bonds, mag, clkM, clkE, steps0);
     }
 
     // write the lattice back
+    __syncwarp();
     int8_t *out = P.spins + (size_t)tr * L * L;
     for (int y = 0; y < L; ++y) {
         const u128 c = row_ld(rows, y);
@@ -524,8 +555,8 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
         P.clkM[tr] = clkM;
         P.clkE[tr] = clkE;
         P.flips[tr] = flips;
-        P.steps[tr] = steps;
-        P.t[tr] = kmcdev::domain_time(EXPO, clkM, clkE, steps, __dmul_rn(N, P.nu));
+        P.steps[tr] = steps0 + total;
+        P.t[tr] = kmcdev::domain_time(EXPO, clkM, clkE, steps0 + total, __dmul_rn(N, P.nu));
     }
 }
 
