@@ -31,19 +31,36 @@ constexpr int PART_MAX_L = 128;
 constexpr int PART_PHASE_SLOTS = 64; // Philox phase index np = n*64 + p
 constexpr int PART_BLOCKS = 0, PART_STRIPES = 1;
 constexpr uint32_t PART_TAG_PERM = 2u;
-// shared memory per warp (64-bit words): bit rows, the domains of the visits
-// (u8: the random orders of the schedules in use, or one colour schedule's
-// visits and after them their phases), each domain's neighbours (u8 [64][4]),
-// the class counts of every domain (u32 [64][12], ten used), the fixed-point
-// rates and their reciprocals (u64 [10][2]) and, when the lattice has at most
-// PART_RC_ROWS domain rows (N_D x domain height, padded to a multiple of 4),
-// the class counts of every domain row (u8 [N_D][10][rows])
-constexpr int PART_RC_ROWS = 768;
+// Bit rows in shared memory: PART_ROW32 32-bit words per row, bit x + 1 =
+// column x (1 = up), bit 0 a copy of column L - 1 and bit L + 1 one of column
+// 0, so that a window of columns and their W and E neighbours is a shift.
+constexpr int PART_ROW32 = 6;
+// The class counts of domain rows are kept (u8 [N_D][10][rows], the rows
+// padded to a multiple of 16: one 128-bit load each 16 rows) when the
+// lattice has at most PART_RC_ROWS padded domain rows.
+constexpr int PART_RC_ROWS = 1024;
 constexpr int PART_ORDER_BYTES = 1024;
-constexpr int PART_OFF_ORDER = 2 * PART_MAX_L, PART_OFF_NBD = PART_OFF_ORDER + PART_ORDER_BYTES / 8,
-              PART_OFF_DCOUNT = PART_OFF_NBD + 64 * 4 / 8, PART_OFF_ATAB = PART_OFF_DCOUNT + 64 * 12 / 2,
-              PART_OFF_RC = PART_OFF_ATAB + 20;
-constexpr int PART_WARP_WORDS = PART_OFF_RC + PART_RC_ROWS * 10 / 8;
+// shared memory of a trajectory in bytes: the class counts of the domain
+// rows, the fixed-point rates and their reciprocals (u64 [10][2]), the class
+// counts of every domain (u32 [N_D][12], ten used), the bit rows, the domains
+// of the visits (u8: the random orders of the schedules in use, or one colour
+// schedule's visits and after them their phases), each domain's neighbours
+// (u8 [N_D][4]) and its first column and row (u8 [N_D][2])
+struct PartLayout {
+    int rc, atab, dcount, rows, order, nbd, org, bytes;
+    __host__ __device__ PartLayout(int L, int ND, int Hd)
+    {
+        const int Hp = (Hd + 15) & ~15;
+        rc = 0;
+        atab = (ND * Hp <= PART_RC_ROWS) ? ND * Hp * 10 : 0;
+        dcount = atab + 160;
+        rows = dcount + ND * 48;
+        order = rows + L * PART_ROW32 * 4;
+        nbd = order + PART_ORDER_BYTES;
+        org = nbd + ND * 4;
+        bytes = (org + ND * 2 + 15) & ~15;
+    }
+};
 
 struct PartParams {
     int n_traj, L, kind, ND, k;
@@ -65,9 +82,12 @@ struct PartParams {
     int *err;
 };
 
-__device__ __forceinline__ u128 row_ld(const uint64_t *rows, int y)
+// Row y, bit x = column x.
+__device__ __forceinline__ u128 row_ld(const uint32_t *rows, int y, u128 Lm)
 {
-    return ((u128)rows[2 * y + 1] << 64) | rows[2 * y];
+    const uint32_t *w = rows + PART_ROW32 * y;
+    const uint64_t lo = ((uint64_t)w[1] << 32) | w[0], hi = ((uint64_t)w[3] << 32) | w[2];
+    return ((((u128)hi << 64 | lo) >> 1) | ((u128)w[4] << 127)) & Lm;
 }
 
 // bit x <- bit x-1 (mod L) / bit x <- bit x+1 (mod L) of an L-bit row
@@ -82,11 +102,11 @@ struct RowPlanes {
     u128 up, dn, b0, b1, b2;
 };
 
-__device__ __forceinline__ RowPlanes row_planes(const uint64_t *rows, int y, int L, u128 Lm, u128 DM)
+__device__ __forceinline__ RowPlanes row_planes(const uint32_t *rows, int y, int L, u128 Lm, u128 DM)
 {
-    const u128 c = row_ld(rows, y);
-    const u128 n = row_ld(rows, (y == 0) ? L - 1 : y - 1);
-    const u128 s = row_ld(rows, (y == L - 1) ? 0 : y + 1);
+    const u128 c = row_ld(rows, y, Lm);
+    const u128 n = row_ld(rows, (y == 0) ? L - 1 : y - 1, Lm);
+    const u128 s = row_ld(rows, (y == L - 1) ? 0 : y + 1, Lm);
     const u128 w = rot_w(c, L, Lm), e = rot_e(c, L);
     const u128 s1 = n ^ s, c1 = n & s, s2 = w ^ e, c2 = w & e, t0 = s1 & s2;
     RowPlanes p;
@@ -108,7 +128,7 @@ __device__ __forceinline__ u128 class_mask(const RowPlanes &p, int c)
 }
 
 // Lane c (< 10) receives n_c of the domain (rows y0 .. y0+H-1).
-__device__ __forceinline__ uint32_t part_counts(const uint64_t *rows, int lane, int y0, int H, int RPL, int L,
+__device__ __forceinline__ uint32_t part_counts(const uint32_t *rows, int lane, int y0, int H, int RPL, int L,
                                                 u128 Lm, u128 DM)
 {
     uint32_t w[5] = {0, 0, 0, 0, 0};
@@ -133,23 +153,11 @@ __device__ __forceinline__ uint32_t part_counts(const uint64_t *rows, int lane, 
     return (lane < 10) ? n : 0u;
 }
 
-// The rr-th (0-based) set bit of a 128-bit mask; rr < popc(m).
-__device__ __forceinline__ int select128(u128 m, uint32_t rr)
+// Class 5 up + (number of up neighbours) of site (x, y), from the live rows.
+__device__ __forceinline__ int site_class(const uint32_t *rows, int x, int y, int ym, int yp)
 {
-    const uint64_t lo = (uint64_t)m;
-    const uint32_t pl = (uint32_t)__popcll(lo);
-    if (rr < pl) return kmcdev::select_bit(lo, rr);
-    return 64 + kmcdev::select_bit((uint64_t)(m >> 64), rr - pl);
-}
-
-// Class 5 up + (number of up neighbours) of site (x, y), from the live rows
-// (32-bit words, four per row).
-__device__ __forceinline__ int site_class(const uint32_t *row32, int x, int y, int L)
-{
-    const int xm = (x == 0) ? L - 1 : x - 1, xp = (x == L - 1) ? 0 : x + 1;
-    const int ym = (y == 0) ? L - 1 : y - 1, yp = (y == L - 1) ? 0 : y + 1;
-    auto bit = [&](int xx, int yy) { return (int)((row32[4 * yy + (xx >> 5)] >> (xx & 31)) & 1u); };
-    return 5 * bit(x, y) + bit(xm, y) + bit(xp, y) + bit(x, ym) + bit(x, yp);
+    auto bit = [&](int b, int yy) { return (int)((rows[PART_ROW32 * yy + (b >> 5)] >> (b & 31)) & 1u); };
+    return 5 * bit(x + 1, y) + bit(x, y) + bit(x + 2, y) + bit(x + 1, ym) + bit(x + 1, yp);
 }
 
 // One warp runs one trajectory's steps in windows of 32 consecutive steps of
@@ -169,35 +177,34 @@ __device__ __forceinline__ int site_class(const uint32_t *row32, int x, int y, i
 template <bool EXPO>
 __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams P)
 {
-    extern __shared__ __align__(16) uint64_t part_smem[];
+    extern __shared__ __align__(16) uint8_t part_smem[];
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int tr = blockIdx.x * PART_WARPS + warp;
     if (tr >= P.n_traj) return; // whole warps only; no CTA-wide barrier below
     const int L = P.L, ND = P.ND;
-    uint64_t *rows = part_smem + (size_t)warp * PART_WARP_WORDS;
-    uint32_t *row32 = reinterpret_cast<uint32_t *>(rows);
-    uint8_t *order = reinterpret_cast<uint8_t *>(rows + PART_OFF_ORDER);
-    uint8_t *nbd = reinterpret_cast<uint8_t *>(rows + PART_OFF_NBD);          // [N_D][4] W, E, N, S domains
-    uint32_t *dcount = reinterpret_cast<uint32_t *>(rows + PART_OFF_DCOUNT);  // [N_D][12] class counts
-    ulonglong2 *atab = reinterpret_cast<ulonglong2 *>(rows + PART_OFF_ATAB);  // [10] A_c, floor((2^64 - 1) / A_c)
-    uint8_t *rc = reinterpret_cast<uint8_t *>(rows + PART_OFF_RC);            // [N_D][10][Hp]
+    const PartLayout lay(L, ND, P.H);
+    uint8_t *base8 = part_smem + (size_t)warp * lay.bytes;
+    uint32_t *rows = reinterpret_cast<uint32_t *>(base8 + lay.rows);
+    uint8_t *order = base8 + lay.order;
+    uint8_t *nbd = base8 + lay.nbd;                                     // [N_D][4] W, E, N, S domains
+    uint8_t *org = base8 + lay.org;                                     // [N_D][2] first column and row
+    uint32_t *dcount = reinterpret_cast<uint32_t *>(base8 + lay.dcount); // [N_D][12] class counts
+    ulonglong2 *atab = reinterpret_cast<ulonglong2 *>(base8 + lay.atab); // [10] A_c, floor((2^64 - 1) / A_c)
+    uint8_t *rc = base8 + lay.rc;                                       // [N_D][10][Hp]
     const u128 Lm = (L == 128) ? ~(u128)0 : (((u128)1 << L) - 1);
     const int8_t *sp = P.spins + (size_t)tr * L * L;
 
     // load the lattice into bit rows (ballots over 32-column chunks)
     int bad = 0;
     for (int y = 0; y < L; ++y) {
-        uint64_t wd[2] = {0, 0};
-        for (int x0 = 0; x0 < L; x0 += 32) {
-            const int x = x0 + lane;
-            const int8_t v = (x < L) ? sp[(size_t)y * L + x] : (int8_t)-1;
+        // bit b: column b - 1, with wrap
+        for (int b0 = 0; b0 < 32 * PART_ROW32; b0 += 32) {
+            const int b = b0 + lane;
+            const int x = (b == 0) ? L - 1 : (b == L + 1) ? 0 : b - 1;
+            const int8_t v = (b < L + 2) ? sp[(size_t)y * L + x] : (int8_t)-1;
             bad |= (v != 1 && v != -1);
-            const uint32_t b = __ballot_sync(FULL_WARP, v == 1);
-            wd[x0 >> 6] |= (uint64_t)b << (x0 & 63);
-        }
-        if (lane == 0) {
-            rows[2 * y] = wd[0];
-            rows[2 * y + 1] = wd[1];
+            const uint32_t w = __ballot_sync(FULL_WARP, v == 1);
+            if (lane == 0) rows[PART_ROW32 * y + (b0 >> 5)] = w;
         }
     }
     if (__any_sync(FULL_WARP, bad) && lane == 0) atomicOr(P.err, 1);
@@ -212,9 +219,8 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
     uint64_t H = P.hash[tr], clkM = P.clkM[tr];
     int64_t clkE = P.clkE[tr], flips = P.flips[tr];
     const int64_t steps0 = P.steps[tr];
-    // lane l holds domain rows l*RPL .. l*RPL+RPL-1, RPL a power of two
-    const int W = P.W, Hd = P.H, RPL = Hd <= 32 ? 1 : Hd <= 64 ? 2 : 4, k = P.k;
-    const int Hp = (Hd + 3) & ~3;
+    const int W = P.W, Hd = P.H, k = P.k;
+    const int Hp = (Hd + 15) & ~15;
     const u128 DM0 = (W == 128) ? ~(u128)0 : (((u128)1 << W) - 1);
     const uint64_t M = P.M;
     const bool stripes = P.kind == PART_STRIPES;
@@ -227,6 +233,8 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
     }
     for (int d = lane; d < ND; d += 32) {
         const int bx = d % nbx, by = d / nbx;
+        org[2 * d] = (uint8_t)(bx * W);
+        org[2 * d + 1] = (uint8_t)(by * Hd);
         nbd[4 * d + 0] = (uint8_t)(by * nbx + (bx == 0 ? nbx - 1 : bx - 1));
         nbd[4 * d + 1] = (uint8_t)(by * nbx + (bx == nbx - 1 ? 0 : bx + 1));
         nbd[4 * d + 2] = (uint8_t)((by == 0 ? nby - 1 : by - 1) * nbx + bx);
@@ -276,8 +284,8 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
     if (want) {
         int unlike = 0, up = 0;
         for (int y = lane; y < L; y += 32) {
-            const u128 c = row_ld(rows, y);
-            const u128 s = row_ld(rows, (y == L - 1) ? 0 : y + 1);
+            const u128 c = row_ld(rows, y, Lm);
+            const u128 s = row_ld(rows, (y == L - 1) ? 0 : y + 1, Lm);
             unlike += popc128((c ^ rot_e(c, L)) & Lm) + popc128(c ^ s);
             up += popc128(c);
         }
@@ -314,6 +322,25 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             ord[jx] = tmp;
         }
     };
+
+    // The clock: each lane multiplies the variates of its own steps, and the
+    // lanes' products are combined only where a record or the launch's end
+    // asks for them.
+    uint64_t lM = 1ull << 63;
+    int lE = 0;
+    auto join = [&]() {
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            const uint64_t m2 = __shfl_xor_sync(FULL_WARP, lM, off);
+            const int e2 = __shfl_xor_sync(FULL_WARP, lE, off);
+            kmcdev::mant_mul32(lM, lE, m2, e2);
+        }
+        kmcdev::mant_mul(clkM, clkE, __shfl_sync(FULL_WARP, lM, 0), (int64_t)__shfl_sync(FULL_WARP, lE, 0));
+        lM = 1ull << 63;
+        lE = 0;
+    };
+    // neighbour of this lane (lanes 1..4: W, E, N, S; lane 0: the site)
+    const int dxl = (lane == 1) ? -1 : (lane == 2) ? 1 : 0, dyl = (lane == 3) ? -1 : (lane == 4) ? 1 : 0;
 
     const int64_t total = P.n_sched * (int64_t)Vs * k;
     // this lane's step: schedule nl (of this launch), visit v, step j of it;
@@ -358,13 +385,28 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             pm = V << z;
             pe = 10 - z;
         }
+        // does a pass with a record end at this lane's step?  (a pass ends with
+        // the last step of its last visit)
+        int64_t rec = -1;
+        bool any_rec = false;
+        if (want) {
+            if (act && j == k - 1 && v - p * dpp == dpp - 1) {
+                const int64_t pass = nl * nph + p + 1;
+                if (pass % P.obs_every == 0) rec = pass / P.obs_every - 1;
+            }
+            any_rec = __any_sync(FULL_WARP, rec >= 0);
+        }
         if (EXPO) {
-            // inclusive products over the lanes
+            if (any_rec) {
+                join(); // everything before this window; then the inclusive products of its steps
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                const uint64_t m2 = __shfl_up_sync(FULL_WARP, pm, off);
-                const int e2 = __shfl_up_sync(FULL_WARP, pe, off);
-                if (lane >= off) kmcdev::mant_mul32(pm, pe, m2, e2);
+                for (int off = 1; off < 32; off <<= 1) {
+                    const uint64_t m2 = __shfl_up_sync(FULL_WARP, pm, off);
+                    const int e2 = __shfl_up_sync(FULL_WARP, pe, off);
+                    if (lane >= off) kmcdev::mant_mul32(pm, pe, m2, e2);
+                }
+            } else {
+                kmcdev::mant_mul32(lM, lE, pm, pe);
             }
         }
         // the real events of the window, in step order
@@ -377,12 +419,21 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
                 const uint4 n1 = *reinterpret_cast<const uint4 *>(dcount + d * 12 + 4);
                 const uint2 n2 = *reinterpret_cast<const uint2 *>(dcount + d * 12 + 8);
                 const uint32_t n[10] = {n0.x, n0.y, n0.z, n0.w, n1.x, n1.y, n1.z, n1.w, n2.x, n2.y};
-                uint64_t acc = 0;
+                uint64_t w[10];
 #pragma unroll
-                for (int c = 0; c < 10; ++c) {
-                    acc += (uint64_t)n[c] * A[c];
-                    C[c] = acc;
-                }
+                for (int c = 0; c < 10; ++c) w[c] = (uint64_t)n[c] * A[c];
+                // prefix sums in a shallow tree (pairs, then a chain over pairs)
+                const uint64_t s23 = w[2] + w[3], s45 = w[4] + w[5], s67 = w[6] + w[7], s89 = w[8] + w[9];
+                C[0] = w[0];
+                C[1] = w[0] + w[1];
+                C[2] = C[1] + w[2];
+                C[3] = C[1] + s23;
+                C[4] = C[3] + w[4];
+                C[5] = C[3] + s45;
+                C[6] = C[5] + w[6];
+                C[7] = C[5] + s67;
+                C[8] = C[7] + w[8];
+                C[9] = C[7] + s89;
             }
             const unsigned real = __ballot_sync(FULL_WARP, lane >= pos && tgt < C[9]);
             if (!real) break;
@@ -406,29 +457,27 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             const uint64_t ev = __shfl_sync(FULL_WARP, ebase, jx);
             const int ec = (int)(pick & 15u), ed = (int)((pick >> 4) & 63u);
             const uint32_t ejj = pick >> 10;
-            const int by = stripes ? 0 : ed / P.Dx;
-            const int x0 = (ed - by * nbx) * W, y0 = by * Hd;
-            // the row of the jj-th member of class c in row-major order
-            uint32_t rw = 0, cl = 0; // counts of this lane's rows, a byte each; their sum
-            u128 DM = 0;
+            const int x0 = org[2 * ed], y0 = org[2 * ed + 1];
+            // the row of the jj-th member of class c in row-major order: lane l
+            // holds the counts of domain rows 16 l .. 16 l + 15, a byte each
+            uint4 rw = make_uint4(0u, 0u, 0u, 0u);
             if (use_rc) {
-                const uint8_t *rp = rc + (ed * 10 + ec) * Hp + lane * RPL;
-                if (lane * RPL < Hd)
-                    rw = RPL == 1 ? *rp
-                                  : RPL == 2 ? *reinterpret_cast<const uint16_t *>(rp)
-                                             : *reinterpret_cast<const uint32_t *>(rp);
-            } else {
-                DM = DM0 << x0;
-                for (int t = 0; t < RPL; ++t) {
-                    const int yy = lane * RPL + t;
-                    if (yy < Hd)
-                        rw |= (uint32_t)popc128(class_mask(row_planes(rows, y0 + yy, L, Lm, DM), ec)) << (8 * t);
-                }
-            }
-            cl = __dp4a(rw, 0x01010101u, 0u);
-            uint32_t incl = cl;
+                if (16 * lane < Hd) rw = *reinterpret_cast<const uint4 *>(rc + (ed * 10 + ec) * Hp + 16 * lane);
+            } else if (16 * lane < Hd) {
+                const u128 DM = DM0 << x0;
+                uint32_t wq[4] = {0u, 0u, 0u, 0u};
 #pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
+                for (int t = 0; t < 16; ++t) {
+                    const int yy = 16 * lane + t;
+                    if (yy < Hd)
+                        wq[t >> 2] |= (uint32_t)popc128(class_mask(row_planes(rows, y0 + yy, L, Lm, DM), ec)) << (8 * (t & 3));
+                }
+                rw = make_uint4(wq[0], wq[1], wq[2], wq[3]);
+            }
+            const uint32_t q0 = __dp4a(rw.x, 0x01010101u, 0u), q1 = __dp4a(rw.y, 0x01010101u, q0),
+                           q2 = __dp4a(rw.z, 0x01010101u, q1), cl = __dp4a(rw.w, 0x01010101u, q2);
+            uint32_t incl = cl;
+            for (int off = 1; 16 * off < Hd; off <<= 1) {
                 const uint32_t u = __shfl_up_sync(FULL_WARP, incl, off);
                 if (lane >= off) incl += u;
             }
@@ -439,65 +488,80 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
                 pos = jx + 1;
                 continue;
             }
-            int t = 0;
+            uint32_t yr;
             {
-                const uint32_t b0 = rw & 255u, b1 = b0 + ((rw >> 8) & 255u), b2 = b1 + ((rw >> 16) & 255u);
-                uint32_t before = 0;
-                if (rr >= b0) { t = 1; before = b0; }
-                if (rr >= b1) { t = 2; before = b1; }
-                if (rr >= b2) { t = 3; before = b2; }
-                rr -= before;
+                const bool g0 = rr >= q0, g1 = rr >= q1, g2 = rr >= q2;
+                const uint32_t w = g2 ? rw.w : g1 ? rw.z : g0 ? rw.y : rw.x;
+                rr -= g2 ? q2 : g1 ? q1 : g0 ? q0 : 0u;
+                const uint32_t b0 = w & 255u, b1 = b0 + ((w >> 8) & 255u), b2 = b1 + ((w >> 16) & 255u);
+                const bool h0 = rr >= b0, h1 = rr >= b1, h2 = rr >= b2;
+                rr -= h2 ? b2 : h1 ? b1 : h0 ? b0 : 0u;
+                const int t = 4 * ((g0 ? 1 : 0) + (g1 ? 1 : 0) + (g2 ? 1 : 0)) + (h0 ? 1 : 0) + (h1 ? 1 : 0) + (h2 ? 1 : 0);
+                yr = __shfl_sync(FULL_WARP, (uint32_t)(16 * lane + t) | (rr << 8), __ffs(win) - 1);
             }
-            const uint32_t yr = __shfl_sync(FULL_WARP, (uint32_t)(lane * RPL + t) | (rr << 8), __ffs(win) - 1);
             const int yy = (int)(yr & 255u), y = y0 + yy;
             rr = yr >> 8;
-            // its column: one lane per column, 32 at a time
+            const int ym = (y == 0) ? L - 1 : y - 1, yp = (y == L - 1) ? 0 : y + 1;
+            // its column: the row's class mask, 32 columns at a time, the same in
+            // every lane; lane i tests whether its column is member rr
             int x = x0;
             for (int t0 = 0; t0 < W; t0 += 32) {
-                const int xx = x0 + t0 + lane;
-                const bool member = t0 + lane < W && site_class(row32, xx, y, L) == ec;
-                const unsigned mk = __ballot_sync(FULL_WARP, member);
+                const int X = x0 + t0, i = X >> 5, sft = X & 31; // bit X: column X - 1
+                auto window = [&](int yq, uint32_t &lo, uint32_t &hi) {
+                    const uint32_t *w = rows + PART_ROW32 * yq + i;
+                    const uint32_t a0 = w[0], a1 = w[1], a2 = w[2]; // i <= 3
+                    lo = __funnelshift_r(a0, a1, sft);
+                    hi = __funnelshift_r(a1, a2, sft);
+                };
+                uint32_t cl0, cl1, nl0, nl1, sl0, sl1;
+                window(y, cl0, cl1);
+                window(ym, nl0, nl1);
+                window(yp, sl0, sl1);
+                const uint32_t wn = cl0, cc = __funnelshift_r(cl0, cl1, 1), en = __funnelshift_r(cl0, cl1, 2);
+                const uint32_t nn = __funnelshift_r(nl0, nl1, 1), ss = __funnelshift_r(sl0, sl1, 1);
+                const uint32_t s1 = nn ^ ss, c1 = nn & ss, s2 = wn ^ en, c2 = wn & en, u0 = s1 & s2;
+                const uint32_t b0 = s1 ^ s2, b1 = c1 ^ c2 ^ u0, b2 = (c1 & c2) | (c1 & u0) | (c2 & u0);
+                const int q = (ec >= 5) ? ec - 5 : ec;
+                const uint32_t diff = (b2 ^ ((q & 4) ? ~0u : 0u)) | (b1 ^ ((q & 2) ? ~0u : 0u)) | (b0 ^ ((q & 1) ? ~0u : 0u));
+                const uint32_t cols = (W - t0 >= 32) ? ~0u : ((1u << (W - t0)) - 1u);
+                const uint32_t mk = (ec >= 5 ? cc : ~cc) & ~diff & cols;
                 const uint32_t pc = (uint32_t)__popc(mk);
-                if (rr < pc) {
-                    const unsigned it = __ballot_sync(FULL_WARP, member && (uint32_t)__popc(mk & ((1u << lane) - 1u)) == rr);
-                    x = x0 + t0 + __ffs(it) - 1;
-                    break;
-                }
+                const unsigned it = __ballot_sync(FULL_WARP, ((mk >> lane) & 1u) && (uint32_t)__popc(mk & ((1u << lane) - 1u)) == rr);
+                x = X + max(__ffs(it) - 1, 0);
+                if (rr < pc) break;
                 rr -= pc;
             }
             // the flip changes the classes of the site and its four
             // neighbours (lanes 0..4: site, W, E, N, S): the site's spin, and
             // every neighbour's count by one (by two on a 2 x 2 lattice, whose
             // opposite neighbours are the same site)
-            int sx = x, sy = y, sd = ed;
-            if (lane == 1) {
-                sx = (x == 0) ? L - 1 : x - 1;
-                if (x == x0) sd = nbd[4 * ed];
-            } else if (lane == 2) {
-                sx = (x == L - 1) ? 0 : x + 1;
-                if (x == x0 + W - 1) sd = nbd[4 * ed + 1];
-            } else if (lane == 3) {
-                sy = (y == 0) ? L - 1 : y - 1;
-                if (yy == 0) sd = nbd[4 * ed + 2];
-            } else if (lane == 4) {
-                sy = (y == L - 1) ? 0 : y + 1;
-                if (yy == Hd - 1) sd = nbd[4 * ed + 3];
-            }
+            int sx = x + dxl, sy = y + dyl, syy = yy + dyl;
+            const int bx = x - x0 + dxl;
+            const bool cross = bx < 0 || bx == W || syy < 0 || syy == Hd;
+            const int sd = cross ? nbd[4 * ed + ((lane + 3) & 3)] : ed;
+            sx = (sx < 0) ? L - 1 : (sx == L) ? 0 : sx;
+            sy = (sy < 0) ? L - 1 : (sy == L) ? 0 : sy;
+            syy = (syy < 0) ? Hd - 1 : (syy == Hd) ? 0 : syy;
             const bool mine = lane < 5 && !(L == 2 && (lane == 2 || lane == 4));
             const int gain = (ec < 5) ? 1 : -1;
-            const int old_c = mine ? site_class(row32, sx, sy, L) : 0;
+            const int old_c = site_class(rows, sx, sy, (sy == 0) ? L - 1 : sy - 1, (sy == L - 1) ? 0 : sy + 1);
             const int new_c = (lane == 0) ? old_c + 5 * gain : old_c + (L == 2 ? 2 : 1) * gain;
             __syncwarp();
-            if (lane == 0) row32[4 * y + (x >> 5)] ^= 1u << (x & 31);
             if (mine) {
                 atomicSub(&dcount[sd * 12 + old_c], 1u);
                 atomicAdd(&dcount[sd * 12 + new_c], 1u);
                 if (use_rc) {
-                    const int syy = stripes ? sy : sy - (sd / P.Dx) * Hd;
                     const int i0 = (sd * 10 + old_c) * Hp + syy, i1 = (sd * 10 + new_c) * Hp + syy;
                     atomicSub(reinterpret_cast<unsigned *>(rc) + (i0 >> 2), 1u << (8 * (i0 & 3))); // the byte holds this site
                     atomicAdd(reinterpret_cast<unsigned *>(rc) + (i1 >> 2), 1u << (8 * (i1 & 3)));
                 }
+            }
+            if (lane == 0) {
+                // the site's bit and its copy at the other end of the row
+                uint32_t *w = rows + PART_ROW32 * y;
+                w[(x + 1) >> 5] ^= 1u << ((x + 1) & 31);
+                if (x == 0) w[(L + 1) >> 5] ^= 1u << ((L + 1) & 31);
+                if (x == L - 1) w[0] ^= 1u;
             }
             __syncwarp();
             H = (H ^ (ev | (uint64_t)(yy * W + (x - x0)))) * HASH_PRIME;
@@ -511,22 +575,18 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             }
             pos = jx + 1;
         }
-        if (want && act && j == k - 1) {
-            // the last step of a visit; a pass ends with its last visit
-            const int64_t pass = nl * nph + p + 1;
-            if (v - p * dpp == dpp - 1 && pass % P.obs_every == 0) {
+        if (want) {
+            if (rec >= 0) {
                 uint64_t cm = clkM;
                 int64_t ce = clkE;
                 if (EXPO) kmcdev::mant_mul(cm, ce, pm, (int64_t)pe);
-                write_record(pass / P.obs_every - 1, bonds, mag, cm, ce, steps0 + s0 + lane + 1);
+                write_record(rec, bonds, mag, cm, ce, steps0 + s0 + lane + 1);
             }
-        }
-        if (want) {
             bonds = __shfl_sync(FULL_WARP, bonds, 31);
             mag = __shfl_sync(FULL_WARP, mag, 31);
+            if (EXPO && any_rec)
+                kmcdev::mant_mul(clkM, clkE, __shfl_sync(FULL_WARP, pm, 31), (int64_t)__shfl_sync(FULL_WARP, pe, 31));
         }
-        if (EXPO)
-            kmcdev::mant_mul(clkM, clkE, __shfl_sync(FULL_WARP, pm, 31), (int64_t)__shfl_sync(FULL_WARP, pe, 31));
         j += jump_j;
         const int carry = (j >= k) ? 1 : 0;
         j -= carry ? k : 0;
@@ -537,6 +597,7 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             ++nl;
         }
     }
+    if (EXPO) join();
     if (k == 0 && want) {
         // visits without steps: every record holds the state as it is
         for (int64_t rec = lane; rec < P.n_sched * nph / P.obs_every; rec += 32)
@@ -547,8 +608,8 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
     __syncwarp();
     int8_t *out = P.spins + (size_t)tr * L * L;
     for (int y = 0; y < L; ++y) {
-        const u128 c = row_ld(rows, y);
-        for (int x = lane; x < L; x += 32) out[(size_t)y * L + x] = ((c >> x) & 1) ? (int8_t)1 : (int8_t)-1;
+        for (int x = lane; x < L; x += 32)
+            out[(size_t)y * L + x] = ((rows[PART_ROW32 * y + ((x + 1) >> 5)] >> ((x + 1) & 31)) & 1u) ? (int8_t)1 : (int8_t)-1;
     }
     if (lane == 0) {
         P.hash[tr] = H;
