@@ -21,7 +21,7 @@ BUILD = os.path.join(HERE, "_build")
 LIB = os.path.join(BUILD, "libkmc_gb300.so")
 SOURCES = [os.path.join(CSRC, "kmc_api.cu")]
 DEPS = SOURCES + [os.path.join(CSRC, name) for name in ("kmc_kernels.cuh", "kmc_ring.cuh", "kmc_part.cuh",
-                                                          "kmc_tpd.cuh", "kmc_tpdr.cuh", "kmc_tpdr64.cuh")] + \
+                                                          "kmc_tpd.cuh", "kmc_tpdr.cuh", "kmc_tpdr64.cuh", "kmc_grp.cuh")] + \
     [os.path.join(ROOT, "include", "kmc.h")]
 
 

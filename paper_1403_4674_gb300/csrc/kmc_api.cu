@@ -12,6 +12,7 @@
 #include "kmc_tpd.cuh"
 #include "kmc_tpdr.cuh"
 #include "kmc_tpdr64.cuh"
+#include "kmc_grp.cuh"
 
 #include <cuda_runtime.h>
 #include <nvtx3/nvToolsExt.h>
@@ -37,8 +38,9 @@ struct Plan {
     int cluster = 0;  // CTAs per cluster (CLUSTER mode)
     int n_cta = 0;
     int wpb = 0;
-    int max_rt = 0;
+    int max_rt = 0;   // replica tables per CTA; sets per warp of a group plan
     int max_slots = 0;
+    int groups = 0;   // THREADS mode of L_d = 16, 32, 64: lanes per domain (grp_kernel), 0: one thread per domain
     size_t smem = 0;
     std::vector<uint32_t> cta_slot_off, cta_col_off, cta_rt_off, rt_rep, slot_g, slot_rt, slot_nb;
 };
@@ -570,9 +572,51 @@ TpdKernel tpd_kernel_for(int LD, bool expo, bool grad)
                     : (expo ? tpdr_kernel<32, true, false> : tpdr_kernel<32, false, false>);
     return expo ? tpd_kernel<true> : tpd_kernel<false>;
 }
+// the lane-group kernel of a domain side and G lanes per domain
+TpdKernel grp_kernel_for(int LD, int G, bool expo)
+{
+#define KMC_GRP(LDV, GV) \
+    if (LD == LDV && G == GV) return expo ? grp_kernel<LDV, GV, true> : grp_kernel<LDV, GV, false>;
+    KMC_GRP(16, 8) KMC_GRP(16, 16)
+    KMC_GRP(32, 8) KMC_GRP(32, 16) KMC_GRP(32, 32)
+    KMC_GRP(64, 16) KMC_GRP(64, 32)
+#undef KMC_GRP
+    return nullptr;
+}
+size_t grp_domain_bytes_for(int LD, int G)
+{
+    if (LD == 16) return G == 8 ? grp_domain_bytes<16, 8>() : grp_domain_bytes<16, 16>();
+    if (LD == 32) return G == 8 ? grp_domain_bytes<32, 8>() : G == 16 ? grp_domain_bytes<32, 16>() : grp_domain_bytes<32, 32>();
+    return G == 16 ? grp_domain_bytes<64, 16>() : grp_domain_bytes<64, 32>();
+}
+TpdKernel thread_plan_kernel(const Plan &pl, int LD, bool expo, bool grad)
+{
+    return pl.groups ? grp_kernel_for(LD, pl.groups, expo) : tpd_kernel_for(LD, expo, grad);
+}
 size_t tpdr_warp_bytes_for(int LD)
 {
     return LD == 16 ? tpdr_warp_bytes<16>() : LD == 32 ? tpdr_warp_bytes<32>() : tpdr64_warp_bytes();
+}
+
+// The domains of each colour, replica after replica, or with `interleave`
+// dealt round-robin over the replicas (the first of each, then the second, ...).
+std::vector<std::vector<uint32_t>> colour_lists(const kmc_ctx *c, bool interleave)
+{
+    std::vector<std::vector<uint32_t>> lists(4);
+    if (!interleave) {
+        for (uint32_t g = 0; g < (uint32_t)c->n_dom; ++g) lists[domain_colour(c, g)].push_back(g);
+    } else {
+        std::vector<std::vector<std::vector<uint32_t>>> per(4, std::vector<std::vector<uint32_t>>(c->n_rep));
+        for (uint32_t g = 0; g < (uint32_t)c->n_dom; ++g) per[domain_colour(c, g)][c->dom_rep[g]].push_back(g);
+        for (int q = 0; q < 4; ++q) {
+            size_t longest = 0;
+            for (const auto &v : per[q]) longest = std::max(longest, v.size());
+            for (size_t j = 0; j < longest; ++j)
+                for (const auto &v : per[q])
+                    if (j < v.size()) lists[q].push_back(v[j]);
+        }
+    }
+    return lists;
 }
 
 // THREADS plan for L_d = 16, 32: warps of 32 domains of one colour, one per
@@ -596,20 +640,7 @@ kmc_status plan_thread_rows(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
     pl = Plan();
     pl.mode = KMC_LAUNCH_THREADS;
     pl.wpb = wpb;
-    std::vector<std::vector<uint32_t>> lists(4);
-    if (!interleave) {
-        for (uint32_t g = 0; g < (uint32_t)c->n_dom; ++g) lists[domain_colour(c, g)].push_back(g);
-    } else {
-        std::vector<std::vector<std::vector<uint32_t>>> per(4, std::vector<std::vector<uint32_t>>(c->n_rep));
-        for (uint32_t g = 0; g < (uint32_t)c->n_dom; ++g) per[domain_colour(c, g)][c->dom_rep[g]].push_back(g);
-        for (int q = 0; q < 4; ++q) {
-            size_t longest = 0;
-            for (const auto &v : per[q]) longest = std::max(longest, v.size());
-            for (size_t j = 0; j < longest; ++j)
-                for (const auto &v : per[q])
-                    if (j < v.size()) lists[q].push_back(v[j]);
-        }
-    }
+    std::vector<std::vector<uint32_t>> lists = colour_lists(c, interleave);
     size_t most = 0;
     for (const auto &lq : lists) most = std::max(most, (lq.size() + 31) / 32);
     for (size_t i = 0; i < most; ++i) {
@@ -624,6 +655,126 @@ kmc_status plan_thread_rows(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
     pl.slot_g.resize((size_t)pl.n_cta * wpb * 32, 0xFFFFFFFFu);
     pl.smem = (size_t)wpb * tpdr_warp_bytes_for(c->LD);
     return KMC_OK;
+}
+
+kmc_status check_plan(kmc_ctx *c, const Plan &pl);
+
+// Group plan for L_d = 16, 32, 64 (grp_kernel) with G lanes per domain: sets
+// of 32 / G domains of one colour of one replica, replica after replica or
+// (`interleave`) dealt round-robin over the replicas.  With ns = 1 every set
+// has a warp of its own, the warps of set i of the four colours next to each
+// other in the grid; otherwise a warp takes ns / 2 sets of colours 0 and 1 or
+// of colours 3 and 2, so that colours 1 and 2, which do not wait for each
+// other, still run side by side.  wpb 0: a whole replica per CTA where 16
+// warps hold it (all its halos then stay in shared memory), else 4 warps.
+kmc_status plan_groups(kmc_ctx *c, int G, int ns, int wpb, Plan &pl, bool interleave)
+{
+    if (!grp_kernel_for(c->LD, G, true)) return fail(c, KMC_EINVAL, "no lane-group kernel for L_d = %d, G = %d", c->LD, G);
+    const int dpw = 32 / G;
+    // set i of the four colours holds domains first .. first + n - 1 of a replica's colour lists
+    struct Set { int r, first, n; };
+    std::vector<Set> sets;
+    int most = 0;
+    for (int r = 0; r < c->n_rep; ++r) {
+        const int per = c->Dx[r] * c->Dx[r] / 4;
+        most = std::max(most, (per + dpw - 1) / dpw);
+        for (int i = 0; i < per && !interleave; i += dpw) sets.push_back({r, i, std::min(dpw, per - i)});
+    }
+    for (int i = 0; i < most && interleave; ++i)
+        for (int r = 0; r < c->n_rep; ++r) {
+            const int per = c->Dx[r] * c->Dx[r] / 4;
+            if (i * dpw < per) sets.push_back({r, i * dpw, std::min(dpw, per - i * dpw)});
+        }
+    if (wpb == 0) {
+        wpb = 4;
+        while (4 * most <= MAX_WPB && wpb < 4 * most) wpb *= 2;
+    }
+    pl = Plan();
+    pl.mode = KMC_LAUNCH_THREADS;
+    pl.groups = G;
+    pl.wpb = wpb;
+    pl.max_rt = ns;
+    const size_t half = ns / 2;
+    const size_t warps = (ns == 1) ? 4 * sets.size() : 2 * ((sets.size() + half - 1) / half);
+    pl.n_cta = (int)((warps + wpb - 1) / wpb);
+    const size_t n_warps = (size_t)pl.n_cta * wpb;
+    pl.smem = GRP_TABLE_BYTES + (size_t)wpb * ns * dpw * grp_domain_bytes_for(c->LD, G);
+    pl.cta_col_off.assign(n_warps * ns, 4u);
+    pl.slot_g.assign(n_warps * ns * dpw, 0xFFFFFFFFu);
+    pl.slot_nb.assign(n_warps * ns * dpw * 4, 0u);
+    std::vector<uint32_t> where(c->n_dom, 0);
+    for (size_t w = 0; w < warps; ++w) {
+        for (int s = 0; s < ns; ++s) {
+            static const int pair[2][2] = {{0, 1}, {3, 2}};
+            const int col = (ns == 1) ? (int)(w % 4) : pair[w % 2][s / half];
+            const size_t set = (ns == 1) ? w / 4 : (w / 2) * half + s % half;
+            if (set >= sets.size()) continue;
+            pl.cta_col_off[w * ns + s] = (uint32_t)col;
+            const Set &t = sets[set];
+            const int D = c->Dx[t.r], h = D / 2;
+            for (int i = 0; i < t.n; ++i) {
+                // the (first + i)-th domain of the colour in row-major order
+                const int by = 2 * ((t.first + i) / h) + (col >> 1), bx = 2 * ((t.first + i) % h) + (col & 1);
+                const uint32_t g = c->dom_off[t.r] + (uint32_t)(by * D + bx);
+                const size_t slot = (w * ns + s) * dpw + i;
+                pl.slot_g[slot] = g;
+                where[g] = (uint32_t)slot;
+            }
+        }
+    }
+    const uint32_t per_cta = (uint32_t)(wpb * ns * dpw);
+    for (uint32_t slot = 0; slot < pl.slot_g.size(); ++slot) {
+        const uint32_t g = pl.slot_g[slot];
+        if (g == 0xFFFFFFFFu) continue;
+        const uint32_t r = c->dom_rep[g], off = c->dom_off[r], D = (uint32_t)c->Dx[r], d = g - off;
+        const uint32_t bx = d % D, by = d / D, cta = slot / per_cta;
+        const uint32_t nb[4] = {off + (by ? by - 1 : D - 1) * D + bx, off + (by + 1 < D ? by + 1 : 0) * D + bx,
+                                off + by * D + (bx ? bx - 1 : D - 1), off + by * D + (bx + 1 < D ? bx + 1 : 0)};
+        for (int side = 0; side < 4; ++side) {
+            const uint32_t at = where[nb[side]];
+            pl.slot_nb[(size_t)slot * 4 + side] = (at / per_cta == cta) ? 0x80000000u | (at % per_cta) : nb[side];
+        }
+    }
+    return KMC_OK;
+}
+
+// THREADS plan of L_d = 16, 32, 64: lane groups per domain while the domains
+// are few enough for about two of their warps per scheduler, else (and with
+// scores) one thread per domain.  Fewer lanes per domain cost fewer
+// instructions per event, more lanes shorten it, and beyond one active warp
+// per scheduler they compete; with long visits (k >= 8, most of the time in
+// events) two colours per warp and half as many warps are faster, with short
+// ones a warp per colour, whose fixed work hides behind the other colours.
+// Measured, us per schedule (G, ns; thread = one thread per domain):
+//   1024 domains of 32x32, k = 4:  (32,1) 5.8  (32,2) 7.3  (8,1) 7.6  thread 16.2
+//   1024 domains of 32x32, k = 16: (32,1) 36.7 (32,2) 33.4 (8,1) 43.8 thread 72.8
+//   4096 domains of 16x16, k = 4:  (8,1) 15.2  (8,2) 16.2  (16,1) 16.8 thread 28.9
+//   4096 domains of 32x32, k = 8:  (8,2) 28.2  (8,1) 31.2  (16,2) 30.0 thread 48.0
+//   12288 domains of 32x32, k = 8: (8,2) 47.8  thread 50.1; 16384: (8,2) 59.2 thread 50.3
+//   1024 domains of 64x64, k = 8:  (32,2) 26.9 (16,1) 36.5 thread 70.1
+//   9216 domains of 64x64, k = 8:  (16,2) 81.4 thread 77.9
+kmc_status plan_thread_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
+{
+    if (!c->grad) {
+        int64_t steps = 0;
+        for (int r = 0; r < c->n_rep; ++r) steps += (int64_t)c->kr[r] * c->Dx[r] * c->Dx[r];
+        const bool lengthy = steps >= 8ll * c->n_dom;
+        auto warps = [&](int G, int ns) {
+            int64_t sets = 0;
+            for (int r = 0; r < c->n_rep; ++r) sets += (c->Dx[r] * c->Dx[r] / 4 + 32 / G - 1) / (32 / G);
+            return 4 * sets / ns;
+        };
+        const int most = std::min(c->LD, 32), fewest = (c->LD == 64) ? 16 : 8;
+        const int ns = lengthy ? 2 : 1;
+        const int64_t room = (int64_t)(lengthy ? 4 : 8) * c->sm_count;
+        for (int G = most; G >= fewest; G /= 2)
+            if (warps(G, ns) <= room && plan_groups(c, G, ns, wpb, pl, interleave) == KMC_OK && check_plan(c, pl) == KMC_OK)
+                return KMC_OK;
+        if (warps(fewest, 2) <= (int64_t)10 * c->sm_count && plan_groups(c, fewest, 2, wpb, pl, interleave) == KMC_OK &&
+            check_plan(c, pl) == KMC_OK)
+            return KMC_OK;
+    }
+    return plan_thread_rows(c, wpb ? wpb : 1, pl, interleave);
 }
 
 // CTAs of `wpb` warps for a thread plan: a phase takes as many rounds as its
@@ -650,8 +801,9 @@ kmc_status check_plan(kmc_ctx *c, const Plan &pl)
     if (pl.mode == KMC_LAUNCH_THREADS) {
         if (c->grad && (c->LD == 8 || c->LD == 64))
             return fail(c, KMC_EINVAL, "the thread-per-domain plan of L_d = %d has no score kernel", c->LD);
+        if (c->grad && pl.groups) return fail(c, KMC_EINVAL, "the lane-group kernel carries no scores");
         for (int e = 0; e < 2; ++e) {
-            const void *kern = (const void *)tpd_kernel_for(c->LD, e == 0, c->grad);
+            const void *kern = (const void *)thread_plan_kernel(pl, c->LD, e == 0, c->grad);
             if (pl.smem > 0) {
                 if (pl.smem > (size_t)c->smem_optin)
                     return fail(c, KMC_EINVAL, "thread plan needs %zu bytes of shared memory per CTA (%d available)",
@@ -746,7 +898,7 @@ kmc_status default_plan(kmc_ctx *c)
     if ((!c->grad && (c->LD == 8 || c->LD == 64)) || c->LD == 16 || c->LD == 32) {
         Plan pl;
         const kmc_status st = (c->LD == 8) ? plan_threads(c, balanced_thread_ctas(c, 4), 4, pl)
-                                           : plan_thread_rows(c, 1, pl, false);
+                                           : plan_thread_domains(c, 0, pl, false);
         if (st == KMC_OK && install_plan(c, pl) == KMC_OK) return KMC_OK;
         cudaGetLastError();
     }
@@ -1383,7 +1535,7 @@ kmc_status kmc_set_launch(kmc_ctx *c, int32_t mode, int32_t size, int32_t warps_
             // one domain per thread: the grid follows from the domains; size
             // 0 or 1: the replicas one after another, 2: round-robin
             if (size < 0 || size > 2) return fail(c, KMC_EINVAL, "thread plans of L_d = %d take size 0, 1 or 2", c->LD);
-            if ((s = plan_thread_rows(c, warps_per_cta, pl, size == 2)) != KMC_OK) return s;
+            if ((s = plan_thread_domains(c, warps_per_cta, pl, size == 2)) != KMC_OK) return s;
         } else if ((s = plan_threads(c, size > 0 ? size : balanced_thread_ctas(c, warps_per_cta), warps_per_cta, pl)) !=
                    KMC_OK) {
             // size 0: the balanced grid of the library's choice
@@ -1563,7 +1715,7 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     const Plan &pl = c->plan;
     const bool cluster = pl.mode == KMC_LAUNCH_CLUSTER;
     const bool threads = pl.mode == KMC_LAUNCH_THREADS;
-    RunKernel kern = threads ? tpd_kernel_for(c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad)
+    RunKernel kern = threads ? thread_plan_kernel(pl, c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad)
                              : run_kernel_for(c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad, cluster);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     const bool prof = c->prof && !cap;
