@@ -554,7 +554,7 @@ kmc_status plan_threads(kmc_ctx *c, int n_cta, int wpb, Plan &pl)
         pl.slot_g.insert(pl.slot_g.end(), lists[q].begin(), lists[q].end());
         pl.cta_col_off[q + 1] = (uint32_t)pl.slot_g.size();
     }
-    pl.smem = 0;
+    pl.smem = (size_t)wpb * 32 * TPD_THREAD_BYTES;
     return KMC_OK;
 }
 
@@ -777,19 +777,21 @@ kmc_status plan_thread_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
     return plan_thread_rows(c, wpb ? wpb : 1, pl, interleave);
 }
 
-// CTAs of `wpb` warps for a thread plan: a phase takes as many rounds as its
-// busiest thread has domains, so the threads are the domains of a colour
-// divided by the rounds that up to three CTAs of 4 warps per SM need (the
-// fastest grid on the 512-replica batch, measured; more resident warps left
-// threads with one domain beside threads with two).
+// CTAs of `wpb` warps for a thread plan: at most three CTAs of 4 warps per SM
+// (what the kernel's registers allow).  A phase takes as many rounds as its
+// busiest thread has domains; while the last round of the full grid is at
+// least half full the full grid is faster (every SM equally loaded: the
+// 512-replica batch, 1.6 domains per thread, 19.1 -> 18.4 ms), else the
+// threads are the domains of a colour divided by the rounds.
 int balanced_thread_ctas(const kmc_ctx *c, int wpb)
 {
     const int64_t per_colour = (c->n_dom + 3) / 4;
     const int64_t tmax = (int64_t)3 * 128 * c->sm_count;
     const int64_t rounds = std::max<int64_t>(1, (per_colour + tmax - 1) / tmax);
-    const int64_t threads = (per_colour + rounds - 1) / rounds;
+    const bool full = rounds > 1 && 2 * (per_colour - (rounds - 1) * tmax) >= tmax;
+    const int64_t threads = full ? tmax : (per_colour + rounds - 1) / rounds;
     const int64_t per_cta = (int64_t)wpb * 32;
-    return (int)std::max<int64_t>(1, (threads + per_cta - 1) / per_cta);
+    return (int)std::max<int64_t>(1, full ? threads / per_cta : (threads + per_cta - 1) / per_cta);
 }
 
 // Can this plan run?  Shared memory, cluster support and (GRID) co-residency.

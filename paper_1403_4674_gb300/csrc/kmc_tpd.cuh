@@ -33,6 +33,10 @@
 namespace kmcdev {
 
 constexpr uint64_t TPD_COL0 = 0x0101010101010101ull; // column 0 of every row
+constexpr int TPD_CACHE = 2;  // rounds of a phase whose domains a thread keeps in shared memory
+// shared memory of a thread: 0 and the cumulative class rates, domain and
+// replica of its visits
+constexpr int TPD_THREAD_BYTES = 80 + 4 * TPD_CACHE * 8;
 constexpr int TPD_OBS_WORDS = 4; // open record per domain: record | steps << 32, bonds | mag << 32, mantissa, exponent
 
 // Bit y of an 8-bit column mask to bit 8y (column 0 of row y).
@@ -60,11 +64,10 @@ struct TpdPlanes {
         const uint64_t D = (T >> 8) | ((uint64_t)(hS & 0xFFu) << 56);
         const uint64_t Wn = ((T << 1) & ~TPD_COL0) | tpd_col_spread(hW);
         const uint64_t En = ((T >> 1) & ~(TPD_COL0 << 7)) | (tpd_col_spread(hE) << 7);
-        const uint64_t s1 = U ^ D, c1 = U & D, s2 = Wn ^ En, c2 = Wn & En;
-        const uint64_t t0 = s1 & s2;
-        b0 = s1 ^ s2;
-        b1 = c1 ^ c2 ^ t0;
-        b2 = (c1 & c2) | (c1 & t0) | (c2 & t0);
+        const uint64_t x = U ^ D ^ Wn, m = (U & D) | (U & Wn) | (D & Wn), k = x & En; // U + D + Wn = x + 2 m
+        b0 = x ^ En;
+        b1 = m ^ k;
+        b2 = m & k;
     }
     // sites with exactly q up neighbours
     __device__ __forceinline__ uint64_t eq(int q) const
@@ -75,44 +78,93 @@ struct TpdPlanes {
 };
 
 // Cumulative class rates C_c = sum_{c' <= c} n_c' A_c' of tile T (classes
-// 5 (s > 0) + q in order 0..9); C[9] = R'.
-__device__ __forceinline__ void tpd_rates(uint64_t T, const TpdPlanes &pl, const uint64_t (&A)[10], uint64_t (&C)[10])
+// 5 (s > 0) + q in order 0..9); C[9] = R'.  Of the five counts of a spin
+// direction four are counted bits of the planes (q = 1 and 3 in b0, q = 2
+// and 3 in b1, both in b0 b1, q = 4 in b2) and q = 0 has the rest.
+// C_0 .. C_8 go to shared memory (element c + 1 of cc, element 0 holding 0;
+// stride elements apart), their high words and R' stay in registers.
+__device__ __forceinline__ uint64_t tpd_rates(uint64_t T, const TpdPlanes &pl, const uint64_t (&A)[10], uint32_t (&Ch)[9],
+                                              uint64_t *cc, int stride)
 {
+    const uint32_t nup = (uint32_t)__popcll(T);
+    const uint64_t b01 = pl.b0 & pl.b1;
     uint64_t acc = 0;
 #pragma unroll
-    for (int c = 0; c < 10; ++c) {
-        const uint64_t m = ((c >= 5) ? T : ~T) & pl.eq(c % 5);
-        acc += (uint64_t)__popcll(m) * A[c];
-        C[c] = acc;
+    for (int s = 0; s < 2; ++s) {
+        const uint64_t S = s ? T : ~T;
+        const uint32_t p0 = (uint32_t)__popcll(pl.b0 & S), p1 = (uint32_t)__popcll(pl.b1 & S),
+                       n3 = (uint32_t)__popcll(b01 & S), n4 = (uint32_t)__popcll(pl.b2 & S);
+        const uint32_t n[5] = {(s ? nup : 64u - nup) - (p0 + p1 - n3) - n4, p0 - n3, p1 - n3, n3, n4};
+#pragma unroll
+        for (int q = 0; q < 5; ++q) {
+            acc += (uint64_t)n[q] * A[5 * s + q];
+            if (5 * s + q < 9) {
+                cc[(5 * s + q + 1) * stride] = acc;
+                Ch[5 * s + q < 9 ? 5 * s + q : 8] = (uint32_t)(acc >> 32);
+            }
+        }
     }
+    return acc;
+}
+
+// Product of a normalised mantissa (value m 2^(e - 63)) and V / 2^64 where on
+// (V then 2^11 or more).
+__device__ __forceinline__ void tpd_mul(uint64_t &m, int &e, uint64_t V, bool on)
+{
+    V = on ? V : 1ull << 63;
+    uint64_t hi = __umul64hi(m, V), lo = m * V;
+    if ((uint32_t)(hi >> 32) == 0) { // (V below 2^33) by 32 bits first
+        hi = (hi << 32) | (lo >> 32);
+        lo <<= 32;
+        e -= 32;
+    }
+    const int z = __clz((int)(uint32_t)(hi >> 32));
+    const uint32_t h = __funnelshift_l((uint32_t)hi, (uint32_t)(hi >> 32), z),
+                   l = __funnelshift_l((uint32_t)(lo >> 32), (uint32_t)hi, z);
+    m = on ? ((uint64_t)h << 32) | l : m;
+    e -= on ? z : 0;
 }
 
 // The open record of domain g goes to its replica's record (records past
 // the launch's last one are dropped), as the warp kernel's flush.
 template <bool EXPO>
-__device__ __forceinline__ void tpd_flush(const RunParams &P, const uint64_t *ob, uint32_t r)
+__device__ __forceinline__ void tpd_flush(const RunParams &P, const ulonglong2 &ob, const ulonglong2 &clk, uint32_t r)
 {
-    const uint32_t o = (uint32_t)ob[0];
+    const uint32_t o = (uint32_t)ob.x;
     if (o == NO_RECORD || (int64_t)o >= P.n_obs) return;
     unsigned long long *acc = P.obs_acc + ((size_t)o * P.n_rep + r) * OBS_WORDS;
-    const int bonds = (int)(uint32_t)ob[1], mag = (int)(uint32_t)(ob[1] >> 32);
+    const int bonds = (int)(uint32_t)ob.y, mag = (int)(uint32_t)(ob.y >> 32);
     if (bonds != 0) atomicAdd(&acc[0], (unsigned long long)(long long)bonds);
     if (mag != 0) atomicAdd(&acc[1], (unsigned long long)(long long)mag);
-    const uint32_t steps = (uint32_t)(ob[0] >> 32);
-    const double dt = EXPO ? domain_time(true, ob[2], (int64_t)ob[3], 0, P.lambda) : __ddiv_rn((double)steps, P.lambda);
+    const uint32_t steps = (uint32_t)(ob.x >> 32);
+    const double dt = EXPO ? domain_time(true, clk.x, (int64_t)clk.y, 0, P.lambda) : __ddiv_rn((double)steps, P.lambda);
     atomicAdd(reinterpret_cast<double *>(&acc[2]), dt);
 }
 
 // Persistent kernel: thread t visits, in every colour phase, the domains
 // t, t + T, t + 2T, ... of that colour's list (T = threads of the grid).
 // P.cta_col_off holds the five offsets of the colour-sorted domain list
-// P.slot_g; P.obs_dom the open records (TPD_OBS_WORDS per domain).  Bounds
-// of two 4-warp CTAs per SM let the compiler keep about 150 registers (three
-// CTAs still fit): 2 % faster on the 512-replica batch than its own choice
-// of 102 with more values recomputed.
+// P.slot_g; P.obs_dom the open records (TPD_OBS_WORDS per domain).
+//
+// What bounds it: with the 166 registers of a visit three 4-warp CTAs fit an
+// SM, and three warps per scheduler issue on about half of the cycles, so a
+// visit's latency counts as much as its instructions.  Hence the order of a
+// visit (the domain's words asked for first, then the first draw, then the
+// halo), the next step's draw in one straight line with this step's event,
+// counters added without reading them, and C_{c-1} through shared memory
+// (the integer pipe is the busiest one, 60 %).  512 uneven replicas, 60
+// schedules, records every 10, on 456 CTAs: k = 1 6.1 -> 5.2 ms, k = 4 8.0 ->
+// 7.4, k = 16 19.7 -> 18.4, k = 32 36.2 -> 33.3.  Threads that jump between
+// their own events (targets in shared memory) took 8.5 / 19.3 / 33.7 ms at k
+// = 4 / 16 / 32, four CTAs per SM at 128 registers 7.9 / 19.9 / 36.4.
 template <bool EXPO>
-__global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
+__global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
 {
+    extern __shared__ __align__(16) uint8_t smem[];
+    uint64_t *cum = reinterpret_cast<uint64_t *>(smem) + threadIdx.x; // 0, C_0 .. C_8 at stride blockDim.x
+    cum[0] = 0;
+    const int bd = blockDim.x;
+    uint2 *cache = reinterpret_cast<uint2 *>(cum + 10 * bd); // element (colour TPD_CACHE + round) bd: {domain, replica}
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthreads = gridDim.x * blockDim.x;
     const uint32_t *col_off = P.cta_col_off;
@@ -136,6 +188,12 @@ __global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
         }
     }
 
+    for (int c = 0; c < 4; ++c)
+        for (int m = 0; m < TPD_CACHE; ++m) {
+            const uint32_t i = col_off[c] + (uint32_t)tid + (uint32_t)m * (uint32_t)nthreads;
+            const uint32_t g = i < col_off[c + 1] ? col_list[i] : col_list[col_off[c]];
+            cache[(c * TPD_CACHE + m) * bd] = make_uint2(g, P.dom_rep[g]);
+        }
     unsigned spins = 0; // halo re-reads (profiling)
     bool ok = true;
     uint32_t gc0 = 0, gc1 = 0, gc2 = 0, gc3 = 0; // completed visit groups per colour in this launch
@@ -174,29 +232,62 @@ __global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
         for (uint32_t m = 0; m < rounds && ok; ++m) {
             const uint32_t i = lo + (uint32_t)tid + m * (uint32_t)nthreads;
             const bool has = i < hi;
-            const uint32_t g = has ? col_list[i] : col_list[lo];
-            const uint32_t r = P.dom_rep[g];
-            const uint32_t base = P.rep_dom_off[r];
-            const uint32_t d = g - base;
-            const int Dx = P.rep_Dx[r];
-            const int bx = (int)(d % (uint32_t)Dx), by = (int)(d / (uint32_t)Dx);
-            const uint32_t gN = base + (uint32_t)(((by + Dx - 1) % Dx) * Dx + bx);
-            const uint32_t gS = base + (uint32_t)(((by + 1) % Dx) * Dx + bx);
-            const uint32_t gW = base + (uint32_t)(by * Dx + (bx + Dx - 1) % Dx);
-            const uint32_t gE = base + (uint32_t)(by * Dx + (bx + 1) % Dx);
-            // everything that does not depend on the halo first
-            const int k = P.rep_k[r];
-            const int total = has ? nf * k : 0;
-            const uint64_t seed = P.rep_seed[r];
-            const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
-            uint64_t A[10];
-#pragma unroll
-            for (int c = 0; c < 10; ++c) A[c] = __ldg(&P.rep_A[(size_t)r * 16 + c]);
+            uint2 gr;
+            if (m < TPD_CACHE) {
+                gr = cache[(colour * TPD_CACHE + (int)m) * bd];
+            } else {
+                gr.x = has ? col_list[i] : col_list[lo];
+                gr.y = P.dom_rep[gr.x];
+            }
+            const uint32_t g = gr.x, r = gr.y;
+            // everything that does not depend on the halo first: the domain's
+            // words are asked for before the draws, which take longer than they do
             uint64_t T = tile64[g];
             uint64_t *ctr = P.dctr + (size_t)g * DCTR_WORDS;
             uint64_t H = ctr[DCTR_HASH];
             uint64_t clkM = ctr[DCTR_CLKM];
             int64_t clkE = (int64_t)ctr[DCTR_CLKE];
+            const int64_t o = P.n_obs > 0 ? (P.obs_pass ? pass : pass / nph) / P.obs_every : 0;
+            uint64_t *ob = P.obs_dom + (size_t)g * TPD_OBS_WORDS;
+            ulonglong2 ob01 = make_ulonglong2(0, 0), obM = make_ulonglong2(0, 0);
+            if (P.n_obs > 0) {
+                ob01 = *reinterpret_cast<const ulonglong2 *>(ob);
+                obM = *reinterpret_cast<const ulonglong2 *>(ob + 2);
+            }
+            const uint32_t base = __ldg(&P.rep_dom_off[r]);
+            const uint32_t Dx = (uint32_t)__ldg(&P.rep_Dx[r]);
+            const int k = __ldg(&P.rep_k[r]);
+            const uint64_t seed = __ldg(&P.rep_seed[r]);
+            uint64_t A[10];
+#pragma unroll
+            for (int c = 0; c < 10; ++c) A[c] = __ldg(&P.rep_A[(size_t)r * 16 + c]);
+            const uint32_t d = g - base;
+            const uint32_t by = d / Dx, bx = d - by * Dx;
+            const uint32_t gN = by == 0 ? g + (Dx - 1) * Dx : g - Dx, gS = by == Dx - 1 ? g - (Dx - 1) * Dx : g + Dx;
+            const uint32_t gW = bx == 0 ? g + Dx - 1 : g - 1, gE = bx == Dx - 1 ? g - (Dx - 1) : g + 1;
+            const int total = has ? nf * k : 0;
+            const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
+            uint64_t vM = 1ull << 63;
+            int vE = 0;
+            const int smax = (int)__reduce_max_sync(FULL_WARP, (unsigned)total);
+            // Step st = f k + j of the visit is step j of global phase np0 + f: its
+            // target (~0 past the last step), and its clock variate into the
+            // visit's product.
+            auto draw = [&](int st) {
+                const bool act = st < total;
+                const int f = st >= k ? 1 : 0; // at most two phases fuse
+                const uint64_t np = np0 + (uint64_t)f;
+                const uint4 w = philox4x32_10(make_uint4((uint32_t)(st - (f ? k : 0)), d, (uint32_t)np,
+                                                         (uint32_t)(np >> 32) & 0xFFFFFFu), key);
+                if (EXPO) {
+                    // clock variate v = V 2^-53, V the top 53 bits plus 1 (2^53 wraps
+                    // to 0: v = 1 leaves the product)
+                    const uint64_t V = ((((uint64_t)w.w << 32) | w.z) & ~0x7FFull) + 0x800ull;
+                    tpd_mul(vM, vE, V, act && V != 0);
+                }
+                return act ? (((uint64_t)w.y << 32) | w.x) >> 1 : ~0ull;
+            };
+            uint64_t tgt = draw(0);
             // halo: the N neighbour's S row, the S neighbour's N row, the W
             // neighbour's E column, the E neighbour's W column (half 0 of
             // each), stamped with the neighbour's completed visits; the warp
@@ -246,43 +337,30 @@ __global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
 
             TpdPlanes pl;
             pl.build(T, hN, hS, hW, hE);
-            uint64_t C[10];
-            tpd_rates(T, pl, A, C);
-            uint64_t flips = 0;
+            uint32_t Ch[9];
+            uint64_t R = tpd_rates(T, pl, A, Ch, cum, bd);
+            uint32_t flips = 0;
             int dbonds = 0, dmag = 0;
-            uint64_t vM = 1ull << 63;
-            int64_t vE = 0;
-            const int smax = (int)__reduce_max_sync(FULL_WARP, (unsigned)total);
-            // step s = f k + j of the visit: step j of global phase np0 + f
-            int j = -1;
-            uint64_t np = np0;
-            for (int s = 0; s < smax; ++s) {
-                const bool act = s < total;
-                if (++j == k) {
-                    j = 0;
-                    ++np;
+            // All lanes step together.  The next step's draw and the event of this
+            // one do not depend on each other: in one straight line they fill each
+            // other's latencies, so a lane without an event runs the event with
+            // no effect.  Only a step that is null in all 32 domains skips it.
+            for (int st = 0; st < smax; ++st) {
+                const bool ev = tgt < R; // else a null step (App. A: the diagonal 1 - R/n_d)
+                if (!__any_sync(FULL_WARP, ev)) {
+                    tgt = draw(st + 1);
+                    continue;
                 }
-                const uint4 w = philox4x32_10(make_uint4((uint32_t)j, d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu),
-                                              key);
-                const uint64_t tgt = (((uint64_t)w.y << 32) | w.x) >> 1;
-                if (EXPO && act) {
-                    // clock variate v = V 2^-53 as a normalised mantissa m / 2^63
-                    // times 2^(10 - z), into the visit's product
-                    const uint64_t V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
-                    const int z = __clzll((long long)V);
-                    mant_mul(vM, vE, V << z, (int64_t)(10 - z));
-                }
-                if (!act || tgt >= C[9]) continue; // null step (App. A: the diagonal 1 - R/n_d)
-                // class: the first c with tgt < C_c; C_{c-1} and A_c along with it
+                const uint64_t next = draw(st + 1);
+                // class: the first c with tgt < C_c; by the high words it may come
+                // out too high where those are equal
                 int c = 0;
-                uint64_t Cprev = 0, Ac = A[0];
+                const uint32_t th = (uint32_t)(tgt >> 32);
 #pragma unroll
-                for (int cc = 0; cc < 9; ++cc) {
-                    const bool past = tgt >= C[cc];
-                    c = past ? cc + 1 : c;
-                    Cprev = past ? C[cc] : Cprev;
-                    Ac = past ? A[cc + 1] : Ac;
-                }
+                for (int cc = 0; cc < 9; ++cc) c += (th >= Ch[cc]) ? 1 : 0;
+                uint64_t Cprev = cum[c * bd];
+                while (tgt < Cprev) Cprev = cum[--c * bd];
+                const uint64_t Ac = __ldg(&P.rep_A[(size_t)r * 16 + c]);
                 // exact jj = floor((tgt - C_{c-1}) / A_c) < n_c <= 64: an FP32
                 // estimate rounded toward the lower side is jj or jj - 1, and
                 // one integer comparison decides which
@@ -292,22 +370,24 @@ __global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
                 jj = (x - (uint64_t)jj * Ac >= Ac) ? jj + 1u : jj;
                 const int qc = (c >= 5) ? c - 5 : c;
                 const uint64_t mask = ((c >= 5) ? T : ~T) & pl.eq(qc);
-                const int site = select_bit(mask, jj);
-                T ^= 1ull << site;
-                H = (H ^ ((np << 32) | ((uint64_t)j << 16) | (uint64_t)site)) * HASH_PRIME;
-                ++flips;
+                const int site = select_bit(mask, jj) & 63;
+                T ^= ev ? 1ull << site : 0ull;
+                const int f = st >= k ? 1 : 0;
+                const uint64_t np = np0 + (uint64_t)f;
+                const uint64_t h = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)site)) * HASH_PRIME;
+                H = ev ? h : H;
+                flips += ev ? 1u : 0u;
                 // flipping spin s with neighbour sum 2 qc - 4 changes the bond
                 // sum by -2 s (2 qc - 4) and the magnetisation by -2 s
-                const int sgn = (c >= 5) ? 1 : -1;
-                dbonds -= 2 * sgn * (2 * qc - 4);
-                dmag -= 2 * sgn;
-                if (s + 1 < total) {
-                    pl.build(T, hN, hS, hW, hE);
-                    tpd_rates(T, pl, A, C);
-                }
+                const int g2 = ev ? (c >= 5 ? -2 : 2) : 0;
+                dbonds += g2 * (2 * qc - 4);
+                dmag += g2;
+                pl.build(T, hN, hS, hW, hE);
+                R = tpd_rates(T, pl, A, Ch, cum, bd);
+                tgt = next;
             }
             if (!has) continue;
-            if (EXPO) mant_mul(clkM, clkE, vM, vE); // the domain clock takes the visit's product
+            if (EXPO) mant_mul(clkM, clkE, vM, (int64_t)vE); // the domain clock takes the visit's product
             // edges first (neighbours wait for them), then tile and counters
             uint64_t *ew = P.edges + (size_t)g * EDGE_WORDS;
             const uint64_t cnt = (uint64_t)after << 32;
@@ -315,32 +395,32 @@ __global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
             st_cg(ew + 2 * EDGE_S, cnt | (T >> 56));
             st_cg(ew + 2 * EDGE_W, cnt | tpd_col_gather(T));
             st_cg(ew + 2 * EDGE_E, cnt | tpd_col_gather(T >> 7));
-            if (flips) tile64w[g] = T;
-            ctr[DCTR_HASH] = H;
-            ctr[DCTR_FLIPS] += flips;
-            ctr[DCTR_STEPS] += (uint64_t)total;
-            ctr[DCTR_CLKM] = clkM;
-            ctr[DCTR_CLKE] = (uint64_t)clkE;
+            if (flips) {
+                tile64w[g] = T;
+                ctr[DCTR_HASH] = H;
+                atomicAdd(reinterpret_cast<unsigned long long *>(ctr + DCTR_FLIPS), (unsigned long long)flips);
+            }
+            atomicAdd(reinterpret_cast<unsigned long long *>(ctr + DCTR_STEPS), (unsigned long long)total); // (no result: no wait)
+            if (EXPO) {
+                ctr[DCTR_CLKM] = clkM;
+                ctr[DCTR_CLKE] = (uint64_t)clkE;
+            }
             if (P.n_obs > 0) {
                 // the visit's changes belong to the first record at or after its pass
-                const int64_t o = (P.obs_pass ? pass : pass / nph) / P.obs_every;
-                uint64_t *ob = P.obs_dom + (size_t)g * TPD_OBS_WORDS;
-                uint64_t o0 = ob[0], o1 = ob[1], om = ob[2];
-                int64_t oe = (int64_t)ob[3];
-                if ((int64_t)(uint32_t)o0 != o) {
-                    tpd_flush<EXPO>(P, ob, r);
-                    o0 = (uint64_t)(uint32_t)o;
-                    o1 = 0;
+                uint64_t om = obM.x;
+                int64_t oe = (int64_t)obM.y;
+                if ((int64_t)(uint32_t)ob01.x != o) {
+                    tpd_flush<EXPO>(P, ob01, obM, r);
+                    ob01 = make_ulonglong2((uint64_t)(uint32_t)o, 0);
                     om = 1ull << 63;
                     oe = 0;
                 }
-                const uint32_t steps = (uint32_t)(o0 >> 32) + (uint32_t)total;
-                const int bonds = (int)(uint32_t)o1 + dbonds, mag = (int)(uint32_t)(o1 >> 32) + dmag;
-                if (EXPO) mant_mul(om, oe, vM, vE);
-                ob[0] = (uint64_t)(uint32_t)o0 | ((uint64_t)steps << 32);
-                ob[1] = (uint64_t)(uint32_t)bonds | ((uint64_t)(uint32_t)mag << 32);
-                ob[2] = om;
-                ob[3] = (uint64_t)oe;
+                const uint32_t steps = (uint32_t)(ob01.x >> 32) + (uint32_t)total;
+                const int bonds = (int)(uint32_t)ob01.y + dbonds, mag = (int)(uint32_t)(ob01.y >> 32) + dmag;
+                if (EXPO) mant_mul(om, oe, vM, (int64_t)vE);
+                *reinterpret_cast<ulonglong2 *>(ob) = make_ulonglong2(
+                    (uint64_t)(uint32_t)o | ((uint64_t)steps << 32), (uint64_t)(uint32_t)bonds | ((uint64_t)(uint32_t)mag << 32));
+                *reinterpret_cast<ulonglong2 *>(ob + 2) = make_ulonglong2(om, (uint64_t)oe);
             }
         }
         if (colour == 0) ++gc0;
@@ -356,7 +436,8 @@ __global__ void __launch_bounds__(128, 2) tpd_kernel(const RunParams P)
         for (int c = 0; c < 4; ++c) {
             for (uint32_t i = col_off[c] + (uint32_t)tid; i < col_off[c + 1]; i += (uint32_t)nthreads) {
                 const uint32_t g = col_list[i];
-                tpd_flush<EXPO>(P, P.obs_dom + (size_t)g * TPD_OBS_WORDS, P.dom_rep[g]);
+                const ulonglong2 *ob = reinterpret_cast<const ulonglong2 *>(P.obs_dom + (size_t)g * TPD_OBS_WORDS);
+                tpd_flush<EXPO>(P, ob[0], ob[1], P.dom_rep[g]);
             }
         }
     }
