@@ -962,7 +962,7 @@ kmc_status launch_observe(kmc_ctx *c, cudaStream_t s, int time_mode, unsigned lo
     const bool expo = time_mode == KMC_TIME_EXPONENTIAL;
     P.horizon = time_mode == KMC_TIME_HORIZON;
     P.dtau = c->dtau;
-    const int blocks = grid_for(c->n_dom, 8);
+    const int blocks = grid_for(c->n_dom, 8 * (c->LD == 8 ? observe_domains<8>() : observe_domains<16>()));
 #define KMC_OBS(LDV)                                                                                         \
     if (expo) observe_kernel<LDV, true><<<blocks, 256, 0, s>>>(P, c->d_dom_rep, c->n_dom, c->visits_done, acc); \
     else observe_kernel<LDV, false><<<blocks, 256, 0, s>>>(P, c->d_dom_rep, c->n_dom, c->visits_done, acc);
@@ -1107,7 +1107,7 @@ kmc_status upload_rates(kmc_ctx *c)
 kmc_status launch_pack(kmc_ctx *c, cudaStream_t s)
 {
     LayoutParams P = layout_params(c);
-    const int blocks = grid_for(c->n_dom, 8);
+    const int blocks = grid_for(c->n_dom, c->LD == 8 ? 256 : 8); // a thread or a warp per domain
     switch (c->LD) {
     case 8: pack_kernel<8><<<blocks, 256, 0, s>>>(P); break;
     case 16: pack_kernel<16><<<blocks, 256, 0, s>>>(P); break;
@@ -1122,7 +1122,7 @@ kmc_status launch_pack(kmc_ctx *c, cudaStream_t s)
 kmc_status launch_unpack(kmc_ctx *c, cudaStream_t s)
 {
     LayoutParams P = layout_params(c);
-    const int blocks = grid_for(c->n_dom, 8);
+    const int blocks = grid_for(c->n_dom, c->LD == 8 ? 256 : 8);
     switch (c->LD) {
     case 8: unpack_kernel<8><<<blocks, 256, 0, s>>>(P); break;
     case 16: unpack_kernel<16><<<blocks, 256, 0, s>>>(P); break;
@@ -1751,7 +1751,7 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
         c->prof_events.emplace_back(ev0, ev1);
     }
     if (want_obs && n_obs > 0) {
-        finalize_obs_kernel<<<grid_for(c->n_rep, 128), 128, 0, s>>>(base, c->d_obs_acc, n_obs, c->n_rep, c->d_L, c->d_Dx,
+        finalize_obs_kernel<<<grid_for(c->n_rep, 4), 128, 0, s>>>(base, c->d_obs_acc, n_obs, c->n_rep, c->d_L, c->d_Dx,
                                                                     c->J, c->d_h, obs_dev, c->grad ? 6 : 4);
         ++c->launches;
         CUDA_TRY(c, cudaGetLastError());

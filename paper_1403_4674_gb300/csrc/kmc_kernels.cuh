@@ -1290,9 +1290,16 @@ struct LayoutParams {
 // init = INIT_PER_REPLICA takes each replica's mode from rep_init (INIT_KEEP leaves it alone).
 __global__ void init_spins_kernel(const LayoutParams P, int init)
 {
+    // Replicas follow one another without gaps and hold whole blocks of 128
+    // sites, so block t starts at byte 128 t.  A warp draws 32 blocks, a lane
+    // each, and writes their 4 KB as whole 512-byte lines: 16 bytes per lane
+    // and round (8 per lane where the buffer is not 16-byte aligned).
     const uint64_t total = P.rep_blk_off[P.n_rep];
-    for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total;
-         t += (uint64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31;
+    const bool wide = (reinterpret_cast<uintptr_t>(P.spins) & 15u) == 0;
+    const uint64_t warp = (blockIdx.x * (uint64_t)blockDim.x + threadIdx.x) >> 5, nwarps = ((uint64_t)gridDim.x * blockDim.x) >> 5;
+    for (uint64_t t0 = warp * 32; t0 < total; t0 += nwarps * 32) {
+        const uint64_t t = t0 + lane < total ? t0 + lane : total - 1;
         int lo = 0, hi = P.n_rep - 1;
         while (lo < hi) {
             const int mid = (lo + hi + 1) >> 1;
@@ -1300,43 +1307,105 @@ __global__ void init_spins_kernel(const LayoutParams P, int init)
         }
         const int r = lo;
         const int mode = (init == INIT_PER_REPLICA) ? P.rep_init[r] : init;
-        if (mode == INIT_KEEP) continue;
-        const uint64_t b = t - P.rep_blk_off[r];
         uint4 w = make_uint4(~0u, ~0u, ~0u, ~0u);
         if (mode == 0) {
+            const uint64_t b = t - P.rep_blk_off[r];
             const uint64_t seed = P.rep_seed[r];
             w = philox4x32_10(make_uint4((uint32_t)b, (uint32_t)(b >> 32), 0u, TAG_INIT << 24),
                               make_uint2((uint32_t)seed, (uint32_t)(seed >> 32)));
         }
-        const uint32_t words[4] = {w.x, w.y, w.z, w.w};
-        uint64_t *out = reinterpret_cast<uint64_t *>(P.spins + P.rep_site_off[r] + b * 128);
-#pragma unroll
-        for (int q = 0; q < 16; ++q) {
-            const uint32_t byte = (words[q >> 2] >> (8 * (q & 3))) & 0xFFu;
-            uint64_t v = ((uint64_t)byte * 0x0101010101010101ull) & 0x8040201008040201ull;
+        const unsigned skip = __ballot_sync(FULL_WARP, mode == INIT_KEEP || t0 + lane >= total);
+        auto spins8 = [](uint32_t byte) {
+            uint64_t v = ((uint64_t)(byte & 0xFFu) * 0x0101010101010101ull) & 0x8040201008040201ull;
             v = ((v + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
-            out[q] = ~0ull ^ (v * 0xFEull);
+            return ~0ull ^ (v * 0xFEull);
+        };
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            // round i: blocks 4 i .. 4 i + 3, lane l bytes 16 (l % 8) .. of block 4 i + l / 8
+            const int src = 4 * i + (lane >> 3);
+            const uint32_t x = __shfl_sync(FULL_WARP, w.x, src), y = __shfl_sync(FULL_WARP, w.y, src),
+                           z = __shfl_sync(FULL_WARP, w.z, src), u = __shfl_sync(FULL_WARP, w.w, src);
+            const int q = (lane >> 1) & 3;
+            const uint32_t half = ((q == 0 ? x : q == 1 ? y : q == 2 ? z : u) >> (16 * (lane & 1))) & 0xFFFFu;
+            if (!((skip >> src) & 1u)) {
+                uint64_t *out = reinterpret_cast<uint64_t *>(P.spins + (t0 + src) * 128 + 16 * (lane & 7));
+                const uint64_t v0 = spins8(half), v1 = spins8(half >> 8);
+                if (wide) {
+                    *reinterpret_cast<ulonglong2 *>(out) = make_ulonglong2(v0, v1);
+                } else {
+                    out[0] = v0;
+                    out[1] = v1;
+                }
+            }
         }
     }
 }
 
-// int8 spins -> bit tiles + edges; one warp per domain; bytes must be +-1.
+// Eight int8 spins to a bit each (bit i: spin i up); ok: every byte is +-1.
+__device__ __forceinline__ uint32_t pack8(uint64_t x, bool &ok)
+{
+    const uint64_t neg = (x >> 7) & 0x0101010101010101ull;
+    ok = ok && x == (0x0101010101010101ull | (neg * 0xFEull));
+    return (uint32_t)(((neg ^ 0x0101010101010101ull) * 0x0102040810204080ull) >> 56);
+}
+// and back
+__device__ __forceinline__ uint64_t unpack8(uint32_t byte)
+{
+    uint64_t v = ((uint64_t)(byte & 0xFFu) * 0x0101010101010101ull) & 0x8040201008040201ull;
+    v = ((v + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
+    return ~0ull ^ (v * 0xFEull);
+}
+
+// int8 spins -> bit tiles + edges; bytes must be +-1.  8x8 domains: one
+// thread each (consecutive threads' rows are consecutive in memory, every row
+// one 8-byte load); larger ones: one warp each, rows as 16-byte loads where
+// the buffer is 16-byte aligned (rows then are: their offsets are multiples
+// of 16).
 template <int LD>
 __global__ void pack_kernel(const LayoutParams P)
 {
     using G = Geo<LD>;
     using row_t = typename G::row_t;
     using mem_t = typename G::mem_t;
+    if (LD == 8) {
+        bool ok = true;
+        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.n_dom; g += gridDim.x * blockDim.x) {
+            const uint32_t r = P.dom_rep[g];
+            const int L = P.rep_L[r], Dx = P.rep_Dx[r];
+            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
+            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
+            const uint64_t *src = reinterpret_cast<const uint64_t *>(
+                P.spins + P.rep_site_off[r] + (uint64_t)(by * 8) * L + (uint64_t)bx * 8);
+            uint64_t x[8];
+#pragma unroll
+            for (int y = 0; y < 8; ++y) x[y] = src[(size_t)y * (L / 8)];
+            uint64_t T = 0;
+#pragma unroll
+            for (int y = 0; y < 8; ++y) T |= (uint64_t)pack8(x[y], ok) << (8 * y);
+            reinterpret_cast<uint64_t *>(P.tiles)[g] = T;
+            // column 0 of every row (bits 8 y) to bit y
+            auto column = [](uint64_t t) { return ((t & 0x0101010101010101ull) * 0x0102040810204080ull) >> 56; };
+            ulonglong2 *e = reinterpret_cast<ulonglong2 *>(P.edges + (uint64_t)g * EDGE_WORDS);
+            e[EDGE_N] = make_ulonglong2(T & 0xFFull, 0ull);
+            e[EDGE_S] = make_ulonglong2(T >> 56, 0ull);
+            e[EDGE_W] = make_ulonglong2(column(T), 0ull);
+            e[EDGE_E] = make_ulonglong2(column(T >> 7), 0ull);
+        }
+        if (!ok) atomicCAS(P.err, 0, ERR_SPIN);
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
+    const bool wide = (reinterpret_cast<uintptr_t>(P.spins) & 15u) == 0;
     for (int g = wg; g < P.n_dom; g += nw) {
         const uint32_t r = P.dom_rep[g];
         const int L = P.rep_L[r], Dx = P.rep_Dx[r];
         const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
-        const int bx = (int)(d % (uint32_t)Dx), by = (int)(d / (uint32_t)Dx);
+        const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
         row_t S[G::RPL];
-        bool bad = false;
+        bool ok = true;
 #pragma unroll
         for (int t = 0; t < G::RPL; ++t) {
             S[t] = 0;
@@ -1344,19 +1413,25 @@ __global__ void pack_kernel(const LayoutParams P)
                 const int y = lane * G::RPL + t;
                 const uint64_t *src = reinterpret_cast<const uint64_t *>(
                     P.spins + P.rep_site_off[r] + (uint64_t)(by * LD + y) * L + (uint64_t)bx * LD);
+                uint64_t x[LD / 8];
+                if (wide) {
+#pragma unroll
+                    for (int q = 0; q < LD / 16; ++q) {
+                        const ulonglong2 v = reinterpret_cast<const ulonglong2 *>(src)[q];
+                        x[2 * q] = v.x;
+                        x[(2 * q + 1) % (LD / 8)] = v.y;
+                    }
+                } else {
+#pragma unroll
+                    for (int q = 0; q < LD / 8; ++q) x[q] = src[q];
+                }
                 uint64_t row = 0;
 #pragma unroll
-                for (int q = 0; q < LD / 8; ++q) {
-                    const uint64_t x = src[q];
-                    const uint64_t neg = (x >> 7) & 0x0101010101010101ull;
-                    bad |= (x != (0x0101010101010101ull | (neg * 0xFEull)));
-                    const uint64_t up = (~x >> 7) & 0x0101010101010101ull;
-                    row |= ((up * 0x0102040810204080ull) >> 56) << (8 * q);
-                }
+                for (int q = 0; q < LD / 8; ++q) row |= (uint64_t)pack8(x[q], ok) << (8 * q);
                 S[t] = (row_t)row;
             }
         }
-        if (__any_sync(FULL_WARP, bad) && lane == 0) atomicCAS(P.err, 0, ERR_SPIN);
+        if (!__all_sync(FULL_WARP, ok) && lane == 0) atomicCAS(P.err, 0, ERR_SPIN);
         mem_t *trow = reinterpret_cast<mem_t *>(P.tiles + (uint64_t)g * G::TILE_BYTES);
         if (lane < G::NACT) {
 #pragma unroll
@@ -1367,41 +1442,63 @@ __global__ void pack_kernel(const LayoutParams P)
     }
 }
 
-// bit tiles -> int8 spins; one warp per domain.
+// bit tiles -> int8 spins; as pack_kernel: one thread per 8x8 domain, one
+// warp per larger one.
 template <int LD>
 __global__ void unpack_kernel(const LayoutParams P)
 {
     using G = Geo<LD>;
     using mem_t = typename G::mem_t;
+    if (LD == 8) {
+        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.n_dom; g += gridDim.x * blockDim.x) {
+            const uint32_t r = P.dom_rep[g];
+            const int L = P.rep_L[r], Dx = P.rep_Dx[r];
+            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
+            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
+            const uint64_t T = reinterpret_cast<const uint64_t *>(P.tiles)[g];
+            uint64_t *dst = reinterpret_cast<uint64_t *>(P.spins + P.rep_site_off[r] + (uint64_t)(by * 8) * L + (uint64_t)bx * 8);
+#pragma unroll
+            for (int y = 0; y < 8; ++y) dst[(size_t)y * (L / 8)] = unpack8((uint32_t)(T >> (8 * y)));
+        }
+        return;
+    }
     const int lane = threadIdx.x & 31;
     const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
+    const bool wide = (reinterpret_cast<uintptr_t>(P.spins) & 15u) == 0;
     for (int g = wg; g < P.n_dom; g += nw) {
         const uint32_t r = P.dom_rep[g];
         const int L = P.rep_L[r], Dx = P.rep_Dx[r];
         const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
-        const int bx = (int)(d % (uint32_t)Dx), by = (int)(d / (uint32_t)Dx);
+        const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
         const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)g * G::TILE_BYTES);
-        if (lane < G::NACT) {
-#pragma unroll
-            for (int t = 0; t < G::RPL; ++t) {
-                const int y = lane * G::RPL + t;
-                const uint64_t row = (uint64_t)trow[y];
-                uint64_t *dst = reinterpret_cast<uint64_t *>(
-                    P.spins + P.rep_site_off[r] + (uint64_t)(by * LD + y) * L + (uint64_t)bx * LD);
-#pragma unroll
-                for (int q = 0; q < LD / 8; ++q) {
-                    const uint64_t byte = (row >> (8 * q)) & 0xFFull;
-                    uint64_t v = (byte * 0x0101010101010101ull) & 0x8040201008040201ull;
-                    v = ((v + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
-                    dst[q] = ~0ull ^ (v * 0xFEull);
-                }
+        int8_t *dst = P.spins + P.rep_site_off[r] + (uint64_t)(by * LD) * L + (uint64_t)bx * LD;
+        // LD / 16 lanes write one row, 16 bytes each, so that a store covers whole lines
+        constexpr int LPR = LD / 16 > 0 ? LD / 16 : 1;
+        for (int y = lane / LPR; y < LD; y += 32 / LPR) {
+            const int q = lane % LPR;
+            const uint32_t bits = (uint32_t)((uint64_t)trow[y] >> (16 * q));
+            uint64_t *out = reinterpret_cast<uint64_t *>(dst + (size_t)y * L + 16 * q);
+            const uint64_t v0 = unpack8(bits), v1 = unpack8(bits >> 8);
+            if (wide) {
+                *reinterpret_cast<ulonglong2 *>(out) = make_ulonglong2(v0, v1);
+            } else {
+                out[0] = v0;
+                out[1] = v1;
             }
         }
     }
 }
 
-// Observables of the current state from the global tiles and edges (kmc_observables).
+// Observables of the current state from the global tiles and edges
+// (kmc_observables, and the base of a launch's records).  A warp takes
+// OBSERVE_DOMAINS consecutive domains: their bond and spin sums by the whole
+// warp in turn (8x8: a lane each), then every domain's clock (an FP64
+// logarithm, this GPU's slowest arithmetic) in a lane of its own, and one
+// atomic per quantity and run of domains of a replica.  A warp per domain
+// with one lane's logarithm each took 1.49 ms on the 373,000 domains of the
+// 512-replica batch.
+template <int LD> __host__ __device__ constexpr int observe_domains() { return LD == 8 ? 32 : 8; }
 template <int LD, bool EXPO>
 __global__ void observe_kernel(const RunParams P, const uint32_t *dom_rep, int n_dom, int64_t visits,
                                unsigned long long *acc /* [n_rep][OBS_WORDS] */)
@@ -1409,75 +1506,153 @@ __global__ void observe_kernel(const RunParams P, const uint32_t *dom_rep, int n
     using G = Geo<LD>;
     using row_t = typename G::row_t;
     using mem_t = typename G::mem_t;
+    constexpr int DPW = observe_domains<LD>();
     const int lane = threadIdx.x & 31;
     const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int g = wg; g < n_dom; g += nw) {
-        const uint32_t r = dom_rep[g];
-        const int Dx = P.rep_Dx[r];
-        const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
-        const int bx = (int)(d % (uint32_t)Dx), by = (int)(d / (uint32_t)Dx);
-        const uint64_t gbase = (uint64_t)g - d;
-        const uint64_t *eS = P.edges + (gbase + (uint32_t)(((by + 1) % Dx) * Dx + bx)) * EDGE_WORDS;
-        const uint64_t *eE = P.edges + (gbase + (uint32_t)(by * Dx + (bx + 1) % Dx)) * EDGE_WORDS;
-        const uint64_t hS = (eS[2 * EDGE_N] & 0xFFFFFFFFull) | (eS[2 * EDGE_N + 1] << 32);
-        const uint64_t hE = (eE[2 * EDGE_W] & 0xFFFFFFFFull) | (eE[2 * EDGE_W + 1] << 32);
-        row_t S[G::RPL];
-        const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)g * G::TILE_BYTES);
+    for (int g0 = wg * DPW; g0 < n_dom; g0 += nw * DPW) {
+        int bonds = 0, mag = 0; // of domain g0 + lane
+        // the edge words of the S neighbour's N row and the E neighbour's W column
+        auto halo = [&](int g, uint64_t &hS, uint64_t &hE) {
+            const uint32_t r = dom_rep[g];
+            const int Dx = P.rep_Dx[r];
+            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
+            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
+            const uint64_t gbase = (uint64_t)g - d;
+            const uint64_t *eS = P.edges + (gbase + (uint32_t)((by + 1 < Dx ? by + 1 : 0) * Dx + bx)) * EDGE_WORDS;
+            const uint64_t *eE = P.edges + (gbase + (uint32_t)(by * Dx + (bx + 1 < Dx ? bx + 1 : 0))) * EDGE_WORDS;
+            hS = (eS[2 * EDGE_N] & 0xFFFFFFFFull) | (eS[2 * EDGE_N + 1] << 32);
+            hE = (eE[2 * EDGE_W] & 0xFFFFFFFFull) | (eE[2 * EDGE_W + 1] << 32);
+        };
+        const int g = g0 + lane;
+        const bool mine = lane < DPW && g < n_dom;
+        if (LD == 8) {
+            if (mine) {
+                const uint64_t T = reinterpret_cast<const uint64_t *>(P.tiles)[g];
+                uint64_t hS, hE;
+                halo(g, hS, hE);
+                // unlike pairs to the east (column 7: the E neighbour's column 0) and to the south
+                uint64_t east = (hE & 0xFFull) * 0x0101010101010101ull & 0x8040201008040201ull; // bit y of row y
+                east = ((east + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
+                const uint64_t E = ((T >> 1) & ~(0x0101010101010101ull << 7)) | (east << 7), S = (T >> 8) | (hS << 56);
+                bonds = 128 - 2 * (__popcll(T ^ E) + __popcll(T ^ S));
+                mag = 2 * __popcll(T) - 64;
+            }
+        } else {
+            for (int i = 0; i < DPW && g0 + i < n_dom; ++i) {
+                uint64_t hS, hE;
+                halo(g0 + i, hS, hE);
+                row_t S[G::RPL];
+                const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)(g0 + i) * G::TILE_BYTES);
 #pragma unroll
-        for (int t = 0; t < G::RPL; ++t) S[t] = (lane < G::NACT) ? (row_t)trow[lane * G::RPL + t] : (row_t)0;
-        int bonds, mag;
-        domain_bonds_mag<LD>(S, hE, hS, lane, bonds, mag);
-        if (lane == 0) {
+                for (int t = 0; t < G::RPL; ++t) S[t] = (lane < G::NACT) ? (row_t)trow[lane * G::RPL + t] : (row_t)0;
+                int b, m;
+                domain_bonds_mag<LD>(S, hE, hS, lane, b, m);
+                if (lane == i) {
+                    bonds = b;
+                    mag = m;
+                }
+            }
+        }
+        double t = 0.0, sb = 0.0, sh = 0.0;
+        uint32_t r = 0;
+        if (mine) {
             const uint64_t *ctr = P.dctr + (uint64_t)g * DCTR_WORDS;
-            const double t = P.horizon ? __dmul_rn((double)visits, P.dtau)
-                                       : domain_time(EXPO, ctr[DCTR_CLKM], (int64_t)ctr[DCTR_CLKE],
-                                                     visits * (int64_t)P.rep_k[r], P.lambda);
-            unsigned long long *a = acc + (size_t)r * OBS_WORDS;
-            atomicAdd(&a[0], (unsigned long long)(long long)bonds);
-            atomicAdd(&a[1], (unsigned long long)(long long)mag);
-            atomicAdd(reinterpret_cast<double *>(&a[2]), t);
-            atomicAdd(reinterpret_cast<double *>(&a[3]), __longlong_as_double((long long)ctr[DCTR_SB]));
-            atomicAdd(reinterpret_cast<double *>(&a[4]), __longlong_as_double((long long)ctr[DCTR_SH]));
+            r = dom_rep[g];
+            t = P.horizon ? __dmul_rn((double)visits, P.dtau)
+                          : domain_time(EXPO, ctr[DCTR_CLKM], (int64_t)ctr[DCTR_CLKE], visits * (int64_t)P.rep_k[r],
+                                        P.lambda);
+            sb = __longlong_as_double((long long)ctr[DCTR_SB]);
+            sh = __longlong_as_double((long long)ctr[DCTR_SH]);
+        }
+        auto add = [&](uint32_t rep, int b, int m, double tt, double s1, double s2) {
+            unsigned long long *a = acc + (size_t)rep * OBS_WORDS;
+            atomicAdd(&a[0], (unsigned long long)(long long)b);
+            atomicAdd(&a[1], (unsigned long long)(long long)m);
+            atomicAdd(reinterpret_cast<double *>(&a[2]), tt);
+            if (s1 != 0.0) atomicAdd(reinterpret_cast<double *>(&a[3]), s1);
+            if (s2 != 0.0) atomicAdd(reinterpret_cast<double *>(&a[4]), s2);
+        };
+        const uint32_t r0 = __shfl_sync(FULL_WARP, r, 0);
+        if (__all_sync(FULL_WARP, !mine || r == r0)) {
+            bonds = __reduce_add_sync(FULL_WARP, bonds);
+            mag = __reduce_add_sync(FULL_WARP, mag);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                t += __shfl_xor_sync(FULL_WARP, t, off);
+                sb += __shfl_xor_sync(FULL_WARP, sb, off);
+                sh += __shfl_xor_sync(FULL_WARP, sh, off);
+            }
+            if (lane == 0) add(r0, bonds, mag, t, sb, sh);
+        } else if (mine) {
+            add(r, bonds, mag, t, sb, sh);
         }
     }
 }
 
 // Records {e, m, e*m, T (, score beta, score h)}: record o = base (the state
-// before the launch) + the changes of every record up to o.  One thread per
-// replica walks its records in order; the integer sums are exact and e, m
+// before the launch) + the changes of every record up to o.  One warp per
+// replica, 32 records at a time: loads and divisions side by side, the sums
+// in record order; the integer sums are exact and e, m
 // follow the oracle's FP64 formula.
 __global__ void finalize_obs_kernel(const unsigned long long *base /* [n_rep][OBS_WORDS] */,
                                          const unsigned long long *acc, int64_t n_obs, int n_rep,
                                          const int32_t *rep_L, const int32_t *rep_Dx, double J,
                                          const double *rep_h, double *out, int stride)
 {
-    const int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= n_rep) return;
+    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    if (r >= n_rep) return; // whole warps
     const unsigned long long *b0 = base + (size_t)r * OBS_WORDS;
     long long bonds = (long long)b0[0], mag = (long long)b0[1];
     double tsum = __longlong_as_double((long long)b0[2]);
     double sb = __longlong_as_double((long long)b0[3]), sh = __longlong_as_double((long long)b0[4]);
     const double N = (double)rep_L[r] * (double)rep_L[r];
     const double nD = (double)rep_Dx[r] * (double)rep_Dx[r];
-    for (int64_t o = 0; o < n_obs; ++o) {
-        const unsigned long long *a = acc + ((size_t)o * n_rep + r) * OBS_WORDS;
-        bonds += (long long)a[0];
-        mag += (long long)a[1];
-        tsum = __dadd_rn(tsum, __longlong_as_double((long long)a[2]));
-        sb = __dadd_rn(sb, __longlong_as_double((long long)a[3]));
-        sh = __dadd_rn(sh, __longlong_as_double((long long)a[4]));
-        const double b = (double)bonds, m = (double)mag;
-        const double e = __ddiv_rn(__dsub_rn(__dmul_rn(-J, b), __dmul_rn(rep_h[r], m)), N);
-        const double mm = __ddiv_rn(m, N);
-        double *w = out + ((size_t)o * n_rep + r) * stride;
-        w[0] = e;
-        w[1] = mm;
-        w[2] = __dmul_rn(e, mm);
-        w[3] = __ddiv_rn(tsum, nD);
-        if (stride >= 6) {
-            w[4] = sb;
-            w[5] = sh;
+    for (int64_t o0 = 0; o0 < n_obs; o0 += 32) {
+        const int64_t o = o0 + lane;
+        const int n = (int)(n_obs - o0 < 32 ? n_obs - o0 : 32);
+        long long vb = 0, vm = 0;
+        double vt = 0.0, v1 = 0.0, v2 = 0.0;
+        if (lane < n) {
+            const unsigned long long *a = acc + ((size_t)o * n_rep + r) * OBS_WORDS;
+            vb = (long long)a[0];
+            vm = (long long)a[1];
+            vt = __longlong_as_double((long long)a[2]);
+            v1 = __longlong_as_double((long long)a[3]);
+            v2 = __longlong_as_double((long long)a[4]);
+        }
+        // the running sums up to this lane's record, added in record order
+        long long mb = 0, mm = 0;
+        double mt = 0.0, m1 = 0.0, m2 = 0.0;
+        for (int i = 0; i < n; ++i) {
+            bonds += __shfl_sync(FULL_WARP, vb, i);
+            mag += __shfl_sync(FULL_WARP, vm, i);
+            tsum = __dadd_rn(tsum, __shfl_sync(FULL_WARP, vt, i));
+            if (stride >= 6) {
+                sb = __dadd_rn(sb, __shfl_sync(FULL_WARP, v1, i));
+                sh = __dadd_rn(sh, __shfl_sync(FULL_WARP, v2, i));
+            }
+            if (lane == i) {
+                mb = bonds;
+                mm = mag;
+                mt = tsum;
+                m1 = sb;
+                m2 = sh;
+            }
+        }
+        if (lane < n) {
+            const double b = (double)mb, m = (double)mm;
+            const double e = __ddiv_rn(__dsub_rn(__dmul_rn(-J, b), __dmul_rn(rep_h[r], m)), N);
+            const double mq = __ddiv_rn(m, N);
+            double *w = out + ((size_t)o * n_rep + r) * stride;
+            w[0] = e;
+            w[1] = mq;
+            w[2] = __dmul_rn(e, mq);
+            w[3] = __ddiv_rn(mt, nD);
+            if (stride >= 6) {
+                w[4] = m1;
+                w[5] = m2;
+            }
         }
     }
 }
@@ -1515,20 +1690,41 @@ __global__ void reset_counters_kernel(uint64_t *dctr, int n_dom)
     c[DCTR_STEPS] = 0;
 }
 
+// Score sums of domains g0 .. g1 - 1 in domain order, eight domains' loads at
+// a time ahead of their additions.
+__device__ __forceinline__ void replica_scores(const uint64_t *dctr, uint32_t g0, uint32_t g1, double &sb, double &sh)
+{
+    sb = 0.0;
+    sh = 0.0;
+    for (uint32_t g = g0; g < g1; g += 8) {
+        double b[8], h[8];
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i) {
+            const uint64_t *c = dctr + (uint64_t)(g + i < g1 ? g + i : g) * DCTR_WORDS;
+            b[i] = __longlong_as_double((long long)c[DCTR_SB]);
+            h[i] = __longlong_as_double((long long)c[DCTR_SH]);
+        }
+#pragma unroll
+        for (uint32_t i = 0; i < 8; ++i) {
+            if (g + i < g1) {
+                sb += b[i];
+                sh += h[i];
+            }
+        }
+    }
+}
+
 // per-replica score sums in fixed domain order (kmc_grad)
 __global__ void score_reduce_kernel(const uint64_t *dctr, const uint32_t *rep_dom_off, int n_rep,
                                     double *score, int reset, uint64_t *dctr_w)
 {
     const int r = blockIdx.x * blockDim.x + threadIdx.x;
     if (r >= n_rep) return;
-    double sb = 0.0, sh = 0.0;
-    for (uint32_t g = rep_dom_off[r]; g < rep_dom_off[r + 1]; ++g) {
-        sb += __longlong_as_double((long long)dctr[(uint64_t)g * DCTR_WORDS + DCTR_SB]);
-        sh += __longlong_as_double((long long)dctr[(uint64_t)g * DCTR_WORDS + DCTR_SH]);
-        if (reset) {
-            dctr_w[(uint64_t)g * DCTR_WORDS + DCTR_SB] = 0;
-            dctr_w[(uint64_t)g * DCTR_WORDS + DCTR_SH] = 0;
-        }
+    double sb, sh;
+    replica_scores(dctr, rep_dom_off[r], rep_dom_off[r + 1], sb, sh);
+    for (uint32_t g = rep_dom_off[r]; reset && g < rep_dom_off[r + 1]; ++g) {
+        dctr_w[(uint64_t)g * DCTR_WORDS + DCTR_SB] = 0;
+        dctr_w[(uint64_t)g * DCTR_WORDS + DCTR_SH] = 0;
     }
     score[2 * r] = sb;
     score[2 * r + 1] = sh;
@@ -1569,11 +1765,8 @@ __global__ void lr_estimate_kernel(const double *A, const double *M, int stride,
     __syncthreads();
     double sb = 0.0, sh = 0.0;
     for (int r = t; r < n_rep; r += blockDim.x) {
-        double xb = 0.0, xh = 0.0;
-        for (uint32_t g = rep_dom_off[r]; g < rep_dom_off[r + 1]; ++g) {
-            xb += __longlong_as_double((long long)dctr[(uint64_t)g * DCTR_WORDS + DCTR_SB]);
-            xh += __longlong_as_double((long long)dctr[(uint64_t)g * DCTR_WORDS + DCTR_SH]);
-        }
+        double xb, xh;
+        replica_scores(dctr, rep_dom_off[r], rep_dom_off[r + 1], xb, xh);
         const double c = A[(size_t)r * stride] - mean;
         sb += c * xb;
         sh += c * xh;
