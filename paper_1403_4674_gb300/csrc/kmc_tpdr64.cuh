@@ -56,9 +56,9 @@ struct Tpdr64Layout {
                          CH = CE + 1, CFL = CH + 1, CST = CH + 2, CCM = CH + 3, CCE = CH + 4, OB0 = CH + 5,
                          OB1 = OB0 + 1, OBM = OB0 + 2, OBE = OB0 + 3, CC = OB0 + 4, AT = CC + 11, MR = AT + 10,
                          TG = MR + 10, N64 = TG + CHUNK + 8;
-    // 32-bit words per lane: neighbour ids, phase offset f << 16 | step j of
-    // each step of the chunk
-    static constexpr int NBN = 0, NBS = 1, NBW = 2, NBE = 3, EB = 4, N32 = EB + CHUNK;
+    // 32-bit words per lane: neighbour ids, the events of the chunk (step |
+    // class << 5 | site << 9)
+    static constexpr int NBN = 0, NBS = 1, NBW = 2, NBE = 3, EV = 4, N32 = EV + CHUNK;
     static constexpr int WARP_BYTES = 32 * (8 * N64 + 4 * N32);
 };
 
@@ -72,10 +72,10 @@ __device__ __forceinline__ void t64_planes(uint64_t S, uint64_t U, uint64_t D, u
 {
     const uint64_t Wn = (S << 1) | wb;         // bit x: the spin at x - 1
     const uint64_t En = (S >> 1) | (eb << 63); // bit x: the spin at x + 1
-    const uint64_t s1 = U ^ D, c1 = U & D, s2 = Wn ^ En, c2 = Wn & En, t0 = s1 & s2;
-    b0 = s1 ^ s2;
-    b1 = c1 ^ c2 ^ t0;
-    b2 = (c1 & c2) | (c1 & t0) | (c2 & t0);
+    const uint64_t x = U ^ D ^ Wn, m = (U & D) | (U & Wn) | (D & Wn), k = x & En; // U + D + Wn = x + 2 m
+    b0 = x ^ En;
+    b1 = m ^ k;
+    b2 = m & k;
 }
 
 __device__ __forceinline__ uint64_t t64_eq(uint64_t b0, uint64_t b1, uint64_t b2, int q)
@@ -295,29 +295,25 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
             // counters to shared memory, clock variates into the visit's
             // product.  Step s = f k + j of the visit is step j of global
             // phase np0 + f.
-            uint32_t jcur = 0, fcur = 0;
             uint64_t vM = 1ull << 63;
-            int64_t vE = 0;
+            int vE = 0;
             auto draw = [&](int base) {
 #pragma unroll 4
                 for (int i = 0; i < CHUNK; ++i) {
                     uint64_t t = ~0ull;
-                    if (base + i < total) {
-                        const uint64_t np = np0 + fcur;
-                        const uint4 w = philox4x32_10(
-                            make_uint4(jcur, d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu), key);
+                    const int st = base + i;
+                    if (st < total) {
+                        const int f = st >= k ? 1 : 0; // at most two phases fuse
+                        const uint64_t np = np0 + (uint64_t)f;
+                        const uint4 w = philox4x32_10(make_uint4((uint32_t)(st - (f ? k : 0)), d, (uint32_t)np,
+                                                                 (uint32_t)(np >> 32) & 0xFFFFFFu), key);
                         t = (((uint64_t)w.y << 32) | w.x) >> 1;
                         if (EXPO) {
                             // clock variate v = V 2^-53 as a normalised mantissa
                             // m / 2^63 times 2^(10 - z)
                             const uint64_t V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
                             const int z = __clzll((long long)V);
-                            mant_mul(vM, vE, V << z, (int64_t)(10 - z));
-                        }
-                        at32(Lay::EB + i) = (fcur << 16) | jcur;
-                        if (++jcur == (uint32_t)k) {
-                            jcur = 0;
-                            ++fcur;
+                            mant_mul32(vM, vE, V << z, 10 - z);
                         }
                     }
                     at(Lay::TG + i) = t;
@@ -434,60 +430,84 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
                     C[8] = C[7] + W[8];
                     C[9] = C[7] + s89;
 #pragma unroll
-                    for (int c = 0; c < 10; ++c) at(Lay::CC + 1 + c) = C[c];
+                    for (int c = 0; c < 9; ++c) at(Lay::CC + 1 + c) = C[c];
                 };
                 rates();
                 uint64_t H = at(Lay::CH);
                 uint64_t colW = at(Lay::CW), colE = at(Lay::CE);
-                uint64_t flips = 0;
+                uint32_t ne = 0, flips = 0; // events of the chunk, of the visit
                 int dbonds = 0, dmag = 0;
+                // What the events add to the event hash, the bond sum and the
+                // magnetisation is worked off from the list of the chunk's events,
+                // after the visit's edges are published: the neighbours do not
+                // wait for it.
+                auto work_off = [&](int base) {
+                    const int most = (int)__reduce_max_sync(FULL_WARP, ne);
+                    for (int i = 0; i < most; ++i) {
+                        const uint32_t e = at32(Lay::EV + i);
+                        const int st = base + (int)(e & 31u), c = (int)((e >> 5) & 15u), f = st >= k ? 1 : 0;
+                        const uint64_t np = np0 + (uint64_t)f;
+                        const uint64_t h = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)(e >> 9))) * HASH_PRIME;
+                        const bool act = i < (int)ne;
+                        H = act ? h : H;
+                        // flipping spin s with neighbour sum 2 q - 4 changes the bond
+                        // sum by -2 s (2 q - 4) and the magnetisation by -2 s
+                        const int g2 = act ? (c < 5 ? 2 : -2) : 0;
+                        dbonds += g2 * (2 * (c < 5 ? c : c - 5) - 4);
+                        dmag += g2;
+                    }
+                    flips += ne;
+                    ne = 0;
+                };
                 bool corrupt = false; // counts and spins disagreed at some event
 
                 for (int base = 0; base < smax; base += CHUNK) {
-                    if (base > 0) draw(base);
+                    if (base > 0) {
+                        work_off(base - CHUNK);
+                        draw(base);
+                    }
                     // Each lane jumps from real event to real event of its own
                     // domain (the steps between are null: App. A, the diagonal
                     // 1 - R/n_d); the warp runs as many rounds as its busiest lane.
                     int i = 0; // this lane's next step, relative to the chunk
                     while (true) {
                         // the lane's next step with target < R' (targets past its
-                        // last step are ~0), eight at a time
+                        // last step are ~0)
                         uint64_t tgt = 0;
                         while (i < CHUNK) {
-                            const uint64_t R = C[9];
                             uint64_t t[8];
                             unsigned m = 0;
 #pragma unroll
                             for (int u = 0; u < 8; ++u) {
                                 t[u] = at(Lay::TG + i + u);
-                                m |= (t[u] < R ? 1u : 0u) << u;
+                                m |= (t[u] < C[9] ? 1u : 0u) << u;
                             }
                             if (m) {
-                                const int f = __ffs(m) - 1;
+                                const int f = __ffs((int)m) - 1;
                                 i += f;
                                 // t[f] by selection (no indexed registers)
-                                const uint64_t q0 = (f & 1) ? t[1] : t[0], q1 = (f & 1) ? t[3] : t[2];
-                                const uint64_t q2 = (f & 1) ? t[5] : t[4], q3 = (f & 1) ? t[7] : t[6];
-                                const uint64_t r0 = (f & 2) ? q1 : q0, r1 = (f & 2) ? q3 : q2;
-                                tgt = (f & 4) ? r1 : r0;
+                                uint64_t q[4];
+#pragma unroll
+                                for (int u = 0; u < 4; ++u) q[u] = (f & 1) ? t[2 * u + 1] : t[2 * u];
+                                q[0] = (f & 2) ? q[1] : q[0];
+                                q[1] = (f & 2) ? q[3] : q[2];
+                                tgt = (f & 4) ? q[1] : q[0];
                                 break;
+                            } else {
+                                i += 8;
                             }
-                            i += 8;
                         }
                         const bool ev = i < CHUNK;
                         if (!__any_sync(FULL_WARP, ev)) break;
                         if (!ev) continue;
-                        const uint32_t eb = at32(Lay::EB + i);
+                        const int ist = i; // the event's step in the chunk
                         ++i;
-                        const uint64_t np = np0 + (eb >> 16);
-                        const uint32_t j = eb & 0xFFFFu;
                         // class: the first c with tgt < C_c
                         int c = 0;
 #pragma unroll
                         for (int cc = 0; cc < 9; ++cc) c += (tgt >= C[cc]) ? 1 : 0;
                         const uint64_t Cprev = at(Lay::CC + c); // C_{c-1}, 0 for c = 0
-                        const uint64_t Ac = at(Lay::AT + c);
-                        const uint64_t Mc = at(Lay::MR + c);
+                        const uint64_t Ac = at(Lay::AT + c), Mc = at(Lay::MR + c);
                         // exact jj = floor((tgt - C_{c-1}) / A_c) < n_c <= 4096: with
                         // M_c = floor((2^64 - 1) / A_c) and x < 2^63, the high word
                         // of x M_c is jj or jj - 1, and one integer comparison
@@ -632,13 +652,8 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
                         h1hi += (hy == 1 ? bYhi : 0ull) + (ho == 1 ? bOhi : 0ull);
                         colW ^= (col == 0) ? (1ull << y) : 0ull;
                         colE ^= (col == LD - 1) ? (1ull << y) : 0ull;
-                        H = (H ^ ((np << 32) | ((uint64_t)j << 16) | (uint64_t)(y * LD + col))) * HASH_PRIME;
-                        ++flips;
-                        // flipping spin s with neighbour sum 2 qc - 4 changes the bond
-                        // sum by -2 s (2 qc - 4) and the magnetisation by -2 s
-                        const int sgn = up ? 1 : -1;
-                        dbonds -= 2 * sgn * (2 * qc - 4);
-                        dmag -= 2 * sgn;
+                        at32(Lay::EV + (int)ne) = (uint32_t)ist | ((uint32_t)c << 5) | ((uint32_t)(y * LD + col) << 9);
+                        ++ne;
                         rates();
                         corrupt |= bad;
                     }
@@ -658,6 +673,9 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
                     st_cg(ew + 2 * EDGE_W + 1, cnt | (uint32_t)(eW >> 32));
                     st_cg(ew + 2 * EDGE_E, cnt | (uint32_t)eE);
                     st_cg(ew + 2 * EDGE_E + 1, cnt | (uint32_t)(eE >> 32));
+                }
+                work_off((smax - 1) / CHUNK * CHUNK);
+                if (has) {
                     at(Lay::HFLO) = h0lo;
                     at(Lay::HFHI) = h0hi;
                     at(Lay::HFLO + 1) = h1lo;
@@ -671,7 +689,7 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
                         // the domain clock takes the visit's product
                         uint64_t m = at(Lay::CCM);
                         int64_t e2 = (int64_t)at(Lay::CCE);
-                        mant_mul(m, e2, vM, vE);
+                        mant_mul(m, e2, vM, (int64_t)vE);
                         at(Lay::CCM) = m;
                         at(Lay::CCE) = (uint64_t)e2;
                     }
@@ -693,7 +711,7 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
                         if (EXPO) {
                             uint64_t m = at(Lay::OBM);
                             int64_t e2 = (int64_t)at(Lay::OBE);
-                            mant_mul(m, e2, vM, vE);
+                            mant_mul(m, e2, vM, (int64_t)vE);
                             at(Lay::OBM) = m;
                             at(Lay::OBE) = (uint64_t)e2;
                         }
