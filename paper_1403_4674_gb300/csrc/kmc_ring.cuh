@@ -5,14 +5,14 @@
 //
 // Data parallelism is over trajectories (the paper's N_TRAJ independent
 // runs per setting, Eq. time dependent averages): one thread owns one
-// trajectory for the whole launch, its configuration a 64-bit register word
+// trajectory for the whole launch, its configuration one register word
 // (bit n set iff spin n is up).  Within a thread the domain processes of a
 // schedule run in schedule order, so the halo of a visit is the live word:
 // no other domain of the trajectory moves while it runs.  Observation records
 // per trajectory are coalesced stores; the ensemble sums over trajectories
 // (integers, so their order does not matter) are reduced per warp with
-// ballots and warp reductions, per CTA in shared memory, and added to global
-// memory with one atomic per CTA and quantity.
+// ballots and warp reductions and added to global memory with one atomic per
+// warp and quantity.
 #pragma once
 
 #include <cstdint>
@@ -27,7 +27,7 @@ using kmcdev::HASH_PRIME;
 constexpr int RING_CLASSES = 6;      // c = 3*up + (number of up neighbours)
 constexpr int RING_PHASE_SLOTS = 64; // Philox phase index np = n*64 + p
 constexpr int RING_ENS_FIXED = 4;    // sum bonds, sum mag, sum bonds*mag, sum mag^2; then per-site up counts
-constexpr int RING_BLOCK = 128;
+constexpr int RING_BLOCK = 64;
 constexpr uint32_t RING_TAG_PERM = 2u;
 
 struct RingParams {
@@ -47,39 +47,62 @@ struct RingParams {
     unsigned long long *ens; // [n_rec][4 + NS] or null (added to)
 };
 
+// A configuration is one word: 32 bits for rings of up to 32 spins (half the
+// instructions of every mask, shift and bit count), else 64.
+__device__ __forceinline__ int ring_popc(uint32_t v) { return __popc(v); }
+__device__ __forceinline__ int ring_popc(uint64_t v) { return __popcll(v); }
+
+// Position of the rr-th (0-based) set bit of m; rr < popc(m).
+__device__ __forceinline__ int ring_select(uint64_t m, uint32_t rr) { return kmcdev::select_bit(m, rr); }
+__device__ __forceinline__ int ring_select(uint32_t w, uint32_t rr)
+{
+    int pos = 0;
+    uint32_t c = __popc(w & 0xFFFFu);
+    if (rr >= c) { rr -= c; w >>= 16; pos += 16; }
+    c = __popc(w & 0xFFu); if (rr >= c) { rr -= c; w >>= 8; pos += 8; }
+    c = __popc(w & 0xFu);  if (rr >= c) { rr -= c; w >>= 4; pos += 4; }
+    c = __popc(w & 0x3u);  if (rr >= c) { rr -= c; w >>= 2; pos += 2; }
+    if (rr >= (w & 1u)) pos += 1;
+    return pos;
+}
+
 // Neighbour words of a ring of NS bits: bit n of lw is spin n-1, of rw spin n+1.
-__device__ __forceinline__ uint64_t ring_left(uint64_t S, int NS, uint64_t NM)
+template <typename word> __device__ __forceinline__ word ring_left(word S, int NS, word NM)
 {
     return ((S << 1) | (S >> (NS - 1))) & NM;
 }
-__device__ __forceinline__ uint64_t ring_right(uint64_t S, int NS, uint64_t NM)
+template <typename word> __device__ __forceinline__ word ring_right(word S, int NS, word NM)
 {
-    return (S >> 1) | ((S & 1ull) << (NS - 1));
+    return (S >> 1) | ((S & (word)1) << (NS - 1));
 }
 
-// Sites of class c = 3 up + q of one domain (DM: its sites).
-__device__ __forceinline__ uint64_t ring_class_mask(uint64_t S, uint64_t DM, int NS, uint64_t NM, int c)
+// Inclusive cumulative rates C_c = sum_{c' <= c} n_c' A_c' in class order 0..5
+// of one domain (DM: its sites), and the words that hold the neighbours.
+template <typename word>
+__device__ __forceinline__ void ring_cumulative(uint64_t (&C)[RING_CLASSES], word &lw, word &rw, word S, word DM, int NS,
+                                                word NM, const uint64_t (&A)[RING_CLASSES])
 {
-    const uint64_t lw = ring_left(S, NS, NM), rw = ring_right(S, NS, NM);
-    const int q = (c >= 3) ? c - 3 : c;
-    const uint64_t qm = (q == 0) ? ~(lw | rw) : ((q == 1) ? (lw ^ rw) : (lw & rw));
-    return ((c >= 3) ? S : ~S) & qm & DM;
-}
-
-// Inclusive cumulative rates C_c = sum_{c' <= c} n_c' A_c' in class order 0..5.
-__device__ __forceinline__ void ring_cumulative(uint64_t (&C)[RING_CLASSES], uint64_t S, uint64_t DM, int NS,
-                                                uint64_t NM, const uint64_t (&A)[RING_CLASSES])
-{
-    const uint64_t lw = ring_left(S, NS, NM), rw = ring_right(S, NS, NM);
-    const uint64_t q0 = ~(lw | rw), q1 = lw ^ rw, q2 = lw & rw;
-    const uint64_t up = S & DM, dn = ~S & DM;
-    const uint64_t M[RING_CLASSES] = {dn & q0, dn & q1, dn & q2, up & q0, up & q1, up & q2};
+    lw = ring_left(S, NS, NM);
+    rw = ring_right(S, NS, NM);
+    const word q0 = ~(lw | rw), q1 = lw ^ rw, q2 = lw & rw;
+    const word up = S & DM, dn = ~S & DM;
+    const word M[RING_CLASSES] = {dn & q0, dn & q1, dn & q2, up & q0, up & q1, up & q2};
     uint64_t acc = 0;
 #pragma unroll
     for (int c = 0; c < RING_CLASSES; ++c) {
-        acc += (uint64_t)__popcll(M[c]) * A[c];
+        acc += (uint64_t)(uint32_t)ring_popc(M[c]) * A[c];
         C[c] = acc;
     }
+}
+
+// One step's random numbers: its target, and its clock variate V 2^-53.
+struct RingDraw {
+    uint64_t tgt, V;
+};
+__device__ __forceinline__ RingDraw ring_draw(uint32_t j, uint32_t d, uint64_t np, uint2 key)
+{
+    const uint4 w = kmcdev::philox4x32_10(make_uint4(j, d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu), key);
+    return {(((uint64_t)w.y << 32) | w.x) >> 1, ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull};
 }
 
 // One domain process: domain d, k steps of global phase np.  Step j draws
@@ -90,67 +113,92 @@ __device__ __forceinline__ void ring_cumulative(uint64_t (&C)[RING_CLASSES], uin
 // n-fold way's cumulative selection of Sec. 2.1).  jj < n_c <= 64: an FP32
 // estimate with every rounding toward the lower side (x down, A_c up, the
 // reciprocal down, the product toward zero) is jj or jj - 1, and one exact
-// integer comparison decides.
-template <bool EXPO>
-__device__ __forceinline__ void ring_visit(uint64_t &S, uint64_t &H, int64_t &flips, uint64_t &clkM, int64_t &clkE,
-                                           int d, int Ld, int k, int NS, uint64_t NM, uint64_t DM0, uint64_t np,
-                                           uint2 key, const uint64_t (&A)[RING_CLASSES],
-                                           const float (&invA)[RING_CLASSES])
+// integer comparison decides.  The 32 trajectories of a warp step together;
+// the next step's draw does not depend on this step's event, so the two stand
+// in one straight line and fill each other's latencies, and a trajectory
+// without an event runs it without effect.  `cur` is the draw of step 0 on
+// entry and, with `more`, that of the next visit's (domain d2, phase np2) on
+// return; a variate enters the clock with its step.
+template <bool EXPO, typename word>
+__device__ __forceinline__ void ring_visit(word &S, uint64_t &H, int64_t &flips, uint64_t &clkM, int64_t &clkE, int d,
+                                           int Ld, int k, int NS, word NM, word DM0, uint64_t np, uint2 key,
+                                           const uint64_t (&A)[RING_CLASSES], const float (&invA)[RING_CLASSES],
+                                           unsigned lanes, RingDraw &cur, bool more, int d2, uint64_t np2)
 {
     const int first = d * Ld;
-    const uint64_t DM = DM0 << first;
+    const word DM = DM0 << first;
     uint64_t C[RING_CLASSES];
-    ring_cumulative(C, S, DM, NS, NM, A);
+    word lw, rw;
+    ring_cumulative(C, lw, rw, S, DM, NS, NM, A);
     for (int j = 0; j < k; ++j) {
-        const uint4 w = kmcdev::philox4x32_10(
-            make_uint4((uint32_t)j, (uint32_t)d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu), key);
-        const uint64_t tgt = (((uint64_t)w.y << 32) | w.x) >> 1;
+        const uint64_t tgt = cur.tgt;
+        const bool ev = tgt < C[RING_CLASSES - 1]; // else a null step
         if (EXPO) {
-            const uint64_t V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
-            const int z = __clzll((long long)V);
-            kmcdev::mant_mul(clkM, clkE, V << z, (int64_t)(10 - z));
+            const int z = __clzll((long long)cur.V);
+            kmcdev::mant_mul(clkM, clkE, cur.V << z, (int64_t)(10 - z));
         }
-        if (tgt >= C[RING_CLASSES - 1]) continue; // null step
-        uint64_t lo = 0, Ac = A[0];
-        float inv = invA[0];
-        int c = 0;
+        const bool last = j + 1 == k;
+        if (!last || more) cur = ring_draw(last ? 0u : (uint32_t)(j + 1), (uint32_t)(last ? d2 : d), last ? np2 : np, key);
+        if (__any_sync(lanes, ev)) {
+            uint64_t lo = 0, Ac = A[0];
+            float inv = invA[0];
+            int c = 0;
 #pragma unroll
-        for (int cc = 1; cc < RING_CLASSES; ++cc) {
-            if (tgt >= C[cc - 1]) {
-                lo = C[cc - 1];
-                Ac = A[cc];
-                inv = invA[cc];
-                c = cc;
+            for (int cc = 1; cc < RING_CLASSES; ++cc) {
+                const bool past = tgt >= C[cc - 1];
+                lo = past ? C[cc - 1] : lo;
+                Ac = past ? A[cc] : Ac;
+                inv = past ? invA[cc] : inv;
+                c = past ? cc : c;
             }
+            const uint64_t x = tgt - lo;
+            uint32_t jj = (uint32_t)__fmul_rz(kmcdev::u64_to_float_rz(x), inv);
+            jj = (x - (uint64_t)jj * Ac >= Ac) ? jj + 1u : jj;
+            const int q = (c >= 3) ? c - 3 : c;
+            const word qm = (q == 0) ? ~(lw | rw) : ((q == 1) ? (lw ^ rw) : (lw & rw));
+            const int site = ring_select(((c >= 3) ? S : ~S) & qm & DM, jj) & (int)(8 * sizeof(word) - 1);
+            S ^= ev ? (word)1 << site : (word)0;
+            flips += ev ? 1 : 0;
+            const uint64_t h = (H ^ ((np << 32) | ((uint64_t)j << 16) | (uint64_t)(site - first))) * HASH_PRIME;
+            H = ev ? h : H;
+            ring_cumulative(C, lw, rw, S, DM, NS, NM, A);
         }
-        const uint64_t x = tgt - lo;
-        uint32_t jj = (uint32_t)__fmul_rz(kmcdev::u64_to_float_rz(x), inv);
-        jj = (x - (uint64_t)jj * Ac >= Ac) ? jj + 1u : jj;
-        const int site = kmcdev::select_bit(ring_class_mask(S, DM, NS, NM, c), jj);
-        S ^= 1ull << site;
-        ++flips;
-        H = (H ^ ((np << 32) | ((uint64_t)j << 16) | (uint64_t)(site - first))) * HASH_PRIME;
-        ring_cumulative(C, S, DM, NS, NM, A);
     }
 }
 
 // Uniform random order of the n_dom domains of schedule n (the paper's
 // random schedule per sweep): Fisher-Yates, draw i (n_dom-1 down to 1) from
 // Philox {i, 0, n_lo, n_hi | TAG_PERM << 24}: position i swaps with
-// floor(x (i+1) / 2^64), x = w0 | w1 << 32.
-__device__ __forceinline__ void ring_perm(uint8_t *order, int n_dom, uint64_t n, uint2 key)
-{
-    for (int i = 0; i < n_dom; ++i) order[i] = (uint8_t)i;
-    for (int i = n_dom - 1; i >= 1; --i) {
-        const uint4 w = kmcdev::philox4x32_10(
-            make_uint4((uint32_t)i, 0u, (uint32_t)n, ((uint32_t)(n >> 32) & 0xFFFFFFu) | (RING_TAG_PERM << 24)), key);
-        const uint64_t x = ((uint64_t)w.y << 32) | w.x;
-        const int jx = (int)__umul64hi(x, (uint64_t)(i + 1));
-        const uint8_t t = order[i];
-        order[i] = order[jx];
-        order[jx] = t;
+// floor(x (i+1) / 2^64), x = w0 | w1 << 32.  Up to 16 domains: the order is 16
+// nibbles in a register; more: bytes in local memory.
+struct RingOrder {
+    uint64_t nib;
+    uint8_t order[64];
+    __device__ __forceinline__ void shuffle(int n_dom, uint64_t n, uint2 key)
+    {
+        nib = 0xFEDCBA9876543210ull;
+        if (n_dom > 16)
+            for (int i = 0; i < n_dom; ++i) order[i] = (uint8_t)i;
+        for (int i = n_dom - 1; i >= 1; --i) {
+            const uint4 w = kmcdev::philox4x32_10(
+                make_uint4((uint32_t)i, 0u, (uint32_t)n, ((uint32_t)(n >> 32) & 0xFFFFFFu) | (RING_TAG_PERM << 24)), key);
+            const uint64_t x = ((uint64_t)w.y << 32) | w.x;
+            const int jx = (int)__umul64hi(x, (uint64_t)(i + 1));
+            if (n_dom > 16) {
+                const uint8_t t = order[i];
+                order[i] = order[jx];
+                order[jx] = t;
+            } else {
+                const uint64_t dif = ((nib >> (4 * i)) ^ (nib >> (4 * jx))) & 0xFull;
+                nib ^= (dif << (4 * i)) ^ (dif << (4 * jx));
+            }
+        }
     }
-}
+    __device__ __forceinline__ int at(int n_dom, int p) const
+    {
+        return n_dom > 16 ? order[p] : (int)((nib >> (4 * p)) & 0xFull);
+    }
+};
 
 // Clock of a trajectory: the mean over domains of t_d (Sec. 2.1), i.e.
 // -ln(product of all its variates) / (N_S nu) (exponential) or
@@ -160,18 +208,22 @@ __device__ __forceinline__ double ring_clock(bool expo, uint64_t M, int64_t E, i
     return kmcdev::domain_time(expo, M, E, steps, __dmul_rn((double)NS, nu));
 }
 
-template <bool EXPO>
-__global__ void __launch_bounds__(RING_BLOCK, 6) ring_kernel(const RingParams P)
+// Two warps per CTA: a CTA's trajectories need nothing of each other (the
+// ensemble sums go out by warp), and small CTAs load the SMs evenly (48000
+// trajectories are 9.9 warps per SM; CTAs of 4 warps put 12 on some and 8 on
+// others).
+template <bool EXPO, typename word>
+__global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
 {
-    __shared__ int ens_blk[RING_ENS_FIXED + 64];
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int lane = threadIdx.x & 31;
     const bool active = tid < P.n_traj;
     const int r = active ? tid : 0;
     const int NS = P.NS, Ld = P.Ld, ND = NS / Ld, k = P.k;
     const int n_ens = RING_ENS_FIXED + NS;
-    const uint64_t NM = (NS == 64) ? ~0ull : ((1ull << NS) - 1ull);
-    const uint64_t DM0 = (Ld == 64) ? ~0ull : ((1ull << Ld) - 1ull);
+    constexpr int WB = 8 * (int)sizeof(word);
+    const word NM = (NS == WB) ? ~(word)0 : (((word)1 << (NS & (WB - 1))) - (word)1);
+    const word DM0 = (Ld == WB) ? ~(word)0 : (((word)1 << (Ld & (WB - 1))) - (word)1);
 
     uint64_t A[RING_CLASSES];
     float invA[RING_CLASSES]; // 1/A_c from below: A_c rounded up, reciprocal rounded down
@@ -183,43 +235,52 @@ __global__ void __launch_bounds__(RING_BLOCK, 6) ring_kernel(const RingParams P)
     const uint64_t seed = P.seed[r];
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     const double hr = P.h[r];
-    uint64_t S = P.state[r], H = P.hash[r], clkM = P.clkM[r];
+    word S = (word)P.state[r];
+    uint64_t H = P.hash[r], clkM = P.clkM[r];
     int64_t clkE = P.clkE[r], flips = P.flips[r], steps = P.steps[r];
-
-    if (P.ens != nullptr)
-        for (int i = threadIdx.x; i < n_ens; i += blockDim.x) ens_blk[i] = 0;
-    __syncthreads();
 
     const bool perm = P.schedule == kmcdev::SCHED_RANDOM_PERM;
     const int ncol = (ND == 1) ? 1 : 2;
     const int nph = perm ? ND : (P.schedule == kmcdev::SCHED_PALINDROME ? 2 * ncol : ncol);
-    uint8_t order[64];
-    int64_t passes = 0;
+    const unsigned lanes = __ballot_sync(FULL_WARP, active);
+    RingOrder order;
+    RingDraw cur = {0, 0};
+    int64_t rec = 0;
+    int until = P.obs_every; // passes before the next record
     for (int64_t nl = 0; nl < P.n_sched; ++nl) {
         const uint64_t n = (uint64_t)(P.sched_begin + nl);
-        if (perm && active) ring_perm(order, ND, n, key);
+        if (perm && active) order.shuffle(ND, n, key);
         for (int p = 0; p < nph; ++p) {
             const uint64_t np = n * RING_PHASE_SLOTS + (uint64_t)p;
-            if (active) {
+            if (active && k > 0) {
                 if (perm) {
-                    ring_visit<EXPO>(S, H, flips, clkM, clkE, order[p], Ld, k, NS, NM, DM0, np, key, A, invA);
+                    // the next visit is known up to the end of the sweep
+                    const int d = order.at(ND, p);
+                    if (p == 0) cur = ring_draw(0u, (uint32_t)d, np, key);
+                    const bool more = p + 1 < nph;
+                    ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, NM, DM0, np, key, A, invA, lanes, cur, more,
+                                     more ? order.at(ND, p + 1) : 0, np + 1);
                     steps += k;
                 } else {
                     // colour of phase p: 0 1 [1 0] (one colour when N_D = 1)
-                    const int col = (p < ncol) ? p : (2 * ncol - 1 - p);
-                    for (int d = col; d < ND; d += ncol) {
-                        ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, NM, DM0, np, key, A, invA);
+                    auto colour = [&](int q) { return (q < ncol) ? q : (2 * ncol - 1 - q); };
+                    if (p == 0 && nl == 0) cur = ring_draw(0u, 0u, np, key);
+                    for (int d = colour(p); d < ND; d += ncol) {
+                        const bool stay = d + ncol < ND, turn = p + 1 == nph;
+                        const bool more = stay || !turn || nl + 1 < P.n_sched;
+                        ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, NM, DM0, np, key, A, invA, lanes, cur, more,
+                                         stay ? d + ncol : turn ? 0 : colour(p + 1),
+                                         stay ? np : turn ? (n + 1) * RING_PHASE_SLOTS : np + 1);
                         steps += k;
                     }
                 }
             }
-            ++passes;
-            if (P.obs_every > 0 && passes % P.obs_every == 0) {
-                const int64_t rec = passes / P.obs_every - 1;
+            if (P.obs_every > 0 && --until == 0) {
+                until = P.obs_every;
                 // bonds = sum_n s_n s_{n+1}: NS - 2 * (number of unlike neighbour pairs)
-                const int unlike = __popcll((S ^ ring_left(S, NS, NM)) & NM);
+                const int unlike = ring_popc((S ^ ring_left(S, NS, NM)) & NM);
                 const int bonds = NS - 2 * unlike;
-                const int mag = 2 * __popcll(S & NM) - NS;
+                const int mag = 2 * ring_popc(S & NM) - NS;
                 if (active) {
                     const size_t o = (size_t)rec * P.n_traj + r;
                     if (P.obs) {
@@ -233,43 +294,33 @@ __global__ void __launch_bounds__(RING_BLOCK, 6) ring_kernel(const RingParams P)
                         v.w = ring_clock(EXPO, clkM, clkE, steps, NS, P.nu);
                         reinterpret_cast<double4_32a *>(P.obs)[o] = v;
                     }
-                    if (P.obs_state) P.obs_state[o] = S;
+                    if (P.obs_state) P.obs_state[o] = (uint64_t)S;
                 }
                 if (P.ens != nullptr) {
-                    // ensemble sums: warp reductions, then one shared atomic per warp
+                    // ensemble sums over the warp, lane i adding quantity i, i + 32, ...
+                    __syncwarp();
                     const int b = active ? bonds : 0, m = active ? mag : 0;
                     const int s0 = __reduce_add_sync(FULL_WARP, b);
                     const int s1 = __reduce_add_sync(FULL_WARP, m);
                     const int s2 = __reduce_add_sync(FULL_WARP, b * m);
                     const int s3 = __reduce_add_sync(FULL_WARP, m * m);
-                    int cnt = 0;
-                    for (int i = 0; i < NS; ++i) {
-                        const int ci = __popc(__ballot_sync(FULL_WARP, active && ((S >> i) & 1ull)));
-                        if (lane == (i & 31)) cnt = ci; // lane i%32 keeps site i's count (two sites when NS > 32)
-                        if (i == 31 || i == NS - 1) {
-                            if (lane <= (i & 31)) atomicAdd(&ens_blk[RING_ENS_FIXED + (i & ~31) + lane], cnt);
+                    unsigned long long *ens = P.ens + (size_t)rec * n_ens;
+                    int mine = (lane == 0) ? s0 : (lane == 1) ? s1 : (lane == 2) ? s2 : s3;
+                    for (int q = 0; q < n_ens; q += 32) {
+                        for (int i = (q == 0 ? RING_ENS_FIXED : 0); i < 32 && q + i < n_ens; ++i) {
+                            const int site = q + i - RING_ENS_FIXED;
+                            const int cnt = __popc(__ballot_sync(FULL_WARP, active && ((S >> (site & (WB - 1))) & (word)1)));
+                            if (lane == i) mine = cnt;
                         }
+                        if (q + lane < n_ens && mine != 0) atomicAdd(&ens[q + lane], (unsigned long long)(long long)mine);
                     }
-                    if (lane == 0) {
-                        atomicAdd(&ens_blk[0], s0);
-                        atomicAdd(&ens_blk[1], s1);
-                        atomicAdd(&ens_blk[2], s2);
-                        atomicAdd(&ens_blk[3], s3);
-                    }
-                    __syncthreads();
-                    for (int i = threadIdx.x; i < n_ens; i += blockDim.x) {
-                        const int v = ens_blk[i];
-                        if (v != 0)
-                            atomicAdd(&P.ens[(size_t)rec * n_ens + i], (unsigned long long)(long long)v);
-                        ens_blk[i] = 0;
-                    }
-                    __syncthreads();
                 }
+                ++rec;
             }
         }
     }
     if (active) {
-        P.state[r] = S;
+        P.state[r] = (uint64_t)S;
         P.hash[r] = H;
         P.clkM[r] = clkM;
         P.clkE[r] = clkE;
