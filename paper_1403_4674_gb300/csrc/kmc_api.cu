@@ -2361,9 +2361,9 @@ kmc_status kmc_ring_run(kmc_ring *g, int64_t n_schedules, int32_t schedule, int3
     P.ens = n_rec > 0 ? reinterpret_cast<unsigned long long *>(ens_dev) : nullptr;
     const int blocks = (g->n_traj + kmcring::RING_BLOCK - 1) / kmcring::RING_BLOCK;
     if (time_mode == KMC_TIME_EXPONENTIAL)
-        (P.NS <= 32 ? kmcring::ring_kernel<true, uint32_t> : kmcring::ring_kernel<true, uint64_t>)<<<blocks, kmcring::RING_BLOCK, 0, g->stream>>>(P);
+        (P.Ld <= 32 ? kmcring::ring_kernel<true, uint32_t> : kmcring::ring_kernel<true, uint64_t>)<<<blocks, kmcring::RING_BLOCK, 0, g->stream>>>(P);
     else
-        (P.NS <= 32 ? kmcring::ring_kernel<false, uint32_t> : kmcring::ring_kernel<false, uint64_t>)<<<blocks, kmcring::RING_BLOCK, 0, g->stream>>>(P);
+        (P.Ld <= 32 ? kmcring::ring_kernel<false, uint32_t> : kmcring::ring_kernel<false, uint64_t>)<<<blocks, kmcring::RING_BLOCK, 0, g->stream>>>(P);
     RING_CUDA_TRY(g, cudaGetLastError());
     ++g->launches;
     g->sched_done += n_schedules;

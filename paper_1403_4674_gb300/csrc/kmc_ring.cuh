@@ -47,46 +47,48 @@ struct RingParams {
     unsigned long long *ens; // [n_rec][4 + NS] or null (added to)
 };
 
-// A configuration is one word: 32 bits for rings of up to 32 spins (half the
-// instructions of every mask, shift and bit count), else 64.
+// A visit works on its domain alone: its spins and its two halo spins as a
+// window of 32 bits (domains of up to 32 spins; half the instructions of
+// every mask, shift and bit count), else of 64.
 __device__ __forceinline__ int ring_popc(uint32_t v) { return __popc(v); }
 __device__ __forceinline__ int ring_popc(uint64_t v) { return __popcll(v); }
 
-// Position of the rr-th (0-based) set bit of m; rr < popc(m).
-__device__ __forceinline__ int ring_select(uint64_t m, uint32_t rr) { return kmcdev::select_bit(m, rr); }
-__device__ __forceinline__ int ring_select(uint32_t w, uint32_t rr)
+// Position of the rr-th (0-based) set bit of m, a window of Ld bits; rr < popc(m).
+__device__ __forceinline__ int ring_select(uint64_t m, uint32_t rr, int) { return kmcdev::select_bit(m, rr); }
+__device__ __forceinline__ int ring_select(uint32_t w, uint32_t rr, int Ld)
 {
     int pos = 0;
-    uint32_t c = __popc(w & 0xFFFFu);
-    if (rr >= c) { rr -= c; w >>= 16; pos += 16; }
-    c = __popc(w & 0xFFu); if (rr >= c) { rr -= c; w >>= 8; pos += 8; }
+    uint32_t c;
+    if (Ld > 8) { // (the same in every lane)
+        c = __popc(w & 0xFFFFu);
+        if (rr >= c) { rr -= c; w >>= 16; pos += 16; }
+        c = __popc(w & 0xFFu);
+        if (rr >= c) { rr -= c; w >>= 8; pos += 8; }
+    }
     c = __popc(w & 0xFu);  if (rr >= c) { rr -= c; w >>= 4; pos += 4; }
     c = __popc(w & 0x3u);  if (rr >= c) { rr -= c; w >>= 2; pos += 2; }
     if (rr >= (w & 1u)) pos += 1;
     return pos;
 }
 
-// Neighbour words of a ring of NS bits: bit n of lw is spin n-1, of rw spin n+1.
-template <typename word> __device__ __forceinline__ word ring_left(word S, int NS, word NM)
+// The left neighbours of a ring of NS bits: bit n is spin n-1.
+__device__ __forceinline__ uint64_t ring_left(uint64_t S, int NS, uint64_t NM)
 {
     return ((S << 1) | (S >> (NS - 1))) & NM;
 }
-template <typename word> __device__ __forceinline__ word ring_right(word S, int NS, word NM)
-{
-    return (S >> 1) | ((S & (word)1) << (NS - 1));
-}
 
 // Inclusive cumulative rates C_c = sum_{c' <= c} n_c' A_c' in class order 0..5
-// of one domain (DM: its sites), and the words that hold the neighbours.
+// of a domain of Ld spins (s; DM: its sites), with the spins left of bit 0
+// and right of bit Ld - 1 (hl, hr), and the words that hold the neighbours.
 template <typename word>
-__device__ __forceinline__ void ring_cumulative(uint64_t (&C)[RING_CLASSES], word &lw, word &rw, word S, word DM, int NS,
-                                                word NM, const uint64_t (&A)[RING_CLASSES])
+__device__ __forceinline__ void ring_cumulative(uint64_t (&C)[RING_CLASSES], word &lw, word &rw, word s, word hl, word hr,
+                                                int Ld, word DM, const uint64_t (&A)[RING_CLASSES])
 {
-    lw = ring_left(S, NS, NM);
-    rw = ring_right(S, NS, NM);
+    lw = (word)(s << 1) | hl;
+    rw = (s >> 1) | (word)(hr << (Ld - 1));
     const word q0 = ~(lw | rw), q1 = lw ^ rw, q2 = lw & rw;
-    const word up = S & DM, dn = ~S & DM;
-    const word M[RING_CLASSES] = {dn & q0, dn & q1, dn & q2, up & q0, up & q1, up & q2};
+    const word dn = ~s & DM;
+    const word M[RING_CLASSES] = {dn & q0, dn & q1, dn & q2, s & q0, s & q1, s & q2};
     uint64_t acc = 0;
 #pragma unroll
     for (int c = 0; c < RING_CLASSES; ++c) {
@@ -120,16 +122,20 @@ __device__ __forceinline__ RingDraw ring_draw(uint32_t j, uint32_t d, uint64_t n
 // entry and, with `more`, that of the next visit's (domain d2, phase np2) on
 // return; a variate enters the clock with its step.
 template <bool EXPO, typename word>
-__device__ __forceinline__ void ring_visit(word &S, uint64_t &H, int64_t &flips, uint64_t &clkM, int64_t &clkE, int d,
-                                           int Ld, int k, int NS, word NM, word DM0, uint64_t np, uint2 key,
+__device__ __forceinline__ void ring_visit(uint64_t &S, uint64_t &H, int64_t &flips, uint64_t &clkM, int64_t &clkE, int d,
+                                           int Ld, int k, int NS, word DM, uint64_t np, uint2 key,
                                            const uint64_t (&A)[RING_CLASSES], const float (&invA)[RING_CLASSES],
                                            unsigned lanes, RingDraw &cur, bool more, int d2, uint64_t np2)
 {
     const int first = d * Ld;
-    const word DM = DM0 << first;
+    const word s0 = (word)(S >> first) & DM;
+    word s = s0;
+    // the halo spins; the only domain of a ring is its own neighbour
+    const bool own = Ld == NS;
+    word hl = (word)(S >> (first == 0 ? NS - 1 : first - 1)) & 1, hr = (word)(S >> (first + Ld == NS ? 0 : first + Ld)) & 1;
     uint64_t C[RING_CLASSES];
     word lw, rw;
-    ring_cumulative(C, lw, rw, S, DM, NS, NM, A);
+    ring_cumulative(C, lw, rw, s, hl, hr, Ld, DM, A);
     for (int j = 0; j < k; ++j) {
         const uint64_t tgt = cur.tgt;
         const bool ev = tgt < C[RING_CLASSES - 1]; // else a null step
@@ -156,14 +162,19 @@ __device__ __forceinline__ void ring_visit(word &S, uint64_t &H, int64_t &flips,
             jj = (x - (uint64_t)jj * Ac >= Ac) ? jj + 1u : jj;
             const int q = (c >= 3) ? c - 3 : c;
             const word qm = (q == 0) ? ~(lw | rw) : ((q == 1) ? (lw ^ rw) : (lw & rw));
-            const int site = ring_select(((c >= 3) ? S : ~S) & qm & DM, jj) & (int)(8 * sizeof(word) - 1);
-            S ^= ev ? (word)1 << site : (word)0;
+            const int site = ring_select((word)(((c >= 3) ? s : ~s) & qm & DM), jj, Ld) & (int)(8 * sizeof(word) - 1);
+            s ^= ev ? (word)1 << site : (word)0;
+            if (own) {
+                hl = s >> (Ld - 1);
+                hr = s & 1;
+            }
             flips += ev ? 1 : 0;
-            const uint64_t h = (H ^ ((np << 32) | ((uint64_t)j << 16) | (uint64_t)(site - first))) * HASH_PRIME;
+            const uint64_t h = (H ^ ((np << 32) | ((uint64_t)j << 16) | (uint64_t)site)) * HASH_PRIME;
             H = ev ? h : H;
-            ring_cumulative(C, lw, rw, S, DM, NS, NM, A);
+            ring_cumulative(C, lw, rw, s, hl, hr, Ld, DM, A);
         }
     }
+    S ^= (uint64_t)(s ^ s0) << first;
 }
 
 // Uniform random order of the n_dom domains of schedule n (the paper's
@@ -222,8 +233,8 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
     const int NS = P.NS, Ld = P.Ld, ND = NS / Ld, k = P.k;
     const int n_ens = RING_ENS_FIXED + NS;
     constexpr int WB = 8 * (int)sizeof(word);
-    const word NM = (NS == WB) ? ~(word)0 : (((word)1 << (NS & (WB - 1))) - (word)1);
-    const word DM0 = (Ld == WB) ? ~(word)0 : (((word)1 << (Ld & (WB - 1))) - (word)1);
+    const uint64_t NM = (NS == 64) ? ~0ull : ((1ull << NS) - 1ull);
+    const word DM = (Ld == WB) ? ~(word)0 : (((word)1 << (Ld & (WB - 1))) - (word)1);
 
     uint64_t A[RING_CLASSES];
     float invA[RING_CLASSES]; // 1/A_c from below: A_c rounded up, reciprocal rounded down
@@ -235,8 +246,7 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
     const uint64_t seed = P.seed[r];
     const uint2 key = make_uint2((uint32_t)seed, (uint32_t)(seed >> 32));
     const double hr = P.h[r];
-    word S = (word)P.state[r];
-    uint64_t H = P.hash[r], clkM = P.clkM[r];
+    uint64_t S = P.state[r], H = P.hash[r], clkM = P.clkM[r];
     int64_t clkE = P.clkE[r], flips = P.flips[r], steps = P.steps[r];
 
     const bool perm = P.schedule == kmcdev::SCHED_RANDOM_PERM;
@@ -258,7 +268,7 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
                     const int d = order.at(ND, p);
                     if (p == 0) cur = ring_draw(0u, (uint32_t)d, np, key);
                     const bool more = p + 1 < nph;
-                    ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, NM, DM0, np, key, A, invA, lanes, cur, more,
+                    ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, DM, np, key, A, invA, lanes, cur, more,
                                      more ? order.at(ND, p + 1) : 0, np + 1);
                     steps += k;
                 } else {
@@ -268,7 +278,7 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
                     for (int d = colour(p); d < ND; d += ncol) {
                         const bool stay = d + ncol < ND, turn = p + 1 == nph;
                         const bool more = stay || !turn || nl + 1 < P.n_sched;
-                        ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, NM, DM0, np, key, A, invA, lanes, cur, more,
+                        ring_visit<EXPO>(S, H, flips, clkM, clkE, d, Ld, k, NS, DM, np, key, A, invA, lanes, cur, more,
                                          stay ? d + ncol : turn ? 0 : colour(p + 1),
                                          stay ? np : turn ? (n + 1) * RING_PHASE_SLOTS : np + 1);
                         steps += k;
@@ -278,9 +288,9 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
             if (P.obs_every > 0 && --until == 0) {
                 until = P.obs_every;
                 // bonds = sum_n s_n s_{n+1}: NS - 2 * (number of unlike neighbour pairs)
-                const int unlike = ring_popc((S ^ ring_left(S, NS, NM)) & NM);
+                const int unlike = __popcll((S ^ ring_left(S, NS, NM)) & NM);
                 const int bonds = NS - 2 * unlike;
-                const int mag = 2 * ring_popc(S & NM) - NS;
+                const int mag = 2 * __popcll(S & NM) - NS;
                 if (active) {
                     const size_t o = (size_t)rec * P.n_traj + r;
                     if (P.obs) {
@@ -294,7 +304,7 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
                         v.w = ring_clock(EXPO, clkM, clkE, steps, NS, P.nu);
                         reinterpret_cast<double4_32a *>(P.obs)[o] = v;
                     }
-                    if (P.obs_state) P.obs_state[o] = (uint64_t)S;
+                    if (P.obs_state) P.obs_state[o] = S;
                 }
                 if (P.ens != nullptr) {
                     // ensemble sums over the warp, lane i adding quantity i, i + 32, ...
@@ -309,7 +319,7 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
                     for (int q = 0; q < n_ens; q += 32) {
                         for (int i = (q == 0 ? RING_ENS_FIXED : 0); i < 32 && q + i < n_ens; ++i) {
                             const int site = q + i - RING_ENS_FIXED;
-                            const int cnt = __popc(__ballot_sync(FULL_WARP, active && ((S >> (site & (WB - 1))) & (word)1)));
+                            const int cnt = __popc(__ballot_sync(FULL_WARP, active && ((S >> site) & 1ull)));
                             if (lane == i) mine = cnt;
                         }
                         if (q + lane < n_ens && mine != 0) atomicAdd(&ens[q + lane], (unsigned long long)(long long)mine);
@@ -320,7 +330,7 @@ __global__ void __launch_bounds__(RING_BLOCK, 8) ring_kernel(const RingParams P)
         }
     }
     if (active) {
-        P.state[r] = (uint64_t)S;
+        P.state[r] = S;
         P.hash[r] = H;
         P.clkM[r] = clkM;
         P.clkE[r] = clkE;
