@@ -267,7 +267,7 @@ RunKernel run_kernel_for(int LD, bool expo, bool grad, bool cluster)
 
 LayoutParams layout_params(kmc_ctx *c)
 {
-    LayoutParams P;
+    LayoutParams P = {};
     P.n_rep = c->n_rep;
     P.n_dom = c->n_dom;
     P.rep_L = c->d_L;
@@ -954,18 +954,19 @@ kmc_status default_warp_plan(kmc_ctx *c)
 }
 
 // Endpoint observables of the packed state into acc[n_rep][OBS_WORDS]
-// (bond sum, magnetisation, summed domain clocks, summed scores).
+// (bond sum, magnetisation, summed domain clocks, summed scores), which the
+// pack kernel has cleared.
 kmc_status launch_observe(kmc_ctx *c, cudaStream_t s, int time_mode, unsigned long long *acc)
 {
-    CUDA_TRY(c, cudaMemsetAsync(acc, 0, (size_t)c->n_rep * OBS_WORDS * 8, s));
     RunParams P = run_params(c);
     const bool expo = time_mode == KMC_TIME_EXPONENTIAL;
     P.horizon = time_mode == KMC_TIME_HORIZON;
     P.dtau = c->dtau;
-    const int blocks = grid_for(c->n_dom, 8 * (c->LD == 8 ? observe_domains<8>() : observe_domains<16>()));
+    const int dpw = c->LD == 8 ? 32 : std::max(1, std::min(8, c->n_dom / (16 * std::max(1, c->sm_count))));
+    const int blocks = grid_for(c->n_dom, 8 * dpw);
 #define KMC_OBS(LDV)                                                                                         \
-    if (expo) observe_kernel<LDV, true><<<blocks, 256, 0, s>>>(P, c->d_dom_rep, c->n_dom, c->visits_done, acc); \
-    else observe_kernel<LDV, false><<<blocks, 256, 0, s>>>(P, c->d_dom_rep, c->n_dom, c->visits_done, acc);
+    if (expo) observe_kernel<LDV, true><<<blocks, 256, 0, s>>>(P, c->d_dom_rep, c->n_dom, c->visits_done, acc, dpw); \
+    else observe_kernel<LDV, false><<<blocks, 256, 0, s>>>(P, c->d_dom_rep, c->n_dom, c->visits_done, acc, dpw);
     switch (c->LD) {
     case 8: KMC_OBS(8) break;
     case 16: KMC_OBS(16) break;
@@ -1080,12 +1081,14 @@ kmc_status upload_horizon(kmc_ctx *c)
 
 kmc_status upload_rates(kmc_ctx *c)
 {
-    std::vector<uint64_t> A16((size_t)c->n_rep * 16, 0);
+    std::vector<uint64_t> A16((size_t)c->n_rep * RATE_WORDS, 0);
     std::vector<int64_t> gfix((size_t)c->n_rep * GFIX_WORDS, 0);
     std::vector<double> g32((size_t)c->n_rep * 32, 0.0);
     for (int r = 0; r < c->n_rep; ++r) {
         for (int q = 0; q < 10; ++q) {
-            A16[(size_t)r * 16 + q] = c->A[(size_t)r * 10 + q];
+            const uint64_t Aq = c->A[(size_t)r * 10 + q];
+            A16[(size_t)r * RATE_WORDS + q] = Aq;
+            A16[(size_t)r * RATE_WORDS + RATE_RECIP + q] = Aq ? ~0ull / Aq : 0ull;
             g32[(size_t)r * 32 + q] = c->a[(size_t)r * 10 + q];
             g32[(size_t)r * 32 + 10 + q] = c->gb[(size_t)r * 10 + q];
             g32[(size_t)r * 32 + 20 + q] = c->gh[(size_t)r * 10 + q];
@@ -1104,9 +1107,15 @@ kmc_status upload_rates(kmc_ctx *c)
     return upload_horizon(c); // the table depends on nu
 }
 
-kmc_status launch_pack(kmc_ctx *c, cudaStream_t s)
+// Pack; base (n_rep record sums) and acc (n_acc words) are cleared with it.
+kmc_status launch_pack(kmc_ctx *c, cudaStream_t s, unsigned long long *base = nullptr, unsigned long long *acc = nullptr,
+                       size_t n_acc = 0)
 {
     LayoutParams P = layout_params(c);
+    P.zero[0] = base;
+    P.n_zero[0] = base ? (uint64_t)c->n_rep * OBS_WORDS : 0;
+    P.zero[1] = acc;
+    P.n_zero[1] = n_acc;
     const int blocks = grid_for(c->n_dom, c->LD == 8 ? 256 : 8); // a thread or a warp per domain
     switch (c->LD) {
     case 8: pack_kernel<8><<<blocks, 256, 0, s>>>(P); break;
@@ -1119,15 +1128,16 @@ kmc_status launch_pack(kmc_ctx *c, cudaStream_t s)
     return KMC_OK;
 }
 
-kmc_status launch_unpack(kmc_ctx *c, cudaStream_t s)
+kmc_status launch_unpack(kmc_ctx *c, cudaStream_t s, const RecordParams &R)
 {
     LayoutParams P = layout_params(c);
-    const int blocks = grid_for(c->n_dom, c->LD == 8 ? 256 : 8);
+    const int unpack = grid_for(c->n_dom, c->LD == 8 ? 256 : 8);
+    const int blocks = unpack + (R.n_obs > 0 ? grid_for(c->n_rep, 8) : 0); // a warp per replica's records
     switch (c->LD) {
-    case 8: unpack_kernel<8><<<blocks, 256, 0, s>>>(P); break;
-    case 16: unpack_kernel<16><<<blocks, 256, 0, s>>>(P); break;
-    case 32: unpack_kernel<32><<<blocks, 256, 0, s>>>(P); break;
-    default: unpack_kernel<64><<<blocks, 256, 0, s>>>(P); break;
+    case 8: unpack_kernel<8><<<blocks, 256, 0, s>>>(P, R, unpack); break;
+    case 16: unpack_kernel<16><<<blocks, 256, 0, s>>>(P, R, unpack); break;
+    case 32: unpack_kernel<32><<<blocks, 256, 0, s>>>(P, R, unpack); break;
+    default: unpack_kernel<64><<<blocks, 256, 0, s>>>(P, R, unpack); break;
     }
     ++c->launches;
     CUDA_TRY(c, cudaGetLastError());
@@ -1349,7 +1359,7 @@ kmc_status kmc_create_lattice(kmc_ctx **out, int32_t n_replicas, const int32_t *
     ALLOC(c->d_site_off, n_replicas);
     ALLOC(c->d_blk_off, n_replicas + 1);
     ALLOC(c->d_seed, n_replicas);
-    ALLOC(c->d_A, (size_t)n_replicas * 16);
+    ALLOC(c->d_A, (size_t)n_replicas * RATE_WORDS);
     ALLOC(c->d_gfix, (size_t)n_replicas * GFIX_WORDS);
     ALLOC(c->d_grad, (size_t)n_replicas * 32);
     ALLOC(c->d_h, n_replicas);
@@ -1401,8 +1411,7 @@ kmc_status kmc_reset(kmc_ctx *c, int32_t init, void *stream)
         any = false;
         for (int32_t m : c->init_r) any = any || m != KMC_INIT_KEEP;
     }
-    if (any && (s = launch_init(c, init, c->stream)) != KMC_OK) return s;
-    if ((s = launch_reset_counters(c, c->stream)) != KMC_OK) return s;
+    if ((s = any ? launch_init(c, init, c->stream) : launch_reset_counters(c, c->stream)) != KMC_OK) return s;
     c->sched_done = 0;
     c->visits_done = 0;
     c->clocks_exponential = true;
@@ -1693,11 +1702,11 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
             if ((st = dev_alloc(c, &c->d_obs_acc, words)) != KMC_OK) return st;
             c->obs_acc_words = words;
         }
-        CUDA_TRY(c, cudaMemsetAsync(c->d_obs_acc, 0, words * 8, s));
     }
-    if ((st = launch_pack(c, s)) != KMC_OK) return st;
     // records are built from the state before the launch plus per-visit changes
     unsigned long long *base = reinterpret_cast<unsigned long long *>(c->d_tmp);
+    if ((st = n_obs > 0 ? launch_pack(c, s, base, c->d_obs_acc, (size_t)n_obs * c->n_rep * OBS_WORDS) : launch_pack(c, s)) != KMC_OK)
+        return st;
     if (n_obs > 0 && (st = launch_observe(c, s, time_mode, base)) != KMC_OK) return st;
     RunParams P = run_params(c);
     P.schedule = schedule;
@@ -1750,13 +1759,8 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
         CUDA_TRY(c, cudaEventRecord(ev1, s));
         c->prof_events.emplace_back(ev0, ev1);
     }
-    if (want_obs && n_obs > 0) {
-        finalize_obs_kernel<<<grid_for(c->n_rep, 4), 128, 0, s>>>(base, c->d_obs_acc, n_obs, c->n_rep, c->d_L, c->d_Dx,
-                                                                    c->J, c->d_h, obs_dev, c->grad ? 6 : 4);
-        ++c->launches;
-        CUDA_TRY(c, cudaGetLastError());
-    }
-    if ((st = launch_unpack(c, s)) != KMC_OK) return st;
+    const RecordParams R = {base, c->d_obs_acc, n_obs, c->n_rep, c->grad ? 6 : 4, c->d_L, c->d_Dx, c->J, c->d_h, obs_dev};
+    if ((st = launch_unpack(c, s, R)) != KMC_OK) return st;
     c->sched_done += n_schedules;
     c->visits_done += n_schedules * (schedule == KMC_SCHEDULE_PALINDROME ? 2 : 1);
     c->last_time_mode = time_mode;
@@ -1776,8 +1780,8 @@ kmc_status kmc_observables(kmc_ctx *c, double *E_per_site, double *m, double *t,
     if (refuse_capture(c, "kmc_observables") != KMC_OK) return KMC_EINVAL;
     kmc_status st;
     cudaStream_t s = c->stream;
-    if ((st = launch_pack(c, s)) != KMC_OK) return st;
     unsigned long long *acc = reinterpret_cast<unsigned long long *>(c->d_tmp);
+    if ((st = launch_pack(c, s, acc)) != KMC_OK) return st;
     const size_t words = (size_t)c->n_rep * OBS_WORDS;
     if ((st = launch_observe(c, s, c->last_time_mode, acc)) != KMC_OK) return st;
     std::vector<unsigned long long> h_acc(words);
@@ -1938,7 +1942,7 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
         c.d_site_off = cv.take<uint64_t>(1);
         c.d_blk_off = cv.take<uint64_t>(2);
         c.d_seed = cv.take<uint64_t>(1);
-        c.d_A = cv.take<uint64_t>(16);
+        c.d_A = cv.take<uint64_t>(RATE_WORDS);
         c.d_gfix = cv.take<int64_t>(GFIX_WORDS);
         c.d_grad = cv.take<double>(32);
         c.d_h = cv.take<double>(1);
@@ -1974,7 +1978,7 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
     // inputs of this call; the array keeps the previous call's contents, so
     // everything the kernels read is written (or cleared) here first
     cudaStream_t s = c.stream;
-    std::vector<uint64_t> A16(16, 0);
+    std::vector<uint64_t> A16(RATE_WORDS, 0); // (the cluster kernel reads no reciprocals)
     std::vector<int64_t> gfix(GFIX_WORDS, 0);
     (void)build_gfix(c.a.data(), c.gb.data(), c.gh.data(), c.log2nd, gfix.data()); // staged, unused: no scores here
     std::vector<double> g32(32, 0.0);
@@ -1987,7 +1991,7 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
     struct Up { void *dst; const void *src; size_t bytes; } ups[] = {
         {c.d_L, c.L.data(), 4}, {c.d_Dx, c.Dx.data(), 4}, {c.d_k, c.kr.data(), 4}, {c.d_dom_off, c.dom_off.data(), 8},
         {c.d_site_off, c.site_off.data(), 8}, {c.d_blk_off, c.blk_off.data(), 16}, {c.d_seed, c.seed.data(), 8},
-        {c.d_A, A16.data(), 128}, {c.d_gfix, gfix.data(), GFIX_WORDS * 8}, {c.d_grad, g32.data(), 256}, {c.d_h, c.h.data(), 8},
+        {c.d_A, A16.data(), RATE_WORDS * 8}, {c.d_gfix, gfix.data(), GFIX_WORDS * 8}, {c.d_grad, g32.data(), 256}, {c.d_h, c.h.data(), 8},
         {c.d_dom_rep, c.dom_rep.data(), (size_t)c.n_dom * 4}, {c.d_plan, flat.data(), flat.size() * 4},
     };
     for (const Up &u : ups) {
@@ -1996,13 +2000,15 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
         if (ce != cudaSuccess) return bad(KMC_ECUDA, std::string("cudaMemcpyAsync: ") + cudaGetErrorString(ce));
     }
     ce = cudaMemsetAsync(c.d_err, 0, sizeof(int), s);
-    if (ce == cudaSuccess && n_obs > 0) ce = cudaMemsetAsync(c.d_obs_acc, 0, (size_t)n_obs * c.n_rep * OBS_WORDS * 8, s);
     if (ce != cudaSuccess) return bad(KMC_ECUDA, std::string("cudaMemsetAsync: ") + cudaGetErrorString(ce));
     c.plan = std::move(pl);
 
     if ((st = launch_reset_counters(&c, s)) != KMC_OK) return bad(st, c.err);
     if (n_schedules > 0) {
-        if ((st = launch_pack(&c, s)) != KMC_OK) return bad(st, c.err);
+        if ((st = n_obs > 0 ? launch_pack(&c, s, reinterpret_cast<unsigned long long *>(c.d_tmp), c.d_obs_acc,
+                                          (size_t)n_obs * OBS_WORDS)
+                            : launch_pack(&c, s)) != KMC_OK)
+            return bad(st, c.err);
         if (n_obs > 0 &&
             (st = launch_observe(&c, s, time_mode, reinterpret_cast<unsigned long long *>(c.d_tmp))) != KMC_OK)
             return bad(st, c.err);
@@ -2029,13 +2035,9 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
         cfg.numAttrs = 1;
         ce = cudaLaunchKernelEx(&cfg, kern, P);
         if (ce != cudaSuccess) return bad(KMC_ECUDA, std::string("cudaLaunchKernelEx: ") + cudaGetErrorString(ce));
-        if (n_obs > 0) {
-            finalize_obs_kernel<<<1, 32, 0, s>>>(reinterpret_cast<unsigned long long *>(c.d_tmp), c.d_obs_acc, n_obs, 1,
-                                                 c.d_L, c.d_Dx, J, c.d_h, obs_dev, 4);
-            ce = cudaGetLastError();
-            if (ce != cudaSuccess) return bad(KMC_ECUDA, std::string("finalize: ") + cudaGetErrorString(ce));
-        }
-        if ((st = launch_unpack(&c, s)) != KMC_OK) return bad(st, c.err);
+        const RecordParams R = {reinterpret_cast<unsigned long long *>(c.d_tmp), c.d_obs_acc, n_obs, 1, 4, c.d_L, c.d_Dx, J,
+                                c.d_h, obs_dev};
+        if ((st = launch_unpack(&c, s, R)) != KMC_OK) return bad(st, c.err);
     }
     // synchronising: the device error word lives in the shared array
     st = sync_ctx(&c);

@@ -132,40 +132,67 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
     auto row = [&](uint8_t *b, int y) -> row_t & { return reinterpret_cast<row_t *>(b + Q::ROWS)[y]; };
 
     // ---- stage the domains: rows, counts with an all-down halo ----
+    // (every lane of a group asks for its share of the domain's words at once)
     for (int s = 0; s < ns; ++s) {
         uint8_t *b = dom(s);
-        const uint32_t g = P.slot_g[((size_t)wg * ns + s) * DPW + grp];
+        const size_t slot = ((size_t)wg * ns + s) * DPW + grp;
+        const uint32_t g = P.slot_g[slot];
         const bool has = g != 0xFFFFFFFFu;
+        const uint32_t nb = P.slot_nb[slot * 4 + (gl & 3)];
         const uint32_t r = has ? P.dom_rep[g] : 0u;
-        if (has) {
-            const uint8_t *tile = P.tiles + (size_t)g * (LD * LD / 8);
-            for (int y = y0; y < y0 + RPL; ++y)
-                row(b, y) = (LD == 64) ? (row_t) reinterpret_cast<const uint64_t *>(tile)[y]
-                            : (LD == 32) ? (row_t) reinterpret_cast<const uint32_t *>(tile)[y]
-                                         : (row_t) reinterpret_cast<const uint16_t *>(tile)[y];
-        } else {
-            for (int y = y0; y < y0 + RPL; ++y) row(b, y) = 0;
+        const uint8_t *tile = P.tiles + (size_t)(has ? g : 0u) * (LD * LD / 8);
+        row_t S[RPL];
+#pragma unroll
+        for (int i = 0; i < RPL; ++i) {
+            S[i] = (LD == 64) ? (row_t) reinterpret_cast<const uint64_t *>(tile)[y0 + i]
+                   : (LD == 32) ? (row_t) reinterpret_cast<const uint32_t *>(tile)[y0 + i]
+                                : (row_t) reinterpret_cast<const uint16_t *>(tile)[y0 + i];
+            if (!has) S[i] = 0;
         }
-        if (gl == 0) row(b, -1) = row(b, LD) = 0;
+        const uint64_t *edges = P.edges + (size_t)(has ? g : 0u) * EDGE_WORDS, *ctr = P.dctr + (size_t)(has ? g : 0u) * DCTR_WORDS;
+        const uint64_t edge = edges[gl & 7];
+        const int cw = (gl == 0) ? DCTR_HASH : (gl == 1) ? DCTR_FLIPS : (gl == 2) ? DCTR_STEPS : (gl == 3) ? DCTR_CLKM : DCTR_CLKE;
+        const uint64_t count = ctr[cw];
+        const uint64_t seed = P.rep_seed[r];
+        const uint32_t k = (uint32_t)P.rep_k[r], doff = P.rep_dom_off[r];
         for (int c = gl; c < 10; c += G) {
-            const uint64_t A = P.rep_A[(size_t)r * 16 + c];
-            u64(b, Q::AT + 8 * c) = A;
-            u64(b, Q::MR + 8 * c) = A ? ~0ull / A : 0ull;
+            u64(b, Q::AT + 8 * c) = P.rep_A[(size_t)r * RATE_WORDS + c];
+            u64(b, Q::MR + 8 * c) = P.rep_A[(size_t)r * RATE_WORDS + RATE_RECIP + c];
         }
+#pragma unroll
+        for (int i = 0; i < RPL; ++i) row(b, y0 + i) = S[i];
+        if (gl == 0) row(b, -1) = row(b, LD) = 0;
+        if (gl < 8) u64(b, Q::EDGE + 8 * gl) = has ? edge : 0ull;
+        if (gl < 5) u64(b, Q::CTR + 8 * gl) = count;
         u64(b, Q::CLK + 16 * gl) = 1ull << 63;
         u64(b, Q::CLK + 16 * gl + 8) = 0;
+        if (gl < 4) {
+            // the neighbour's facing edge (N: its S row, S: its N row, W: its E
+            // column, E: its W column); bit 0 of the address: in this CTA
+            const int facing = gl ^ 1;
+            uint64_t a = 0;
+            if (has)
+                a = (nb & 0x80000000u)
+                        ? (uint64_t)(domains + (size_t)(nb & 0x7FFFFFFFu) * Q::BYTES + Q::EDGE + 16 * facing) | 1ull
+                        : (uint64_t)(P.edges + (size_t)nb * EDGE_WORDS + 2 * facing);
+            u64(b, Q::NBP + 8 * gl) = a;
+        }
         __syncwarp();
-        uint64_t lo = 0, hi = 0;
-        for (int y = y0; y < y0 + RPL; ++y) {
-            const row_t S = row(b, y), U = row(b, y - 1), D = row(b, y + 1);
-            const row_t Wn = (row_t)(S << 1) & FULL, En = (row_t)(S >> 1);
+        uint64_t lo = 0, hi = 0, cW = 0, cE = 0;
+#pragma unroll
+        for (int i = 0; i < RPL; ++i) {
+            const int y = y0 + i;
+            const row_t U = row(b, y - 1), D = row(b, y + 1);
+            const row_t Wn = (row_t)(S[i] << 1) & FULL, En = (row_t)(S[i] >> 1);
             const row_t s1 = U ^ D, c1 = U & D, s2 = Wn ^ En, c2 = Wn & En, t0 = s1 & s2;
             const row_t b0 = s1 ^ s2, b1 = c1 ^ c2 ^ t0, b2 = (c1 & c2) | (c1 & t0) | (c2 & t0);
             for (int q = 0; q < 5; ++q) {
                 const row_t m = (row_t)(((q & 4) ? b2 : ~b2) & ((q & 2) ? b1 : ~b1) & ((q & 1) ? b0 : ~b0)) & FULL;
-                lo += (uint64_t)popc_row((row_t)(m & ~S)) << grp_shift(q);
-                hi += (uint64_t)popc_row((row_t)(m & S)) << grp_shift(5 + q);
+                lo += (uint64_t)popc_row((row_t)(m & ~S[i])) << grp_shift(q);
+                hi += (uint64_t)popc_row((row_t)(m & S[i])) << grp_shift(5 + q);
             }
+            cW |= (uint64_t)(S[i] & 1u) << y;
+            cE |= (uint64_t)((S[i] >> (LD - 1)) & 1u) << y;
         }
         uint64_t ilo = lo, ihi = hi;
 #pragma unroll
@@ -173,6 +200,8 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
             const uint64_t a = __shfl_up_sync(FULL_WARP, ilo, off, G), c = __shfl_up_sync(FULL_WARP, ihi, off, G);
             ilo += (gl >= off) ? a : 0ull;
             ihi += (gl >= off) ? c : 0ull;
+            cW |= __shfl_xor_sync(FULL_WARP, cW, off);
+            cE |= __shfl_xor_sync(FULL_WARP, cE, off);
         }
         u64(b, Q::E + 16 * gl) = ilo - lo;
         u64(b, Q::E + 16 * gl + 8) = ihi - hi;
@@ -181,43 +210,13 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
             u64(b, Q::T + 8) = ihi;
         }
         if (gl == 0) {
-            uint64_t cw = 0, ce = 0;
-            for (int y = 0; y < LD; ++y) {
-                cw |= (uint64_t)(row(b, y) & 1u) << y;
-                ce |= (uint64_t)((row(b, y) >> (LD - 1)) & 1u) << y;
-            }
-            u64(b, Q::COLS) = cw;
-            u64(b, Q::COLS + 8) = ce;
+            u64(b, Q::COLS) = cW;
+            u64(b, Q::COLS + 8) = cE;
             u64(b, Q::HALO) = u64(b, Q::HALO + 8) = 0;
-            u64(b, Q::SEED) = has ? P.rep_seed[r] : 0ull;
-            u32(b, Q::META) = g;
-            u32(b, Q::META + 4) = has ? g - P.rep_dom_off[r] : 0u;
-            u32(b, Q::META + 8) = has ? (uint32_t)P.rep_k[r] : 0u;
-            u32(b, Q::META + 12) = r;
+            u64(b, Q::SEED) = seed;
+            *reinterpret_cast<uint4 *>(b + Q::META) = make_uint4(g, has ? g - doff : 0u, has ? k : 0u, r);
             u64(b, Q::OBS) = (uint64_t)NO_RECORD;
             u64(b, Q::OBS + 8) = 0;
-            if (has) {
-                const uint64_t *ctr = P.dctr + (size_t)g * DCTR_WORDS;
-                u64(b, Q::CTR) = ctr[DCTR_HASH];
-                u64(b, Q::CTR + 8) = ctr[DCTR_FLIPS];
-                u64(b, Q::CTR + 16) = ctr[DCTR_STEPS];
-                u64(b, Q::CTR + 24) = ctr[DCTR_CLKM];
-                u64(b, Q::CTR + 32) = ctr[DCTR_CLKE];
-                for (int q = 0; q < 8; ++q) u64(b, Q::EDGE + 8 * q) = P.edges[(size_t)g * EDGE_WORDS + q];
-            }
-        }
-        if (gl < 4) {
-            // the neighbour's facing edge (N: its S row, S: its N row, W: its E
-            // column, E: its W column); bit 0 of the address: in this CTA
-            const int facing = gl ^ 1;
-            uint64_t a = 0;
-            if (has) {
-                const uint32_t nb = P.slot_nb[(((size_t)wg * ns + s) * DPW + grp) * 4 + gl];
-                a = (nb & 0x80000000u)
-                        ? (uint64_t)(domains + (size_t)(nb & 0x7FFFFFFFu) * Q::BYTES + Q::EDGE + 16 * facing) | 1ull
-                        : (uint64_t)(P.edges + (size_t)nb * EDGE_WORDS + 2 * facing);
-            }
-            u64(b, Q::NBP + 8 * gl) = a;
         }
         __syncwarp();
     }

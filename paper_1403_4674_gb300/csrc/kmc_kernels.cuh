@@ -48,6 +48,7 @@ constexpr int HORIZON_MAX_STEPS = 1024; // table length limit of the fixed-time 
 constexpr int ERR_TIMEOUT = 1, ERR_SPIN = 2, ERR_INTERNAL = 3;
 constexpr int SCHED_PALINDROME = 0, SCHED_FIXED = 1, SCHED_RANDOM_PERM = 2;
 constexpr int INIT_KEEP = 2, INIT_PER_REPLICA = 3;
+constexpr int RATE_WORDS = 32, RATE_RECIP = 16; // words per replica of the rate table
 constexpr int OBS_WORDS = 5; // bonds, mag, clock sum, score beta sum, score h sum
 
 // Replica table staged in shared memory (bytes):
@@ -97,7 +98,7 @@ struct RunParams {
     const int32_t *rep_k;    // steps per domain visit
     const uint32_t *rep_dom_off;
     const uint64_t *rep_seed;
-    const uint64_t *rep_A;   // [n_rep][16]
+    const uint64_t *rep_A;   // [n_rep][RATE_WORDS]: A_c[16], floor((2^64 - 1) / A_c)[16] (0 where A_c is)
     const int64_t *rep_gfix; // [n_rep][GFIX_WORDS]
     const double *rep_grad;  // [n_rep][32]
     // plan: per CTA slot ranges (colour-sorted), replica tables, neighbours
@@ -887,7 +888,7 @@ __global__ void __maxnreg__((run_kernel_regs<LD, GRAD>())) run_kernel(const RunP
         const uint32_t r = P.rt_rep[rt0 + i];
         uint8_t *t = tables + (size_t)i * RT_BYTES;
         if (lane < 16) {
-            reinterpret_cast<uint64_t *>(t)[lane] = P.rep_A[(size_t)r * 16 + lane];
+            reinterpret_cast<uint64_t *>(t)[lane] = P.rep_A[(size_t)r * RATE_WORDS + lane];
             reinterpret_cast<int64_t *>(t + RT_GB)[lane] = (lane < 10) ? P.rep_gfix[(size_t)r * GFIX_WORDS + lane] : 0;
         }
         if (lane < 10) {
@@ -1284,12 +1285,40 @@ struct LayoutParams {
     uint64_t *edges;
     uint64_t *dctr;
     int *err;
+    // words that the pack kernel clears for the kernels after it (the sums of
+    // the launch's records)
+    unsigned long long *zero[2];
+    uint64_t n_zero[2];
 };
 
+// What the kernels need to form records (finalize_records).
+struct RecordParams {
+    const unsigned long long *base, *acc;
+    int64_t n_obs; // 0: none
+    int n_rep, stride;
+    const int32_t *rep_L, *rep_Dx;
+    double J;
+    const double *rep_h;
+    double *out;
+};
+
+// Zero counters of a domain: hash basis, flips 0, clock 1.0 (m = 2^63, e = 0), scores 0.
+__device__ __forceinline__ void reset_counters(uint64_t *dctr, int n_dom)
+{
+    // (word i of all domains' counters: whole lines)
+    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < (uint64_t)n_dom * DCTR_WORDS;
+         i += (uint64_t)gridDim.x * blockDim.x) {
+        const int w = (int)(i % DCTR_WORDS);
+        dctr[i] = w == DCTR_HASH ? HASH_BASIS : w == DCTR_CLKM ? 1ull << 63 : 0ull;
+    }
+}
+
 // iid +-1 from Philox (block b of 128 sites: counter {b_lo, b_hi, 0, TAG_INIT<<24}) or all up;
-// init = INIT_PER_REPLICA takes each replica's mode from rep_init (INIT_KEEP leaves it alone).
+// init = INIT_PER_REPLICA takes each replica's mode from rep_init (INIT_KEEP leaves it alone);
+// the domains' counters are reset with it.
 __global__ void init_spins_kernel(const LayoutParams P, int init)
 {
+    reset_counters(P.dctr, P.n_dom);
     // Replicas follow one another without gaps and hold whole blocks of 128
     // sites, so block t starts at byte 128 t.  A warp draws 32 blocks, a lane
     // each, and writes their 4 KB as whole 512-byte lines: 16 bytes per lane
@@ -1368,6 +1397,9 @@ __global__ void pack_kernel(const LayoutParams P)
     using G = Geo<LD>;
     using row_t = typename G::row_t;
     using mem_t = typename G::mem_t;
+    for (int z = 0; z < 2; ++z)
+        for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < P.n_zero[z]; i += (uint64_t)gridDim.x * blockDim.x)
+            P.zero[z][i] = 0;
     if (LD == 8) {
         bool ok = true;
         for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.n_dom; g += gridDim.x * blockDim.x) {
@@ -1442,166 +1474,20 @@ __global__ void pack_kernel(const LayoutParams P)
     }
 }
 
-// bit tiles -> int8 spins; as pack_kernel: one thread per 8x8 domain, one
-// warp per larger one.
-template <int LD>
-__global__ void unpack_kernel(const LayoutParams P)
-{
-    using G = Geo<LD>;
-    using mem_t = typename G::mem_t;
-    if (LD == 8) {
-        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.n_dom; g += gridDim.x * blockDim.x) {
-            const uint32_t r = P.dom_rep[g];
-            const int L = P.rep_L[r], Dx = P.rep_Dx[r];
-            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
-            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
-            const uint64_t T = reinterpret_cast<const uint64_t *>(P.tiles)[g];
-            uint64_t *dst = reinterpret_cast<uint64_t *>(P.spins + P.rep_site_off[r] + (uint64_t)(by * 8) * L + (uint64_t)bx * 8);
-#pragma unroll
-            for (int y = 0; y < 8; ++y) dst[(size_t)y * (L / 8)] = unpack8((uint32_t)(T >> (8 * y)));
-        }
-        return;
-    }
-    const int lane = threadIdx.x & 31;
-    const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    const bool wide = (reinterpret_cast<uintptr_t>(P.spins) & 15u) == 0;
-    for (int g = wg; g < P.n_dom; g += nw) {
-        const uint32_t r = P.dom_rep[g];
-        const int L = P.rep_L[r], Dx = P.rep_Dx[r];
-        const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
-        const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
-        const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)g * G::TILE_BYTES);
-        int8_t *dst = P.spins + P.rep_site_off[r] + (uint64_t)(by * LD) * L + (uint64_t)bx * LD;
-        // LD / 16 lanes write one row, 16 bytes each, so that a store covers whole lines
-        constexpr int LPR = LD / 16 > 0 ? LD / 16 : 1;
-        for (int y = lane / LPR; y < LD; y += 32 / LPR) {
-            const int q = lane % LPR;
-            const uint32_t bits = (uint32_t)((uint64_t)trow[y] >> (16 * q));
-            uint64_t *out = reinterpret_cast<uint64_t *>(dst + (size_t)y * L + 16 * q);
-            const uint64_t v0 = unpack8(bits), v1 = unpack8(bits >> 8);
-            if (wide) {
-                *reinterpret_cast<ulonglong2 *>(out) = make_ulonglong2(v0, v1);
-            } else {
-                out[0] = v0;
-                out[1] = v1;
-            }
-        }
-    }
-}
-
-// Observables of the current state from the global tiles and edges
-// (kmc_observables, and the base of a launch's records).  A warp takes
-// OBSERVE_DOMAINS consecutive domains: their bond and spin sums by the whole
-// warp in turn (8x8: a lane each), then every domain's clock (an FP64
-// logarithm, this GPU's slowest arithmetic) in a lane of its own, and one
-// atomic per quantity and run of domains of a replica.  A warp per domain
-// with one lane's logarithm each took 1.49 ms on the 373,000 domains of the
-// 512-replica batch.
-template <int LD> __host__ __device__ constexpr int observe_domains() { return LD == 8 ? 32 : 8; }
-template <int LD, bool EXPO>
-__global__ void observe_kernel(const RunParams P, const uint32_t *dom_rep, int n_dom, int64_t visits,
-                               unsigned long long *acc /* [n_rep][OBS_WORDS] */)
-{
-    using G = Geo<LD>;
-    using row_t = typename G::row_t;
-    using mem_t = typename G::mem_t;
-    constexpr int DPW = observe_domains<LD>();
-    const int lane = threadIdx.x & 31;
-    const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int g0 = wg * DPW; g0 < n_dom; g0 += nw * DPW) {
-        int bonds = 0, mag = 0; // of domain g0 + lane
-        // the edge words of the S neighbour's N row and the E neighbour's W column
-        auto halo = [&](int g, uint64_t &hS, uint64_t &hE) {
-            const uint32_t r = dom_rep[g];
-            const int Dx = P.rep_Dx[r];
-            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
-            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
-            const uint64_t gbase = (uint64_t)g - d;
-            const uint64_t *eS = P.edges + (gbase + (uint32_t)((by + 1 < Dx ? by + 1 : 0) * Dx + bx)) * EDGE_WORDS;
-            const uint64_t *eE = P.edges + (gbase + (uint32_t)(by * Dx + (bx + 1 < Dx ? bx + 1 : 0))) * EDGE_WORDS;
-            hS = (eS[2 * EDGE_N] & 0xFFFFFFFFull) | (eS[2 * EDGE_N + 1] << 32);
-            hE = (eE[2 * EDGE_W] & 0xFFFFFFFFull) | (eE[2 * EDGE_W + 1] << 32);
-        };
-        const int g = g0 + lane;
-        const bool mine = lane < DPW && g < n_dom;
-        if (LD == 8) {
-            if (mine) {
-                const uint64_t T = reinterpret_cast<const uint64_t *>(P.tiles)[g];
-                uint64_t hS, hE;
-                halo(g, hS, hE);
-                // unlike pairs to the east (column 7: the E neighbour's column 0) and to the south
-                uint64_t east = (hE & 0xFFull) * 0x0101010101010101ull & 0x8040201008040201ull; // bit y of row y
-                east = ((east + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
-                const uint64_t E = ((T >> 1) & ~(0x0101010101010101ull << 7)) | (east << 7), S = (T >> 8) | (hS << 56);
-                bonds = 128 - 2 * (__popcll(T ^ E) + __popcll(T ^ S));
-                mag = 2 * __popcll(T) - 64;
-            }
-        } else {
-            for (int i = 0; i < DPW && g0 + i < n_dom; ++i) {
-                uint64_t hS, hE;
-                halo(g0 + i, hS, hE);
-                row_t S[G::RPL];
-                const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)(g0 + i) * G::TILE_BYTES);
-#pragma unroll
-                for (int t = 0; t < G::RPL; ++t) S[t] = (lane < G::NACT) ? (row_t)trow[lane * G::RPL + t] : (row_t)0;
-                int b, m;
-                domain_bonds_mag<LD>(S, hE, hS, lane, b, m);
-                if (lane == i) {
-                    bonds = b;
-                    mag = m;
-                }
-            }
-        }
-        double t = 0.0, sb = 0.0, sh = 0.0;
-        uint32_t r = 0;
-        if (mine) {
-            const uint64_t *ctr = P.dctr + (uint64_t)g * DCTR_WORDS;
-            r = dom_rep[g];
-            t = P.horizon ? __dmul_rn((double)visits, P.dtau)
-                          : domain_time(EXPO, ctr[DCTR_CLKM], (int64_t)ctr[DCTR_CLKE], visits * (int64_t)P.rep_k[r],
-                                        P.lambda);
-            sb = __longlong_as_double((long long)ctr[DCTR_SB]);
-            sh = __longlong_as_double((long long)ctr[DCTR_SH]);
-        }
-        auto add = [&](uint32_t rep, int b, int m, double tt, double s1, double s2) {
-            unsigned long long *a = acc + (size_t)rep * OBS_WORDS;
-            atomicAdd(&a[0], (unsigned long long)(long long)b);
-            atomicAdd(&a[1], (unsigned long long)(long long)m);
-            atomicAdd(reinterpret_cast<double *>(&a[2]), tt);
-            if (s1 != 0.0) atomicAdd(reinterpret_cast<double *>(&a[3]), s1);
-            if (s2 != 0.0) atomicAdd(reinterpret_cast<double *>(&a[4]), s2);
-        };
-        const uint32_t r0 = __shfl_sync(FULL_WARP, r, 0);
-        if (__all_sync(FULL_WARP, !mine || r == r0)) {
-            bonds = __reduce_add_sync(FULL_WARP, bonds);
-            mag = __reduce_add_sync(FULL_WARP, mag);
-#pragma unroll
-            for (int off = 1; off < 32; off <<= 1) {
-                t += __shfl_xor_sync(FULL_WARP, t, off);
-                sb += __shfl_xor_sync(FULL_WARP, sb, off);
-                sh += __shfl_xor_sync(FULL_WARP, sh, off);
-            }
-            if (lane == 0) add(r0, bonds, mag, t, sb, sh);
-        } else if (mine) {
-            add(r, bonds, mag, t, sb, sh);
-        }
-    }
-}
-
 // Records {e, m, e*m, T (, score beta, score h)}: record o = base (the state
 // before the launch) + the changes of every record up to o.  One warp per
 // replica, 32 records at a time: loads and divisions side by side, the sums
 // in record order; the integer sums are exact and e, m
 // follow the oracle's FP64 formula.
-__global__ void finalize_obs_kernel(const unsigned long long *base /* [n_rep][OBS_WORDS] */,
-                                         const unsigned long long *acc, int64_t n_obs, int n_rep,
-                                         const int32_t *rep_L, const int32_t *rep_Dx, double J,
-                                         const double *rep_h, double *out, int stride)
+__device__ __forceinline__ void finalize_records(const RecordParams &R, int warp, int lane)
 {
-    const int r = (blockIdx.x * blockDim.x + threadIdx.x) >> 5, lane = threadIdx.x & 31;
+    const int r = warp, n_rep = R.n_rep, stride = R.stride;
     if (r >= n_rep) return; // whole warps
+    const unsigned long long *base = R.base, *acc = R.acc;
+    const int64_t n_obs = R.n_obs;
+    const int32_t *rep_L = R.rep_L, *rep_Dx = R.rep_Dx;
+    const double *rep_h = R.rep_h, J = R.J;
+    double *out = R.out;
     const unsigned long long *b0 = base + (size_t)r * OBS_WORDS;
     long long bonds = (long long)b0[0], mag = (long long)b0[1];
     double tsum = __longlong_as_double((long long)b0[2]);
@@ -1657,6 +1543,158 @@ __global__ void finalize_obs_kernel(const unsigned long long *base /* [n_rep][OB
     }
 }
 
+// bit tiles -> int8 spins; as pack_kernel: one thread per 8x8 domain, one
+// warp per larger one.  The blocks from n_unpack on form the launch's records.
+template <int LD>
+__global__ void unpack_kernel(const LayoutParams P, const RecordParams R, int n_unpack)
+{
+    using G = Geo<LD>;
+    using mem_t = typename G::mem_t;
+    if ((int)blockIdx.x >= n_unpack) {
+        for (int w = ((int)blockIdx.x - n_unpack) * (int)(blockDim.x >> 5) + (int)(threadIdx.x >> 5); w < R.n_rep;
+             w += ((int)gridDim.x - n_unpack) * (int)(blockDim.x >> 5))
+            finalize_records(R, w, threadIdx.x & 31);
+        return;
+    }
+    if (LD == 8) {
+        for (int g = blockIdx.x * blockDim.x + threadIdx.x; g < P.n_dom; g += n_unpack * blockDim.x) {
+            const uint32_t r = P.dom_rep[g];
+            const int L = P.rep_L[r], Dx = P.rep_Dx[r];
+            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
+            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
+            const uint64_t T = reinterpret_cast<const uint64_t *>(P.tiles)[g];
+            uint64_t *dst = reinterpret_cast<uint64_t *>(P.spins + P.rep_site_off[r] + (uint64_t)(by * 8) * L + (uint64_t)bx * 8);
+#pragma unroll
+            for (int y = 0; y < 8; ++y) dst[(size_t)y * (L / 8)] = unpack8((uint32_t)(T >> (8 * y)));
+        }
+        return;
+    }
+    const int lane = threadIdx.x & 31;
+    const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nw = (n_unpack * blockDim.x) >> 5;
+    const bool wide = (reinterpret_cast<uintptr_t>(P.spins) & 15u) == 0;
+    for (int g = wg; g < P.n_dom; g += nw) {
+        const uint32_t r = P.dom_rep[g];
+        const int L = P.rep_L[r], Dx = P.rep_Dx[r];
+        const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
+        const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
+        const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)g * G::TILE_BYTES);
+        int8_t *dst = P.spins + P.rep_site_off[r] + (uint64_t)(by * LD) * L + (uint64_t)bx * LD;
+        // LD / 16 lanes write one row, 16 bytes each, so that a store covers whole lines
+        constexpr int LPR = LD / 16 > 0 ? LD / 16 : 1;
+        for (int y = lane / LPR; y < LD; y += 32 / LPR) {
+            const int q = lane % LPR;
+            const uint32_t bits = (uint32_t)((uint64_t)trow[y] >> (16 * q));
+            uint64_t *out = reinterpret_cast<uint64_t *>(dst + (size_t)y * L + 16 * q);
+            const uint64_t v0 = unpack8(bits), v1 = unpack8(bits >> 8);
+            if (wide) {
+                *reinterpret_cast<ulonglong2 *>(out) = make_ulonglong2(v0, v1);
+            } else {
+                out[0] = v0;
+                out[1] = v1;
+            }
+        }
+    }
+}
+
+// Observables of the current state from the global tiles and edges
+// (kmc_observables, and the base of a launch's records).  A warp takes
+// dpw consecutive domains (8x8: 32; else up to 8 while the GPU is full): their bond and spin sums by the whole
+// warp in turn (8x8: a lane each), then every domain's clock (an FP64
+// logarithm, this GPU's slowest arithmetic) in a lane of its own, and one
+// atomic per quantity and run of domains of a replica.  A warp per domain
+// with one lane's logarithm each took 1.49 ms on the 373,000 domains of the
+// 512-replica batch.
+template <int LD, bool EXPO>
+__global__ void observe_kernel(const RunParams P, const uint32_t *dom_rep, int n_dom, int64_t visits,
+                               unsigned long long *acc /* [n_rep][OBS_WORDS] */, int dpw)
+{
+    using G = Geo<LD>;
+    using row_t = typename G::row_t;
+    using mem_t = typename G::mem_t;
+    const int lane = threadIdx.x & 31;
+    const int wg = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int nw = (gridDim.x * blockDim.x) >> 5;
+    for (int g0 = wg * dpw; g0 < n_dom; g0 += nw * dpw) {
+        int bonds = 0, mag = 0; // of domain g0 + lane
+        // the edge words of the S neighbour's N row and the E neighbour's W column
+        auto halo = [&](int g, uint64_t &hS, uint64_t &hE) {
+            const uint32_t r = dom_rep[g];
+            const int Dx = P.rep_Dx[r];
+            const uint32_t d = (uint32_t)g - P.rep_dom_off[r];
+            const int by = (int)(d / (uint32_t)Dx), bx = (int)(d - (uint32_t)by * (uint32_t)Dx);
+            const uint64_t gbase = (uint64_t)g - d;
+            const uint64_t *eS = P.edges + (gbase + (uint32_t)((by + 1 < Dx ? by + 1 : 0) * Dx + bx)) * EDGE_WORDS;
+            const uint64_t *eE = P.edges + (gbase + (uint32_t)(by * Dx + (bx + 1 < Dx ? bx + 1 : 0))) * EDGE_WORDS;
+            hS = (eS[2 * EDGE_N] & 0xFFFFFFFFull) | (eS[2 * EDGE_N + 1] << 32);
+            hE = (eE[2 * EDGE_W] & 0xFFFFFFFFull) | (eE[2 * EDGE_W + 1] << 32);
+        };
+        const int g = g0 + lane;
+        const bool mine = lane < dpw && g < n_dom;
+        if (LD == 8) {
+            if (mine) {
+                const uint64_t T = reinterpret_cast<const uint64_t *>(P.tiles)[g];
+                uint64_t hS, hE;
+                halo(g, hS, hE);
+                // unlike pairs to the east (column 7: the E neighbour's column 0) and to the south
+                uint64_t east = (hE & 0xFFull) * 0x0101010101010101ull & 0x8040201008040201ull; // bit y of row y
+                east = ((east + 0x7F7F7F7F7F7F7F7Full) >> 7) & 0x0101010101010101ull;
+                const uint64_t E = ((T >> 1) & ~(0x0101010101010101ull << 7)) | (east << 7), S = (T >> 8) | (hS << 56);
+                bonds = 128 - 2 * (__popcll(T ^ E) + __popcll(T ^ S));
+                mag = 2 * __popcll(T) - 64;
+            }
+        } else {
+            for (int i = 0; i < dpw && g0 + i < n_dom; ++i) {
+                uint64_t hS, hE;
+                halo(g0 + i, hS, hE);
+                row_t S[G::RPL];
+                const mem_t *trow = reinterpret_cast<const mem_t *>(P.tiles + (uint64_t)(g0 + i) * G::TILE_BYTES);
+#pragma unroll
+                for (int t = 0; t < G::RPL; ++t) S[t] = (lane < G::NACT) ? (row_t)trow[lane * G::RPL + t] : (row_t)0;
+                int b, m;
+                domain_bonds_mag<LD>(S, hE, hS, lane, b, m);
+                if (lane == i) {
+                    bonds = b;
+                    mag = m;
+                }
+            }
+        }
+        double t = 0.0, sb = 0.0, sh = 0.0;
+        uint32_t r = 0;
+        if (mine) {
+            const uint64_t *ctr = P.dctr + (uint64_t)g * DCTR_WORDS;
+            r = dom_rep[g];
+            t = P.horizon ? __dmul_rn((double)visits, P.dtau)
+                          : domain_time(EXPO, ctr[DCTR_CLKM], (int64_t)ctr[DCTR_CLKE], visits * (int64_t)P.rep_k[r],
+                                        P.lambda);
+            sb = __longlong_as_double((long long)ctr[DCTR_SB]);
+            sh = __longlong_as_double((long long)ctr[DCTR_SH]);
+        }
+        auto add = [&](uint32_t rep, int b, int m, double tt, double s1, double s2) {
+            unsigned long long *a = acc + (size_t)rep * OBS_WORDS;
+            atomicAdd(&a[0], (unsigned long long)(long long)b);
+            atomicAdd(&a[1], (unsigned long long)(long long)m);
+            atomicAdd(reinterpret_cast<double *>(&a[2]), tt);
+            if (s1 != 0.0) atomicAdd(reinterpret_cast<double *>(&a[3]), s1);
+            if (s2 != 0.0) atomicAdd(reinterpret_cast<double *>(&a[4]), s2);
+        };
+        const uint32_t r0 = __shfl_sync(FULL_WARP, r, 0);
+        if (__all_sync(FULL_WARP, !mine || r == r0)) {
+            bonds = __reduce_add_sync(FULL_WARP, bonds);
+            mag = __reduce_add_sync(FULL_WARP, mag);
+#pragma unroll
+            for (int off = 1; off < 32; off <<= 1) {
+                t += __shfl_xor_sync(FULL_WARP, t, off);
+                sb += __shfl_xor_sync(FULL_WARP, sb, off);
+                sh += __shfl_xor_sync(FULL_WARP, sh, off);
+            }
+            if (lane == 0) add(r0, bonds, mag, t, sb, sh);
+        } else if (mine) {
+            add(r, bonds, mag, t, sb, sh);
+        }
+    }
+}
+
 // per-domain counters -> host-facing arrays (hash, flips, clock)
 // dtau > 0: fixed-time visits, the clock is visits * dtau.
 template <bool EXPO>
@@ -1675,20 +1713,7 @@ __global__ void domain_state_kernel(const uint64_t *dctr, int n_dom, int64_t vis
                                     lambda);
 }
 
-// zero counters: hash basis, flips 0, clock 1.0 (m = 2^63, e = 0), scores 0
-__global__ void reset_counters_kernel(uint64_t *dctr, int n_dom)
-{
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g >= n_dom) return;
-    uint64_t *c = dctr + (uint64_t)g * DCTR_WORDS;
-    c[DCTR_HASH] = HASH_BASIS;
-    c[DCTR_FLIPS] = 0;
-    c[DCTR_CLKM] = 1ull << 63;
-    c[DCTR_CLKE] = 0;
-    c[DCTR_SB] = 0;
-    c[DCTR_SH] = 0;
-    c[DCTR_STEPS] = 0;
-}
+__global__ void reset_counters_kernel(uint64_t *dctr, int n_dom) { reset_counters(dctr, n_dom); }
 
 // Score sums of domains g0 .. g1 - 1 in domain order, eight domains' loads at
 // a time ahead of their additions.

@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
             const uint64_t seed = __ldg(&P.rep_seed[r]);
             uint64_t A[10];
 #pragma unroll
-            for (int c = 0; c < 10; ++c) A[c] = __ldg(&P.rep_A[(size_t)r * 16 + c]);
+            for (int c = 0; c < 10; ++c) A[c] = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + c]);
             const uint32_t d = g - base;
             const uint32_t by = d / Dx, bx = d - by * Dx;
             const uint32_t gN = by == 0 ? g + (Dx - 1) * Dx : g - Dx, gS = by == Dx - 1 ? g - (Dx - 1) * Dx : g + Dx;
@@ -360,7 +360,7 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
                 for (int cc = 0; cc < 9; ++cc) c += (th >= Ch[cc]) ? 1 : 0;
                 uint64_t Cprev = cum[c * bd];
                 while (tgt < Cprev) Cprev = cum[--c * bd];
-                const uint64_t Ac = __ldg(&P.rep_A[(size_t)r * 16 + c]);
+                const uint64_t Ac = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + c]);
                 // exact jj = floor((tgt - C_{c-1}) / A_c) < n_c <= 64: an FP32
                 // estimate rounded toward the lower side is jj or jj - 1, and
                 // one integer comparison decides which

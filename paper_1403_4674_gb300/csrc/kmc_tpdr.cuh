@@ -178,9 +178,9 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
     uint64_t A[10];
 #pragma unroll
     for (int c = 0; c < 10; ++c) {
-        A[c] = __ldg(&P.rep_A[(size_t)r * 16 + c]);
+        A[c] = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + c]);
         at(Lay::AT + c) = A[c];
-        at(Lay::MR + c) = A[c] ? ~0ull / A[c] : 0ull;
+        at(Lay::MR + c) = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + RATE_RECIP + c]);
     }
 #pragma unroll
     for (int i = CHUNK; i < CHUNK + 8; ++i) at(Lay::TG + i) = ~0ull;
