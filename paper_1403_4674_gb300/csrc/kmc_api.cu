@@ -42,6 +42,7 @@ struct Plan {
     int max_slots = 0;
     int groups = 0;   // THREADS mode of L_d = 16, 32, 64: lanes per domain (grp_kernel), 0: one thread per domain
     size_t smem = 0;
+    bool checked = false; // check_plan has passed for the kernels of now
     std::vector<uint32_t> cta_slot_off, cta_col_off, cta_rt_off, rt_rep, slot_g, slot_rt, slot_nb;
 };
 
@@ -768,11 +769,15 @@ kmc_status plan_thread_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
         const int ns = lengthy ? 2 : 1;
         const int64_t room = (int64_t)(lengthy ? 4 : 8) * c->sm_count;
         for (int G = most; G >= fewest; G /= 2)
-            if (warps(G, ns) <= room && plan_groups(c, G, ns, wpb, pl, interleave) == KMC_OK && check_plan(c, pl) == KMC_OK)
+            if (warps(G, ns) <= room && plan_groups(c, G, ns, wpb, pl, interleave) == KMC_OK && check_plan(c, pl) == KMC_OK) {
+                pl.checked = true;
                 return KMC_OK;
+            }
         if (warps(fewest, 2) <= (int64_t)10 * c->sm_count && plan_groups(c, fewest, 2, wpb, pl, interleave) == KMC_OK &&
-            check_plan(c, pl) == KMC_OK)
+            check_plan(c, pl) == KMC_OK) {
+            pl.checked = true;
             return KMC_OK;
+        }
     }
     return plan_thread_rows(c, wpb ? wpb : 1, pl, interleave);
 }
@@ -871,8 +876,9 @@ kmc_status check_plan(kmc_ctx *c, const Plan &pl)
 
 kmc_status install_plan(kmc_ctx *c, Plan &pl)
 {
-    kmc_status s = check_plan(c, pl);
+    kmc_status s = pl.checked ? KMC_OK : check_plan(c, pl);
     if (s != KMC_OK) return s;
+    pl.checked = false;
     std::vector<uint32_t> flat;
     for (auto *v : {&pl.cta_slot_off, &pl.cta_col_off, &pl.cta_rt_off, &pl.rt_rep, &pl.slot_g, &pl.slot_rt, &pl.slot_nb})
         flat.insert(flat.end(), v->begin(), v->end());

@@ -243,25 +243,33 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
         uint64_t m = 1ull << 63;
         int e = 0;
         if (EXPO) joined_clock(b, m, e);
-        if (gl == 0 && u32(b, Q::META) != 0xFFFFFFFFu) {
-            if (EXPO) {
-                uint64_t cm = u64(b, Q::CTR + 24);
-                int64_t ce = (int64_t)u64(b, Q::CTR + 32);
-                mant_mul(cm, ce, m, (int64_t)e);
-                u64(b, Q::CTR + 24) = cm;
-                u64(b, Q::CTR + 32) = (uint64_t)ce;
-            }
-            const uint64_t o0 = u64(b, Q::OBS), o1 = u64(b, Q::OBS + 8);
-            const uint32_t o = (uint32_t)o0;
-            if (o != NO_RECORD && (int64_t)o < P.n_obs) {
-                unsigned long long *acc = P.obs_acc + ((size_t)o * P.n_rep + u32(b, Q::META + 12)) * OBS_WORDS;
-                const int bonds = (int)(uint32_t)o1, mag = (int)(uint32_t)(o1 >> 32);
-                if (bonds != 0) atomicAdd(&acc[0], (unsigned long long)(long long)bonds);
-                if (mag != 0) atomicAdd(&acc[1], (unsigned long long)(long long)mag);
-                const double dt = EXPO ? domain_time(true, m, (int64_t)e, 0, P.lambda)
-                                       : __ddiv_rn((double)(uint32_t)(o0 >> 32), P.lambda);
-                atomicAdd(reinterpret_cast<double *>(&acc[2]), dt);
-            }
+        const bool mine = gl == 0 && u32(b, Q::META) != 0xFFFFFFFFu;
+        const uint64_t o0 = u64(b, Q::OBS), o1 = u64(b, Q::OBS + 8);
+        const uint32_t o = (uint32_t)o0;
+        const bool on = mine && o != NO_RECORD && (int64_t)o < P.n_obs;
+        double dt = 0.0;
+        if (mine && EXPO) {
+            uint64_t cm = u64(b, Q::CTR + 24);
+            int64_t ce = (int64_t)u64(b, Q::CTR + 32);
+            mant_mul(cm, ce, m, (int64_t)e);
+            u64(b, Q::CTR + 24) = cm;
+            u64(b, Q::CTR + 32) = (uint64_t)ce;
+        }
+        if (on)
+            dt = EXPO ? domain_time(true, m, (int64_t)e, 0, P.lambda) : __ddiv_rn((double)(uint32_t)(o0 >> 32), P.lambda);
+        // the set's domains are one replica's and share the record: one sum
+        int bonds = on ? (int)(uint32_t)o1 : 0, mag = on ? (int)(uint32_t)(o1 >> 32) : 0;
+#pragma unroll
+        for (int off = G; off < 32; off <<= 1) {
+            dt += __shfl_xor_sync(FULL_WARP, dt, off);
+            bonds += __shfl_xor_sync(FULL_WARP, bonds, off);
+            mag += __shfl_xor_sync(FULL_WARP, mag, off);
+        }
+        if (on && lane == 0) {
+            unsigned long long *acc = P.obs_acc + ((size_t)o * P.n_rep + u32(b, Q::META + 12)) * OBS_WORDS;
+            if (bonds != 0) atomicAdd(&acc[0], (unsigned long long)(long long)bonds);
+            if (mag != 0) atomicAdd(&acc[1], (unsigned long long)(long long)mag);
+            atomicAdd(reinterpret_cast<double *>(&acc[2]), dt);
         }
         __syncwarp();
     };

@@ -280,6 +280,47 @@ __device__ __forceinline__ double domain_time(bool expo, uint64_t M, int64_t E, 
     return __ddiv_rn((double)steps, lambda);
 }
 
+// A warp's lanes add the changes of a record (bond sum, magnetisation, clock,
+// scores) to their replicas' sums.  Lanes of one replica and record (the usual
+// case) are summed first: one atomic per quantity instead of 32, and fewer
+// roundings.  Called by the whole warp; on: this lane has something to add.
+template <bool GRAD>
+__device__ __forceinline__ void add_to_record(const RunParams &P, bool on, uint32_t o, uint32_t r, int bonds, int mag,
+                                              double dt, double sb, double sh)
+{
+    const unsigned who = __ballot_sync(FULL_WARP, on);
+    if (!who) return;
+    const int first = __ffs((int)who) - 1;
+    const uint32_t o0 = __shfl_sync(FULL_WARP, o, first), r0 = __shfl_sync(FULL_WARP, r, first);
+    bool lead = on;
+    if (__all_sync(FULL_WARP, !on || (o == o0 && r == r0))) {
+        bonds = __reduce_add_sync(FULL_WARP, on ? bonds : 0);
+        mag = __reduce_add_sync(FULL_WARP, on ? mag : 0);
+        dt = on ? dt : 0.0;
+        sb = on ? sb : 0.0;
+        sh = on ? sh : 0.0;
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1) {
+            dt += __shfl_xor_sync(FULL_WARP, dt, off);
+            if (GRAD) {
+                sb += __shfl_xor_sync(FULL_WARP, sb, off);
+                sh += __shfl_xor_sync(FULL_WARP, sh, off);
+            }
+        }
+        lead = (int)(threadIdx.x & 31) == first;
+    }
+    if (lead) {
+        unsigned long long *acc = P.obs_acc + ((size_t)o * P.n_rep + r) * OBS_WORDS;
+        if (bonds != 0) atomicAdd(&acc[0], (unsigned long long)(long long)bonds);
+        if (mag != 0) atomicAdd(&acc[1], (unsigned long long)(long long)mag);
+        atomicAdd(reinterpret_cast<double *>(&acc[2]), dt);
+        if (GRAD) {
+            atomicAdd(reinterpret_cast<double *>(&acc[3]), sb);
+            atomicAdd(reinterpret_cast<double *>(&acc[4]), sh);
+        }
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Row-plane state of one domain held by one warp: lane l holds rows
 // l*RPL .. l*RPL+RPL-1 (bit x = column x), plus the bit-sliced count of up

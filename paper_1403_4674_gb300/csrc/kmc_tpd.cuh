@@ -125,20 +125,17 @@ __device__ __forceinline__ void tpd_mul(uint64_t &m, int &e, uint64_t V, bool on
     e -= on ? z : 0;
 }
 
-// The open record of domain g goes to its replica's record (records past
-// the launch's last one are dropped), as the warp kernel's flush.
+// The lanes' open records go to their replicas' records (records past the
+// launch's last one are dropped), as the warp kernel's flush; called by the
+// whole warp, on: this lane has one to close.
 template <bool EXPO>
-__device__ __forceinline__ void tpd_flush(const RunParams &P, const ulonglong2 &ob, const ulonglong2 &clk, uint32_t r)
+__device__ __forceinline__ void tpd_flush(const RunParams &P, bool on, const ulonglong2 &ob, const ulonglong2 &clk, uint32_t r)
 {
     const uint32_t o = (uint32_t)ob.x;
-    if (o == NO_RECORD || (int64_t)o >= P.n_obs) return;
-    unsigned long long *acc = P.obs_acc + ((size_t)o * P.n_rep + r) * OBS_WORDS;
-    const int bonds = (int)(uint32_t)ob.y, mag = (int)(uint32_t)(ob.y >> 32);
-    if (bonds != 0) atomicAdd(&acc[0], (unsigned long long)(long long)bonds);
-    if (mag != 0) atomicAdd(&acc[1], (unsigned long long)(long long)mag);
-    const uint32_t steps = (uint32_t)(ob.x >> 32);
-    const double dt = EXPO ? domain_time(true, clk.x, (int64_t)clk.y, 0, P.lambda) : __ddiv_rn((double)steps, P.lambda);
-    atomicAdd(reinterpret_cast<double *>(&acc[2]), dt);
+    on = on && o != NO_RECORD && (int64_t)o < P.n_obs;
+    double dt = 0.0;
+    if (on) dt = EXPO ? domain_time(true, clk.x, (int64_t)clk.y, 0, P.lambda) : __ddiv_rn((double)(uint32_t)(ob.x >> 32), P.lambda);
+    add_to_record<false>(P, on, o, r, (int)(uint32_t)ob.y, (int)(uint32_t)(ob.y >> 32), dt, 0.0, 0.0);
 }
 
 // Persistent kernel: thread t visits, in every colour phase, the domains
@@ -386,15 +383,20 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
                 R = tpd_rates(T, pl, A, Ch, cum, bd);
                 tgt = next;
             }
+            // edges first (neighbours wait for them), then tile, counters and record
+            if (has) {
+                uint64_t *ew = P.edges + (size_t)g * EDGE_WORDS;
+                const uint64_t cnt = (uint64_t)after << 32;
+                st_cg(ew + 2 * EDGE_N, cnt | (T & 0xFFull));
+                st_cg(ew + 2 * EDGE_S, cnt | (T >> 56));
+                st_cg(ew + 2 * EDGE_W, cnt | tpd_col_gather(T));
+                st_cg(ew + 2 * EDGE_E, cnt | tpd_col_gather(T >> 7));
+            }
+            // the visit's changes belong to the first record at or after its pass
+            const bool turn = P.n_obs > 0 && has && (int64_t)(uint32_t)ob01.x != o;
+            if (__any_sync(FULL_WARP, turn)) tpd_flush<EXPO>(P, turn, ob01, obM, r);
             if (!has) continue;
             if (EXPO) mant_mul(clkM, clkE, vM, (int64_t)vE); // the domain clock takes the visit's product
-            // edges first (neighbours wait for them), then tile and counters
-            uint64_t *ew = P.edges + (size_t)g * EDGE_WORDS;
-            const uint64_t cnt = (uint64_t)after << 32;
-            st_cg(ew + 2 * EDGE_N, cnt | (T & 0xFFull));
-            st_cg(ew + 2 * EDGE_S, cnt | (T >> 56));
-            st_cg(ew + 2 * EDGE_W, cnt | tpd_col_gather(T));
-            st_cg(ew + 2 * EDGE_E, cnt | tpd_col_gather(T >> 7));
             if (flips) {
                 tile64w[g] = T;
                 ctr[DCTR_HASH] = H;
@@ -406,11 +408,9 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
                 ctr[DCTR_CLKE] = (uint64_t)clkE;
             }
             if (P.n_obs > 0) {
-                // the visit's changes belong to the first record at or after its pass
                 uint64_t om = obM.x;
                 int64_t oe = (int64_t)obM.y;
                 if ((int64_t)(uint32_t)ob01.x != o) {
-                    tpd_flush<EXPO>(P, ob01, obM, r);
                     ob01 = make_ulonglong2((uint64_t)(uint32_t)o, 0);
                     om = 1ull << 63;
                     oe = 0;
@@ -434,10 +434,13 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
     // every owned domain's open record
     if (P.n_obs > 0) {
         for (int c = 0; c < 4; ++c) {
-            for (uint32_t i = col_off[c] + (uint32_t)tid; i < col_off[c + 1]; i += (uint32_t)nthreads) {
-                const uint32_t g = col_list[i];
+            const uint32_t lo = col_off[c], hi = col_off[c + 1];
+            const uint32_t rounds = (hi - lo + (uint32_t)nthreads - 1) / (uint32_t)nthreads;
+            for (uint32_t m = 0; m < rounds; ++m) {
+                const uint32_t i = lo + (uint32_t)tid + m * (uint32_t)nthreads;
+                const uint32_t g = i < hi ? col_list[i] : col_list[lo];
                 const ulonglong2 *ob = reinterpret_cast<const ulonglong2 *>(P.obs_dom + (size_t)g * TPD_OBS_WORDS);
-                tpd_flush<EXPO>(P, ob[0], ob[1], P.dom_rep[g]);
+                tpd_flush<EXPO>(P, i < hi, ob[0], ob[1], P.dom_rep[g]);
             }
         }
     }
