@@ -40,7 +40,7 @@ struct Plan {
     int wpb = 0;
     int max_rt = 0;   // replica tables per CTA; sets per warp of a group plan
     int max_slots = 0;
-    int groups = 0;   // THREADS mode of L_d = 16, 32, 64: lanes per domain (grp_kernel), 0: one thread per domain
+    int groups = 0;   // lanes per domain (grp_kernel; THREADS mode of L_d = 16, 32, 64, or GRID), 0: the mode's own kernel
     size_t smem = 0;
     bool checked = false; // check_plan has passed for the kernels of now
     std::vector<uint32_t> cta_slot_off, cta_col_off, cta_rt_off, rt_rep, slot_g, slot_rt, slot_nb;
@@ -82,6 +82,11 @@ struct kmc_ctx {
     // device copy of the launch plan
     uint32_t *d_plan = nullptr;
     size_t plan_words = 0;
+    // beside a random-order run's lane groups: the warp plan that such a run
+    // installs otherwise, ready for a fixed-time run (also while capturing)
+    uint32_t *d_alt = nullptr;
+    size_t alt_words = 0;
+    Plan alt;
 
     double J = 1.0, nu = 1.0;
     std::vector<double> beta, h, a, gb, gh;
@@ -739,46 +744,50 @@ kmc_status plan_groups(kmc_ctx *c, int G, int ns, int wpb, Plan &pl, bool interl
     return KMC_OK;
 }
 
-// THREADS plan of L_d = 16, 32, 64: lane groups per domain while the domains
-// are few enough for about two of their warps per scheduler, else (and with
-// scores) one thread per domain.  Fewer lanes per domain cost fewer
-// instructions per event, more lanes shorten it, and beyond one active warp
-// per scheduler they compete; with long visits (k >= 8, most of the time in
-// events) two colours per warp and half as many warps are faster, with short
-// ones a warp per colour, whose fixed work hides behind the other colours.
-// Measured, us per schedule (G, ns; thread = one thread per domain):
+// Lane groups per domain (L_d = 16, 32, 64) while the domains are few enough
+// for about two of their warps per scheduler.  Fewer lanes per domain cost
+// fewer instructions per event, more lanes shorten it, and beyond one active
+// warp per scheduler they compete; with long visits (k >= 8, most of the time
+// in events) two colours per warp and half as many warps are faster, with
+// short ones a warp per colour, whose fixed work hides behind the other
+// colours.  Measured, us per schedule (G, ns; thread = one thread per domain):
 //   1024 domains of 32x32, k = 4:  (32,1) 5.8  (32,2) 7.3  (8,1) 7.6  thread 16.2
-//   1024 domains of 32x32, k = 16: (32,1) 36.7 (32,2) 33.4 (8,1) 43.8 thread 72.8
-//   4096 domains of 16x16, k = 4:  (8,1) 15.2  (8,2) 16.2  (16,1) 16.8 thread 28.9
-//   4096 domains of 32x32, k = 8:  (8,2) 28.2  (8,1) 31.2  (16,2) 30.0 thread 48.0
-//   12288 domains of 32x32, k = 8: (8,2) 47.8  thread 50.1; 16384: (8,2) 59.2 thread 50.3
-//   1024 domains of 64x64, k = 8:  (32,2) 26.9 (16,1) 36.5 thread 70.1
-//   9216 domains of 64x64, k = 8:  (16,2) 81.4 thread 77.9
+//   1024 domains of 32x32, k = 16: (32,1) 36.7 (32,2) 33.4 (8,1) 42.4 thread 65.6
+//   4096 domains of 16x16, k = 4:  (8,1) 15.2  (8,2) 16.0  (16,1) 16.6 thread 25.5
+//   4096 domains of 32x32, k = 8:  (8,2) 27.3  (8,1) 29.5  (16,2) 30.1 thread 40.7
+//   8192 domains of 32x32, k = 8:  (8,2) 37.5  thread 42.7; 12288: (8,2) 47.8 thread 43.8
+//   1024 domains of 64x64, k = 8:  (32,2) 26.9 (16,1) 36.7 thread 61.4
+//   4096 domains of 64x64, k = 8:  (16,2) 50.5 thread 65.0; 9216: (16,2) 81.4 thread 77.9
+kmc_status plan_few_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
+{
+    if (c->LD == 8) return fail(c, KMC_EINVAL, "no lane-group kernel for L_d = 8");
+    int64_t steps = 0;
+    for (int r = 0; r < c->n_rep; ++r) steps += (int64_t)c->kr[r] * c->Dx[r] * c->Dx[r];
+    const bool lengthy = steps >= 8ll * c->n_dom;
+    auto warps = [&](int G, int ns) {
+        int64_t sets = 0;
+        for (int r = 0; r < c->n_rep; ++r) sets += (c->Dx[r] * c->Dx[r] / 4 + 32 / G - 1) / (32 / G);
+        return 4 * sets / ns;
+    };
+    auto take = [&](int G, int ns) {
+        if (plan_groups(c, G, ns, wpb, pl, interleave) != KMC_OK || check_plan(c, pl) != KMC_OK) return false;
+        pl.checked = true;
+        return true;
+    };
+    const int most = std::min(c->LD, 32), fewest = (c->LD == 64) ? 16 : 8;
+    const int ns = lengthy ? 2 : 1;
+    const int64_t room = (int64_t)(lengthy ? 4 : 8) * c->sm_count;
+    for (int G = most; G >= fewest; G /= 2)
+        if (warps(G, ns) <= room && take(G, ns)) return KMC_OK;
+    if (warps(fewest, 2) <= (int64_t)8 * c->sm_count && take(fewest, 2)) return KMC_OK;
+    return fail(c, KMC_EINVAL, "too many domains for lane groups");
+}
+
+// THREADS plan of L_d = 16, 32, 64: lane groups while they pay, else (and
+// with scores) one thread per domain.
 kmc_status plan_thread_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
 {
-    if (!c->grad) {
-        int64_t steps = 0;
-        for (int r = 0; r < c->n_rep; ++r) steps += (int64_t)c->kr[r] * c->Dx[r] * c->Dx[r];
-        const bool lengthy = steps >= 8ll * c->n_dom;
-        auto warps = [&](int G, int ns) {
-            int64_t sets = 0;
-            for (int r = 0; r < c->n_rep; ++r) sets += (c->Dx[r] * c->Dx[r] / 4 + 32 / G - 1) / (32 / G);
-            return 4 * sets / ns;
-        };
-        const int most = std::min(c->LD, 32), fewest = (c->LD == 64) ? 16 : 8;
-        const int ns = lengthy ? 2 : 1;
-        const int64_t room = (int64_t)(lengthy ? 4 : 8) * c->sm_count;
-        for (int G = most; G >= fewest; G /= 2)
-            if (warps(G, ns) <= room && plan_groups(c, G, ns, wpb, pl, interleave) == KMC_OK && check_plan(c, pl) == KMC_OK) {
-                pl.checked = true;
-                return KMC_OK;
-            }
-        if (warps(fewest, 2) <= (int64_t)10 * c->sm_count && plan_groups(c, fewest, 2, wpb, pl, interleave) == KMC_OK &&
-            check_plan(c, pl) == KMC_OK) {
-            pl.checked = true;
-            return KMC_OK;
-        }
-    }
+    if (!c->grad && plan_few_domains(c, wpb, pl, interleave) == KMC_OK) return KMC_OK;
     return plan_thread_rows(c, wpb ? wpb : 1, pl, interleave);
 }
 
@@ -805,7 +814,7 @@ int balanced_thread_ctas(const kmc_ctx *c, int wpb)
 // registers, so fewer of its CTAs fit an SM; kmc_enable_grad re-checks).
 kmc_status check_plan(kmc_ctx *c, const Plan &pl)
 {
-    if (pl.mode == KMC_LAUNCH_THREADS) {
+    if (pl.mode == KMC_LAUNCH_THREADS || pl.groups) {
         if (c->grad && (c->LD == 8 || c->LD == 64))
             return fail(c, KMC_EINVAL, "the thread-per-domain plan of L_d = %d has no score kernel", c->LD);
         if (c->grad && pl.groups) return fail(c, KMC_EINVAL, "the lane-group kernel carries no scores");
@@ -879,6 +888,8 @@ kmc_status install_plan(kmc_ctx *c, Plan &pl)
     kmc_status s = pl.checked ? KMC_OK : check_plan(c, pl);
     if (s != KMC_OK) return s;
     pl.checked = false;
+    if (c->d_alt) cudaFree(c->d_alt);
+    c->d_alt = nullptr;
     std::vector<uint32_t> flat;
     for (auto *v : {&pl.cta_slot_off, &pl.cta_col_off, &pl.cta_rt_off, &pl.rt_rep, &pl.slot_g, &pl.slot_rt, &pl.slot_nb})
         flat.insert(flat.end(), v->begin(), v->end());
@@ -1190,7 +1201,7 @@ kmc_status sync_ctx(kmc_ctx *c)
 void free_all(kmc_ctx *c)
 {
     void **ptrs[] = {(void **)&c->d_L, (void **)&c->d_Dx, (void **)&c->d_k, (void **)&c->d_init, (void **)&c->d_dom_off, (void **)&c->d_dom_rep,
-                     (void **)&c->d_site_off, (void **)&c->d_blk_off, (void **)&c->d_seed, (void **)&c->d_A,
+                     (void **)&c->d_alt, (void **)&c->d_site_off, (void **)&c->d_blk_off, (void **)&c->d_seed, (void **)&c->d_A,
                      (void **)&c->d_gfix, (void **)&c->d_grad, (void **)&c->d_h, (void **)&c->d_tiles,
                      (void **)&c->d_edges, (void **)&c->d_dctr, (void **)&c->d_err,
                      (void **)&c->d_obs_acc, (void **)&c->d_tmp, (void **)&c->d_plan, (void **)&c->d_htab,
@@ -1687,15 +1698,44 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     const int64_t units = pass_obs ? n_schedules * (schedule == KMC_SCHEDULE_PALINDROME ? 8 : 4) : n_schedules;
     const int64_t n_obs = want_obs ? units / obs_every : 0;
     const bool cap = capturing(c);
-    if (c->plan.mode == KMC_LAUNCH_THREADS && ((c->grad && (c->LD == 8 || c->LD == 64)) ||
-                                               time_mode == KMC_TIME_HORIZON || schedule == KMC_SCHEDULE_RANDOM_PERM)) {
+    const bool random_order = schedule == KMC_SCHEDULE_RANDOM_PERM, fixed_time = time_mode == KMC_TIME_HORIZON;
+    const bool scores8_64 = c->grad && (c->LD == 8 || c->LD == 64);
+    if (c->plan.groups && c->plan.mode == KMC_LAUNCH_GRID && fixed_time && c->d_alt) {
+        // back to the warp plan (earlier launches keep reading the other buffer)
+        std::swap(c->plan, c->alt);
+        std::swap(c->d_plan, c->d_alt);
+        std::swap(c->plan_words, c->alt_words);
+    }
+    if ((c->plan.mode == KMC_LAUNCH_THREADS && (scores8_64 || fixed_time || random_order)) ||
+        (c->plan.groups && (c->grad || fixed_time))) {
         // the thread kernels cover fixed-length visits of the palindromic
-        // and fixed schedules (with scores at L_d = 16, 32): this run takes a warp plan
-        // (installed once the stream has drained: earlier launches read the
-        // plan buffer)
+        // and fixed schedules (with scores at L_d = 16, 32), and lane groups
+        // random orders too: this run takes a warp plan, or a grid of lane
+        // groups with the warp plan kept beside it (installed once the stream
+        // has drained: earlier launches read the plan buffer)
         if (cap) return fail(c, KMC_EINVAL, "this run needs a warp launch plan; set one before capturing");
         CUDA_TRY(c, cudaStreamSynchronize(s));
         if ((st = default_warp_plan(c)) != KMC_OK) return st;
+        Plan pl;
+        if (random_order && !fixed_time && !c->grad && plan_few_domains(c, 0, pl, false) == KMC_OK) {
+            pl.mode = KMC_LAUNCH_GRID;
+            Plan warp = c->plan;
+            uint32_t *d_warp = c->d_plan;
+            const size_t words = c->plan_words;
+            c->d_plan = nullptr;
+            c->plan_words = 0;
+            if (install_plan(c, pl) == KMC_OK) {
+                c->alt = std::move(warp);
+                c->d_alt = d_warp;
+                c->alt_words = words;
+            } else {
+                cudaGetLastError();
+                if (c->d_plan) cudaFree(c->d_plan);
+                c->plan = std::move(warp);
+                c->d_plan = d_warp;
+                c->plan_words = words;
+            }
+        }
     }
     if (want_obs && n_obs > 0) {
         const size_t words = (size_t)n_obs * c->n_rep * OBS_WORDS;
@@ -1731,7 +1771,7 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     P.visits_before = c->visits_done;
     const Plan &pl = c->plan;
     const bool cluster = pl.mode == KMC_LAUNCH_CLUSTER;
-    const bool threads = pl.mode == KMC_LAUNCH_THREADS;
+    const bool threads = pl.mode == KMC_LAUNCH_THREADS || pl.groups;
     RunKernel kern = threads ? thread_plan_kernel(pl, c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad)
                              : run_kernel_for(c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad, cluster);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;

@@ -26,9 +26,9 @@
 // Halos come from the neighbours' stamped edge words: in shared memory when
 // the neighbour is in the same CTA, else in global memory (L2).
 //
-// Scope: palindromic and fixed colour schedules, exponential and expected
-// clocks, per-replica k, records at schedule endpoints or every colour pass.
-// Fixed-time visits and random colour orders use the warp kernel.
+// Scope: every colour schedule, exponential and expected clocks, per-replica
+// k, records at schedule endpoints or every colour pass.  Fixed-time visits
+// and scores use the other kernels.
 #pragma once
 
 #include "kmc_tpdr.cuh"
@@ -709,11 +709,13 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
     // domains have completed before it, in closed form.  Two phases of one
     // colour in a row are one visit (the palindrome's middle, and its ends
     // where two schedules meet) unless an observation falls between them.
-    const bool pal = P.schedule == SCHED_PALINDROME, fuse = pal && !P.obs_pass;
+    // With random orders every replica has its own order of the four colours in
+    // every schedule; a colour's domains then complete one visit per schedule.
+    const bool pal = P.schedule == SCHED_PALINDROME, fuse = pal && !P.obs_pass, perm = P.schedule == SCHED_RANDOM_PERM;
     uint32_t phases = 0;
     for (int p = 0; p < nph; ++p)
         for (int s = 0; s < ns; ++s)
-            if ((int)((setcol >> (4 * s)) & 15u) == fixed_colour(P.schedule, p)) phases |= 1u << p;
+            if (perm || (int)((setcol >> (4 * s)) & 15u) == fixed_colour(P.schedule, p)) phases |= 1u << p;
     if (fuse) phases &= ~(1u << 4);
     uint32_t rec = 0;                     // records completed by whole schedules
     int32_t until = P.obs_every;          // schedules left before the next one
@@ -722,27 +724,37 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
         const uint32_t n32 = (uint32_t)nl;
         const bool ends = P.obs_every > 0 && !P.obs_pass && until == 1; // a record follows this schedule
         const bool join = fuse && !ends && nl + 1 < P.n_sched;
+        const uint64_t n = (uint64_t)P.sched_begin + (uint64_t)nl;
+        uint32_t orders = 0; // of the sets' replicas, a byte each
+        if (perm)
+            for (int s = 0; s < ns; ++s)
+                orders |= perm_order(u64(domains + (size_t)((wib * ns + s) * DPW) * Q::BYTES, Q::SEED), n) << (8 * s);
         for (uint32_t rest = joined ? phases & ~1u : phases; rest != 0 && ok; rest &= rest - 1) {
             const int p = __ffs((int)rest) - 1;
-            const int colour = fixed_colour(P.schedule, p);
-            // visits of colour c completed before phase p of schedule nl
-            auto before = [&](int c) -> uint32_t {
-                if (!pal) return n32 + (p > c ? 1u : 0u);
-                if (!fuse) return 2 * n32 + (p > c ? 1u : 0u) + (p > 7 - c ? 1u : 0u);
-                if (c == 0) return n32 + rec + (p > 0 ? 1u : 0u);
-                if (c == 3) return n32 + (p > 3 ? 1u : 0u);
-                return 2 * n32 + (p > c ? 1u : 0u) + (p > 7 - c ? 1u : 0u);
-            };
             const int nf = (fuse && (p == 3 || (p == 7 && join))) ? 2 : 1;
-            // a neighbour across a row has colour ^ 2, across a column colour ^ 1
-            const uint32_t needNS = before(colour ^ 2) + (uint32_t)P.debug_extra;
-            const uint32_t needWE = before(colour ^ 1) + (uint32_t)P.debug_extra;
-            const uint32_t after = before(colour) + 1;
             // the visit's changes belong to the first record at or after its pass
             const int64_t o = P.obs_pass ? (nl * nph + p) / P.obs_every : (int64_t)rec;
-            for (int s = 0; s < ns && ok; ++s)
-                if ((int)((setcol >> (4 * s)) & 15u) == colour)
-                    visit(s, ((uint64_t)P.sched_begin + (uint64_t)nl) * 8 + (uint64_t)p, nf, needNS, needWE, after, o);
+            for (int s = 0; s < ns && ok; ++s) {
+                const int colour = (int)((setcol >> (4 * s)) & 15u);
+                const uint32_t order = (orders >> (8 * s)) & 0xFFu;
+                if (colour != (perm ? (int)((order >> (2 * p)) & 3u) : fixed_colour(P.schedule, p))) continue;
+                // visits of colour c completed before phase p of schedule nl
+                auto before = [&](int c) -> uint32_t {
+                    if (perm) {
+                        const uint32_t twice = (uint32_t)c * 0x55u, hit = ~(order ^ twice), // both bits set where order holds c
+                            at = hit & (hit >> 1) & 0x55u;
+                        return n32 + ((at & ((1u << (2 * p)) - 1u)) ? 1u : 0u);
+                    }
+                    if (!pal) return n32 + (p > c ? 1u : 0u);
+                    if (!fuse) return 2 * n32 + (p > c ? 1u : 0u) + (p > 7 - c ? 1u : 0u);
+                    if (c == 0) return n32 + rec + (p > 0 ? 1u : 0u);
+                    if (c == 3) return n32 + (p > 3 ? 1u : 0u);
+                    return 2 * n32 + (p > c ? 1u : 0u) + (p > 7 - c ? 1u : 0u);
+                };
+                // a neighbour across a row has colour ^ 2, across a column colour ^ 1
+                visit(s, n * 8 + (uint64_t)p, nf, before(colour ^ 2) + (uint32_t)P.debug_extra,
+                      before(colour ^ 1) + (uint32_t)P.debug_extra, before(colour) + 1, o);
+            }
         }
         joined = join;
         if (P.obs_every > 0 && !P.obs_pass && --until == 0) {

@@ -881,6 +881,15 @@ __device__ __forceinline__ int perm_colour(uint64_t seed, uint64_t n, int p)
     return colour;
 }
 
+// The four colours of schedule n in that order, two bits each (first lowest).
+__device__ __forceinline__ uint32_t perm_order(uint64_t seed, uint64_t n)
+{
+    uint32_t order = 0;
+#pragma unroll
+    for (int p = 0; p < 4; ++p) order |= (uint32_t)perm_colour(seed, n, p) << (2 * p);
+    return order;
+}
+
 __device__ __forceinline__ int fixed_colour(int schedule, int p)
 {
     if (schedule == SCHED_PALINDROME) return (p < 4) ? p : 7 - p;

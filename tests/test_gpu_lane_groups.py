@@ -66,3 +66,57 @@ def test_lane_groups_equal_the_warp_kernel(L, Ld, ks, mode):
         np.testing.assert_allclose(got[3], want[3], rtol=1e-12, atol=0)
         assert np.array_equal(got[4][..., :3], want[4][..., :3])
         np.testing.assert_allclose(got[4][..., 3], want[4][..., 3], rtol=1e-12, atol=0)
+
+
+@pytest.mark.parametrize("L,Ld,ks", [
+    ([32, 96, 64], 16, [3, 1, 40]),   # 16 lanes
+    ([256, 192, 256], 16, [9, 8, 16]),  # two sets per warp, of different replicas
+    ([64, 192], 32, [4, 9]),          # 32 lanes
+    ([2048], 32, [9]),                # 8 lanes
+    ([128, 256], 64, [5, 20]),        # 32 lanes, 64 columns
+])
+@pytest.mark.parametrize("per_pass,time_mode", [(False, 0), (True, 1)])
+def test_random_orders_equal_the_warp_kernel(L, Ld, ks, per_pass, time_mode):
+    """Each replica's own order of the colours, run after run, on the grid of
+    lane groups that a random-order run takes by itself."""
+    args = dict(time_mode=time_mode, schedule=2, per_pass=per_pass, interleave_init=True)
+    n = [4, 3]
+    want = _run(L, Ld, ks, (GRID, 152, 8), n, **args)
+    got = _run(L, Ld, ks, None, n, **args)
+    assert got[-1][0] == GRID
+    assert np.array_equal(got[0], want[0]) and np.array_equal(got[1], want[1]) and np.array_equal(got[2], want[2])
+    np.testing.assert_allclose(got[3], want[3], rtol=1e-12, atol=0)
+    assert np.array_equal(got[4][..., :3], want[4][..., :3])
+    np.testing.assert_allclose(got[4][..., 3], want[4][..., 3], rtol=1e-12, atol=0)
+
+
+def test_fixed_time_and_scores_after_a_random_order():
+    """A fixed-time run (also captured in a graph) and scores after a
+    random-order run leave the lane groups for a kernel that has them."""
+    import torch
+    import paper_1403_4674_gb300 as kmc
+    out = []
+    for plan in (None, (GRID, 152, 8)):
+        lat = kmc.Lattice([64, 96], 16, 8, [5, 6])
+        if plan:
+            lat.set_launch(*plan)
+        lat.set_rates([0.4, 0.3], [0.01, 0.0])
+        lat.run(2, schedule=kmc.KMC_SCHEDULE_RANDOM_PERM)
+        lat.set_horizon(0.02)
+        g = torch.cuda.CUDAGraph()
+        side = torch.cuda.Stream()
+        side.wait_stream(torch.cuda.current_stream())
+        with torch.cuda.stream(side):
+            with torch.cuda.graph(g, stream=side):
+                lat.run(2, time_mode=kmc.KMC_TIME_HORIZON)
+        torch.cuda.current_stream().wait_stream(side)
+        g.replay()
+        torch.cuda.synchronize()
+        lat.run(2, schedule=kmc.KMC_SCHEDULE_RANDOM_PERM)
+        lat.enable_grad(True)
+        lat.run(2)
+        lat.sync()
+        out.append((lat.spins.cpu().numpy(), *lat.domain_state()[:2]))
+        lat.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
