@@ -567,16 +567,23 @@ kmc_status plan_threads(kmc_ctx *c, int n_cta, int wpb, Plan &pl)
 using TpdKernel = void (*)(const RunParams);
 // the thread-per-domain kernel of the context's domain side (scores: the
 // shared-memory kernel of 16x16 and 32x32 domains only)
-TpdKernel tpd_kernel_for(int LD, bool expo, bool grad)
+// (scores: NO_SCORES, SCORES_AFTER or SCORES_INLINE)
+TpdKernel tpd_kernel_for(int LD, bool expo, int scores)
 {
     if (LD == 64) return expo ? tpdr64_kernel<true> : tpdr64_kernel<false>;
-    if (LD == 16)
-        return grad ? (expo ? tpdr_kernel<16, true, true> : tpdr_kernel<16, false, true>)
-                    : (expo ? tpdr_kernel<16, true, false> : tpdr_kernel<16, false, false>);
-    if (LD == 32)
-        return grad ? (expo ? tpdr_kernel<32, true, true> : tpdr_kernel<32, false, true>)
-                    : (expo ? tpdr_kernel<32, true, false> : tpdr_kernel<32, false, false>);
+#define KMC_TPDR(LDV, SV) \
+    if (LD == LDV && scores == SV) return expo ? tpdr_kernel<LDV, true, SV> : tpdr_kernel<LDV, false, SV>;
+    KMC_TPDR(16, NO_SCORES) KMC_TPDR(16, SCORES_AFTER) KMC_TPDR(16, SCORES_INLINE)
+    KMC_TPDR(32, NO_SCORES) KMC_TPDR(32, SCORES_AFTER) KMC_TPDR(32, SCORES_INLINE)
+#undef KMC_TPDR
     return expo ? tpd_kernel<true> : tpd_kernel<false>;
+}
+// Scores are worked off after a visit whose lists hold it: at most 32 steps,
+// two fused phases of 16.
+int scores_of(const kmc_ctx *c)
+{
+    if (!c->grad) return NO_SCORES;
+    return *std::max_element(c->kr.begin(), c->kr.end()) <= 16 ? SCORES_AFTER : SCORES_INLINE;
 }
 // the lane-group kernel of a domain side and G lanes per domain
 TpdKernel grp_kernel_for(int LD, int G, bool expo)
@@ -595,9 +602,9 @@ size_t grp_domain_bytes_for(int LD, int G)
     if (LD == 32) return G == 8 ? grp_domain_bytes<32, 8>() : G == 16 ? grp_domain_bytes<32, 16>() : grp_domain_bytes<32, 32>();
     return G == 16 ? grp_domain_bytes<64, 16>() : grp_domain_bytes<64, 32>();
 }
-TpdKernel thread_plan_kernel(const Plan &pl, int LD, bool expo, bool grad)
+TpdKernel thread_plan_kernel(const kmc_ctx *c, const Plan &pl, bool expo)
 {
-    return pl.groups ? grp_kernel_for(LD, pl.groups, expo) : tpd_kernel_for(LD, expo, grad);
+    return pl.groups ? grp_kernel_for(c->LD, pl.groups, expo) : tpd_kernel_for(c->LD, expo, scores_of(c));
 }
 size_t tpdr_warp_bytes_for(int LD)
 {
@@ -819,7 +826,7 @@ kmc_status check_plan(kmc_ctx *c, const Plan &pl)
             return fail(c, KMC_EINVAL, "the thread-per-domain plan of L_d = %d has no score kernel", c->LD);
         if (c->grad && pl.groups) return fail(c, KMC_EINVAL, "the lane-group kernel carries no scores");
         for (int e = 0; e < 2; ++e) {
-            const void *kern = (const void *)thread_plan_kernel(pl, c->LD, e == 0, c->grad);
+            const void *kern = (const void *)thread_plan_kernel(c, pl, e == 0);
             if (pl.smem > 0) {
                 if (pl.smem > (size_t)c->smem_optin)
                     return fail(c, KMC_EINVAL, "thread plan needs %zu bytes of shared memory per CTA (%d available)",
@@ -1772,7 +1779,7 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     const Plan &pl = c->plan;
     const bool cluster = pl.mode == KMC_LAUNCH_CLUSTER;
     const bool threads = pl.mode == KMC_LAUNCH_THREADS || pl.groups;
-    RunKernel kern = threads ? thread_plan_kernel(pl, c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad)
+    RunKernel kern = threads ? thread_plan_kernel(c, pl, time_mode == KMC_TIME_EXPONENTIAL)
                              : run_kernel_for(c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad, cluster);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     const bool prof = c->prof && !cap;

@@ -39,10 +39,15 @@
 
 namespace kmcdev {
 
-template <int LD> struct TpdrLayout {
+// What a kernel does about path scores: nothing; work them off after the
+// visit's edges are published (visits of up to 32 steps); form them event by
+// event.
+constexpr int NO_SCORES = 0, SCORES_AFTER = 1, SCORES_INLINE = 2;
+
+template <int LD, int SCORES> struct TpdrLayout {
     static_assert(LD == 16 || LD == 32, "rows of at most 32 sites");
     static constexpr int NB = LD / 8;  // blocks of 8 rows
-    static constexpr int CHUNK = 32;   // steps drawn at a time
+    static constexpr int CHUNK = SCORES == SCORES_AFTER ? 16 : 32; // steps drawn at a time (the states before the chunk's events need the room)
     static constexpr uint32_t FULL = (LD == 32) ? 0xFFFFFFFFu : ((1u << LD) - 1u);
     // 64-bit words per lane: row counts lo / hi, block counts lo / hi (one
     // spare block each, the target of updates that have no second block),
@@ -52,13 +57,13 @@ template <int LD> struct TpdrLayout {
     // those of the open record (FP64 bits), 0 and the cumulative class rates
     // C_c, acceptances A_c, their reciprocals floor((2^64 - 1) / A_c), the
     // step targets of the current chunk (eight spare words past its end hold
-    // ~0, a target no rate sum reaches, so that a scan of eight never reads
-    // past them)
+    // ~0, a target no rate sum reaches, so that a look at eight never reads past
+    // them); for scores the domain's counts before each event of the chunk
     static constexpr int ROWLO = 0, ROWHI = LD, BLKLO = 2 * LD, BLKHI = BLKLO + NB + 1, TOTLO = BLKHI + NB + 1,
                          TOTHI = TOTLO + 1, CH = TOTLO + 2, CFL = CH + 1, CST = CH + 2, CCM = CH + 3, CCE = CH + 4,
                          OB0 = CH + 5, OB1 = OB0 + 1, OBM = OB0 + 2, OBE = OB0 + 3, CSB = OB0 + 4, CSH = CSB + 1,
                          OSB = CSB + 2, OSH = CSB + 3, CC = CSB + 4, AT = CC + 11, MR = AT + 10, TG = MR + 10,
-                         N64 = TG + CHUNK + 8;
+                         SN = TG + CHUNK + 8, N64 = SN + (SCORES == SCORES_AFTER ? 2 * CHUNK : 0);
     // 32-bit words per lane: spin rows, the halo the counts hold (N row, S
     // row, W column, E column), the domain's W and E columns, neighbour ids,
     // the events of the chunk (step | class << 5 | site << 9)
@@ -67,7 +72,13 @@ template <int LD> struct TpdrLayout {
     static constexpr int WARP_BYTES = 32 * (8 * N64 + 4 * N32);
 };
 
-template <int LD> __host__ __device__ constexpr int tpdr_warp_bytes() { return TpdrLayout<LD>::WARP_BYTES; }
+// (one size with and without scores, so that a plan serves both)
+template <int LD> __host__ __device__ constexpr int tpdr_warp_bytes()
+{
+    return TpdrLayout<LD, SCORES_AFTER>::WARP_BYTES > TpdrLayout<LD, NO_SCORES>::WARP_BYTES
+               ? TpdrLayout<LD, SCORES_AFTER>::WARP_BYTES
+               : TpdrLayout<LD, NO_SCORES>::WARP_BYTES;
+}
 
 // Bit-sliced count (b2 b1 b0) of the up neighbours of every site of row S,
 // with U and D the rows above and below and wb, eb the spins left of column 0
@@ -76,7 +87,7 @@ template <int LD>
 __device__ __forceinline__ void tpdr_planes(uint32_t S, uint32_t U, uint32_t D, uint32_t wb, uint32_t eb,
                                             uint32_t &b0, uint32_t &b1, uint32_t &b2)
 {
-    constexpr uint32_t FULL = TpdrLayout<LD>::FULL;
+    constexpr uint32_t FULL = TpdrLayout<LD, NO_SCORES>::FULL;
     const uint32_t Wn = ((S << 1) | wb) & FULL;       // bit x: the spin at x - 1
     const uint32_t En = (S >> 1) | (eb << (LD - 1));  // bit x: the spin at x + 1
     const uint32_t x = U ^ D ^ Wn, m = (U & D) | (U & Wn) | (D & Wn), k = x & En; // U + D + Wn = x + 2 m
@@ -96,7 +107,7 @@ template <int LD>
 __device__ __forceinline__ void tpdr_row_counts(uint32_t S, uint32_t U, uint32_t D, uint32_t wb, uint32_t eb,
                                                 uint64_t &lo, uint64_t &hi)
 {
-    constexpr uint32_t FULL = TpdrLayout<LD>::FULL;
+    constexpr uint32_t FULL = TpdrLayout<LD, NO_SCORES>::FULL;
     uint32_t b0, b1, b2;
     tpdr_planes<LD>(S, U, D, wb, eb, b0, b1, b2);
     lo = 0;
@@ -138,10 +149,11 @@ __device__ __forceinline__ int tpdr_select(uint32_t w, uint32_t rr)
 // Persistent kernel.  P.slot_g holds 32 domain ids per warp of the grid (one
 // colour per warp, 0xFFFFFFFF for an empty lane); the dynamic shared memory
 // holds a TpdrLayout region per warp.
-template <int LD, bool EXPO, bool GRAD>
+template <int LD, bool EXPO, int SCORES>
 __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
 {
-    using Lay = TpdrLayout<LD>;
+    constexpr bool GRAD = SCORES != NO_SCORES;
+    using Lay = TpdrLayout<LD, SCORES>;
     constexpr int NB = Lay::NB;
     constexpr int CHUNK = Lay::CHUNK;
     constexpr uint32_t FULL = Lay::FULL;
@@ -149,7 +161,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
     const int lane = threadIdx.x & 31;
     const int wib = threadIdx.x >> 5;
     const int wg = blockIdx.x * (blockDim.x >> 5) + wib;
-    uint64_t *w64 = reinterpret_cast<uint64_t *>(smem + (size_t)wib * Lay::WARP_BYTES);
+    uint64_t *w64 = reinterpret_cast<uint64_t *>(smem + (size_t)wib * tpdr_warp_bytes<LD>());
     uint32_t *w32 = reinterpret_cast<uint32_t *>(w64 + 32 * Lay::N64);
     auto at = [&](int i) -> uint64_t & { return w64[i * 32 + lane]; };
     auto at32 = [&](int i) -> uint32_t & { return w32[i * 32 + lane]; };
@@ -461,28 +473,6 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                 uint32_t colW = at32(Lay::CW), colE = at32(Lay::CE);
                 uint32_t ne = 0, flips = 0; // events of the chunk, of the visit
                 int dbonds = 0, dmag = 0;
-                // What the events add to the event hash, the bond sum and the
-                // magnetisation is worked off from the list of the chunk's events,
-                // after the visit's edges are published: the neighbours do not
-                // wait for it.
-                auto work_off = [&](int base) {
-                    const int most = (int)__reduce_max_sync(FULL_WARP, ne);
-                    for (int i = 0; i < most; ++i) {
-                        const uint32_t e = at32(Lay::EV + i);
-                        const int st = base + (int)(e & 31u), c = (int)((e >> 5) & 15u), f = st >= k ? 1 : 0;
-                        const uint64_t np = np0 + (uint64_t)f;
-                        const uint64_t h = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)(e >> 9))) * HASH_PRIME;
-                        const bool act = i < (int)ne;
-                        H = act ? h : H;
-                        // flipping spin s with neighbour sum 2 q - 4 changes the bond
-                        // sum by -2 s (2 q - 4) and the magnetisation by -2 s
-                        const int g2 = act ? (c < 5 ? 2 : -2) : 0;
-                        dbonds += g2 * (2 * (c < 5 ? c : c - 5) - 4);
-                        dmag += g2;
-                    }
-                    flips += ne;
-                    ne = 0;
-                };
 
                 // Path score of the visit (scores only): a real event of class c
                 // adds dlog a_c, a null step dlog(1 - R/n_d) = -sum_c n_c a_c
@@ -493,24 +483,27 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                 // the exact rate sum as (2^63 - R') 2^-P; its reciprocal from the
                 // FP32 one x0 = (1 - e)/g by x0 (1 + e + e^2) = (1 - e^3)/g
                 // (|e| < 2^-21: truncation 2^-63).  Terms are added in step
-                // order, a null run split at the 32-step chunk boundaries.
-                double sb = 0.0, sh = 0.0, nbo = 0.0, nho = 0.0;
-                bool scored = false;
-                auto grad_state = [&]() {
+                // order, a null run split at multiples of 32 steps.
+                double sb = 0.0, sh = 0.0;
+                int pos = 0; // first step of the current run of null steps, relative to the chunk
+                double nbo = 0.0, nho = 0.0;
+                auto score_state = [&](uint64_t lo, uint64_t hi) { // a null step in the state with these counts
                     int64_t xb = 0, xh = 0;
                     int yb = 0, yh = 0;
+                    uint64_t R = (SCORES == SCORES_INLINE) ? C[9] : 0;
 #pragma unroll
                     for (int c = 0; c < 10; ++c) {
-                        const uint32_t n = tpdr_field(c < 5 ? tlo : thi, 12 * (c % 5));
+                        const uint32_t n = tpdr_field(c < 5 ? lo : hi, 12 * (c % 5));
                         xb += (int64_t)n * Xb[c];
                         xh += (int64_t)n * Xh[c];
                         yb += (int)n * Yb[c];
                         yh += (int)n * Yh[c];
+                        if (SCORES != SCORES_INLINE) R += (uint64_t)n * A[c];
                     }
                     constexpr int SH = GFIX_LO_BITS - GFIX_T_BITS;
                     const int64_t tb = xb * (1ll << GFIX_T_BITS) + (int64_t)((yb + (1 << (SH - 1))) >> SH);
                     const int64_t th = xh * (1ll << GFIX_T_BITS) + (int64_t)((yh + (1 << (SH - 1))) >> SH);
-                    const uint64_t gap = (1ull << 63) - C[9];
+                    const uint64_t gap = (1ull << 63) - R;
                     const double gd = __ull2double_rn(gap);
                     const double x0 = (double)__frcp_rn(u64_to_float_rz(gap));
                     const double e = __fma_rn(-gd, x0, 1.0);
@@ -518,26 +511,82 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                     const double w = inv * scaleP;
                     nbo = (double)tb * w;
                     nho = (double)th * w;
-                    scored = true;
+                };
+                auto null_steps = [&](int n) { // n of them in the scored state
+                    const double q = (double)n;
+                    sb -= q * nbo;
+                    sh -= q * nho;
+                };
+
+                // What the events add to the event hash, the bond sum, the
+                // magnetisation and the scores is worked off from the list of the
+                // chunk's events (with scores also the counts before each), after
+                // the visit's edges are published: the neighbours do not wait for
+                // it.  With scores this is most of a visit's work: 256 x 256^2,
+                // 100 schedules, k = 8 7.43 -> 4.11 ms, k = 2 6.09 -> 3.89, k = 16
+                // 12.1 -> 9.7.  Visits of more than 32 steps (k = 33: 24 % slower
+                // with lists of 16 steps, and longer ones do not fit) form their
+                // scores event by event.
+                auto work_off = [&](int base) {
+                    const int most = (int)__reduce_max_sync(FULL_WARP, ne);
+                    for (int i = 0; i < most; ++i) {
+                        const uint32_t e = at32(Lay::EV + i);
+                        const int ist = (int)(e & 31u), st = base + ist, c = (int)((e >> 5) & 15u), f = st >= k ? 1 : 0;
+                        const uint64_t np = np0 + (uint64_t)f;
+                        const uint64_t h = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)(e >> 9))) * HASH_PRIME;
+                        const bool act = i < (int)ne;
+                        H = act ? h : H;
+                        // flipping spin s with neighbour sum 2 q - 4 changes the bond
+                        // sum by -2 s (2 q - 4) and the magnetisation by -2 s
+                        const int g2 = act ? (c < 5 ? 2 : -2) : 0;
+                        dbonds += g2 * (2 * (c < 5 ? c : c - 5) - 4);
+                        dmag += g2;
+                        if (SCORES == SCORES_AFTER && act) {
+                            if (ist > pos) {
+                                score_state(at(Lay::SN + 2 * i), at(Lay::SN + 2 * i + 1));
+                                null_steps(ist - pos);
+                            }
+                            // dlog a_c / d(beta, h) of the chosen class
+                            sb += __ldg(gr + 10 + c);
+                            sh += __ldg(gr + 20 + c);
+                            pos = ist + 1;
+                        }
+                    }
+                    if (SCORES == SCORES_AFTER) {
+                        // the null steps after the last event: up to the visit's end or a
+                        // multiple of 32 steps; else the run goes on in the next chunk
+                        const int end = min(CHUNK, total - base);
+                        if (base + CHUNK >= total || ((base + CHUNK) & 31) == 0) {
+                            if (end > pos) {
+                                score_state(tlo, thi);
+                                null_steps(end - pos);
+                            }
+                            pos = CHUNK;
+                        }
+                        pos -= CHUNK;
+                    }
+                    flips += ne;
+                    ne = 0;
                 };
 
                 bool corrupt = false; // counts and spins disagreed at some event
                 for (int base = 0; base < smax; base += CHUNK) {
                     if (base > 0) {
-                        work_off(base - CHUNK);
+                        if (SCORES != SCORES_INLINE) work_off(base - CHUNK);
                         draw(base);
                     }
                     // Each lane jumps from real event to real event of its own
                     // domain (the steps between are null: App. A, the diagonal
                     // 1 - R/n_d); the warp runs as many rounds as its busiest lane.
-                    int i = 0;   // this lane's next step, relative to the chunk
-                    int pos = 0; // first step of the current run of null steps (scores)
+                    int i = 0; // this lane's next step, relative to the chunk
+                    bool scored = false; // nbo, nho belong to the current state
+                    if (SCORES == SCORES_INLINE) pos = 0;
                     while (true) {
                         // the lane's next step with target < R' (targets past its
                         // last step are ~0)
                         uint64_t tgt = 0;
                         bool ev = false;
-                        if (GRAD) {
+                        if (SCORES == SCORES_INLINE) {
                             // every round in which some lane's state is scored costs
                             // FP64 time, so the lanes look on until each has an event
                             while (i < CHUNK) {
@@ -563,6 +612,15 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                                 i += 8;
                             }
                             ev = i < CHUNK;
+                            // the null steps before this event, or up to the chunk's
+                            // (or the visit's) end, all in the current state
+                            const int end = ev ? i : min(CHUNK, total - base);
+                            if (end > pos) {
+                                if (!scored) score_state(tlo, thi);
+                                scored = true;
+                                null_steps(end - pos);
+                            }
+                            pos = ev ? i + 1 : CHUNK;
                         } else if (i < CHUNK) {
                             // One look at four steps per round: a lane that finds none
                             // in them sits out this round's events, as the lane with
@@ -584,18 +642,6 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                             const uint64_t q0 = (f & 1) ? t[1] : t[0], q1 = (f & 1) ? t[3] : t[2];
                             tgt = (f & 2) ? q1 : q0;
                         }
-                        if (GRAD) {
-                            // the null steps before this event, or up to the chunk's
-                            // (or the visit's) end, all in the current state
-                            const int end = ev ? i : min(CHUNK, total - base);
-                            if (end > pos) {
-                                if (!scored) grad_state();
-                                const double q = (double)(end - pos);
-                                sb -= q * nbo;
-                                sh -= q * nho;
-                            }
-                            pos = ev ? i + 1 : CHUNK;
-                        }
                         if (!__any_sync(FULL_WARP, ev || i < CHUNK)) break;
                         if (!ev) continue;
                         const int ist = i; // the event's step in the chunk
@@ -606,10 +652,14 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                         for (int cc = 0; cc < 9; ++cc) c += (tgt >= C[cc]) ? 1 : 0;
                         const uint64_t Cprev = at(Lay::CC + c); // C_{c-1}, 0 for c = 0
                         const uint64_t Ac = at(Lay::AT + c), Mc = at(Lay::MR + c);
-                        if (GRAD) {
-                            // dlog a_c / d(beta, h) of the chosen class
+                        if (SCORES == SCORES_AFTER) {
+                            at(Lay::SN + 2 * (int)ne) = tlo;
+                            at(Lay::SN + 2 * (int)ne + 1) = thi;
+                        }
+                        if (SCORES == SCORES_INLINE) {
                             sb += __ldg(gr + 10 + c);
                             sh += __ldg(gr + 20 + c);
+                            scored = false;
                         }
                         // exact jj = floor((tgt - C_{c-1}) / A_c) < n_c <= 1024: with
                         // M_c = floor((2^64 - 1) / A_c) and x < 2^63, the high word
@@ -743,10 +793,18 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                         thi += dYhi + dNhi + dShi;
                         colW ^= (col == 0) ? (1u << y) : 0u;
                         colE ^= (col == LD - 1) ? (1u << y) : 0u;
-                        at32(Lay::EV + (int)ne) = (uint32_t)ist | ((uint32_t)c << 5) | ((uint32_t)(y * LD + col) << 9);
-                        ++ne;
+                        if (SCORES == SCORES_INLINE) {
+                            const int st = base + ist, f = st >= k ? 1 : 0;
+                            const uint64_t np = np0 + (uint64_t)f;
+                            H = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)(y * LD + col))) * HASH_PRIME;
+                            ++flips;
+                            dbonds += (up ? -2 : 2) * (2 * qc - 4);
+                            dmag += up ? -2 : 2;
+                        } else {
+                            at32(Lay::EV + (int)ne) = (uint32_t)ist | ((uint32_t)c << 5) | ((uint32_t)(y * LD + col) << 9);
+                            ++ne;
+                        }
                         rates();
-                        scored = false;
                         corrupt |= bad;
                     }
                 }
@@ -760,7 +818,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                     st_cg(ew + 2 * EDGE_W, cnt | colW);
                     st_cg(ew + 2 * EDGE_E, cnt | colE);
                 }
-                work_off((smax - 1) / CHUNK * CHUNK);
+                if (SCORES != SCORES_INLINE) work_off((smax - 1) / CHUNK * CHUNK);
                 // the visit's changes belong to the first record at or after its pass
                 const int64_t o = P.n_obs > 0 ? (P.obs_pass ? pass : pass / nph) / P.obs_every : 0;
                 if (P.n_obs > 0 && __any_sync(FULL_WARP, has && (int64_t)(uint32_t)at(Lay::OB0) != o))

@@ -120,3 +120,30 @@ def test_fixed_time_and_scores_after_a_random_order():
         lat.close()
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("Ld,ks", [(32, [2, 8, 5]), (32, [16, 9, 1]), (16, [17, 3, 16]), (32, [16, 33, 40]), (16, [8, 16, 12])])
+@pytest.mark.parametrize("per_pass", [False, True])
+def test_scores_after_the_visit_equal_the_warp_kernels(Ld, ks, per_pass):
+    """Scores worked off after a visit's edges (k <= 16: lists of 16 steps, a
+    null run going on past a list's end unless at a multiple of 32 steps) or
+    event by event (longer visits): the same terms in the same order as the
+    warp kernel's, hence the same numbers."""
+    import paper_1403_4674_gb300 as kmc
+    L, out = [4 * Ld, 8 * Ld, 2 * Ld], []
+    for plan in ((THREADS, 0, 4), (GRID, 152, 8)):
+        lat = kmc.Lattice(L, Ld, 1, [41, 42, 43])
+        lat.set_replica_params(k=ks)
+        lat.set_launch(*plan)
+        lat.enable_grad(True)
+        lat.set_rates([0.42, 0.35, 0.5], [0.02, 0.01, -0.02])
+        if per_pass:
+            lat.set_observation(kmc.KMC_OBS_PASS)
+        obs = np.concatenate([lat.run(n, obs_every=3).cpu().numpy() for n in (7, 8)])
+        assert lat.launch()[0] == plan[0]
+        out.append((lat.spins.cpu().numpy(), lat.score().cpu().numpy(), obs))
+        lat.close()
+    (s0, g0, o0), (s1, g1, o1) = out
+    assert np.array_equal(s0, s1) and np.array_equal(g0, g1)
+    assert np.array_equal(o0[..., :3], o1[..., :3])
+    np.testing.assert_allclose(o0[..., 4:6], o1[..., 4:6], rtol=1e-12, atol=1e-12)
