@@ -332,7 +332,7 @@ kmc_status kmc_rate_table_error(const kmc_ctx *ctx, double *max_rel_err);
  *   KMC_LAUNCH_AUTO: the library's choice: KMC_LAUNCH_THREADS for L_d = 16
  *     and 32 when the domains' state fits the GPU's shared memory, for L_d =
  *     64 when it fits and scores are off, and for L_d = 8 while scores are
- *     off; otherwise CLUSTER when every replica
+ *     off (random colour orders: below); otherwise CLUSTER when every replica
  *     fits one cluster of at most 16 CTAs at one visit per warp and phase,
  *     else a cooperative GRID (the shape with the most resident warps per SM
  *     that fits: three CTAs of 8 warps, two of 12 or 10, one of 16, ...),
@@ -346,16 +346,23 @@ kmc_status kmc_rate_table_error(const kmc_ctx *ctx, double *max_rel_err);
  *     neighbour domain is in the same CTA.  The run kernels hold 80 to 128
  *     registers per thread (by domain side and scores), so two or three CTAs
  *     of 8-12 warps can share an SM.
- *   KMC_LAUNCH_THREADS (L_d = 8, 16, 32 or 64): one thread runs a whole
- *     domain process and a warp 32 of them at once, with no warp collective
- *     on the step path; warps_per_cta 1..4.
- *     L_d = 8: a cooperative grid of `size` CTAs (0: as many as spread each
- *     colour's domains evenly over at most three 4-warp CTAs per SM), thread
- *     t visiting the t-th, (t+T)-th, ... domain of each colour's list (T the
+ *   KMC_LAUNCH_THREADS (L_d = 8, 16, 32 or 64): a warp runs several domain
+ *     processes at once; warps_per_cta 1..4.
+ *     L_d = 8: one thread per domain visit, a cooperative grid of `size` CTAs
+ *     (0: three 4-warp CTAs per SM when their last round of a colour's
+ *     domains is at least half full, else as many as spread each colour's
+ *     domains evenly over the rounds), thread t visiting the t-th, (t+T)-th, ... domain of each colour's list (T the
  *     grid's threads); an 8x8 domain is one 64-bit word, so the domain
  *     process runs in registers, with state, edge words and counters in
  *     global memory (L2).
- *     L_d = 16, 32, 64: one domain per thread for the whole launch, a warp
+ *     L_d = 16, 32, 64 with few domains (about two warps per scheduler at 8
+ *     or more lanes per domain: 128 to 8192 domains on 152 SMs; scores off):
+ *     8, 16 or 32 lanes per domain, by how many fill the SMs, the domain in
+ *     the CTA's shared memory (0.8 to 2.3 KB); warps_per_cta as given, under
+ *     KMC_LAUNCH_AUTO a whole replica per CTA where 16 warps hold it, else 4.
+ *     `size` as below.
+ *     L_d = 16, 32, 64 otherwise: one domain per thread for the whole launch,
+ *     with no warp collective on the step path, a warp
  *     holding 32 domains of one colour; the domain's rows, the class counts
  *     of every row (not at L_d = 64, where an event counts the 8 rows of
  *     its block from their spins), of every block of 8 rows and of the
@@ -369,11 +376,17 @@ kmc_status kmc_rate_table_error(const kmc_ctx *ctx, double *max_rel_err);
  *     steps per visit or temperature, slower on a batch of alike replicas);
  *     other values KMC_EINVAL.
  *     All cover the palindromic and fixed schedules with the exponential or
- *     expected clock, and the L_d = 16, 32 kernel also path scores
- *     (kmc_enable_grad; each thread forms its own domain's FP64 score
- *     terms); a run that needs fixed-time visits, random colour orders or,
- *     at L_d = 8 or 64, scores first replaces the plan by the library's
- *     choice among the others (KMC_EINVAL while the stream is capturing).
+ *     expected clock, and one thread per domain of L_d = 16, 32 also path
+ *     scores (kmc_enable_grad; each thread forms its own domain's FP64 score
+ *     terms, after the visit's edges are published when no replica has more
+ *     than 16 steps per visit, else event by event).  A run that needs
+ *     fixed-time visits, random colour orders or, at L_d = 8 or 64, scores
+ *     first replaces the plan by the library's choice among the others
+ *     (KMC_EINVAL while the stream is capturing).  For random colour orders
+ *     of L_d = 16, 32, 64 without scores that is a GRID of lane groups where
+ *     the domains are few, as above; the one-warp-per-domain plan stays
+ *     beside it and is taken again by a run with fixed-time visits, also
+ *     while the stream is capturing.
  * In all plans a visit starts as soon as its four neighbours have finished
  * their visits of earlier colour phases (per-domain dataflow instead of a
  * barrier per phase; Sec. 2.2 lets non-interacting domains run at once); observation records are built from per-visit changes,
@@ -381,9 +394,10 @@ kmc_status kmc_rate_table_error(const kmc_ctx *ctx, double *max_rel_err);
  * warps_per_cta: 1..16.  Returns KMC_EINVAL if the plan cannot be scheduled
  * or the state does not fit in shared memory; the previous plan then stays.
  * Results do not depend on the plan, except the last bits of the FP64 domain
- * clocks: the thread plan multiplies a visit's clock variates in step order,
- * the others in pairs (both within 1e-12 of the oracle).  Path scores are
- * the same on every plan (the same terms in the same order per domain). */
+ * clocks: the plans multiply a visit's clock variates in different orders
+ * (one thread per domain: in step order; lane groups: each lane its own steps;
+ * one warp per domain: in pairs; all within 1e-12 of the oracle).  Path scores
+ * are the same on every plan (the same terms in the same order per domain). */
 enum { KMC_LAUNCH_AUTO = 0, KMC_LAUNCH_CLUSTER = 1, KMC_LAUNCH_GRID = 2, KMC_LAUNCH_THREADS = 3 };
 kmc_status kmc_set_launch(kmc_ctx *ctx, int32_t mode, int32_t size, int32_t warps_per_cta);
 /* Current plan: mode, size (cluster size or CTA count), CTAs, warps per CTA,
@@ -415,8 +429,9 @@ kmc_status kmc_profile_read(kmc_ctx *ctx, double *run_kernel_ms, int64_t *run_ke
  * warps of the times a warp re-read a neighbour's edge word because the
  * neighbour had not finished its earlier visit yet (the first read of a halo
  * is not counted; a warp polling several neighbours at once counts its
- * slowest lane; under KMC_LAUNCH_THREADS at L_d = 8 the sum over threads,
- * at 16 and 32 the sum over warps of their poll rounds).  With instructions per poll iteration this separates
+ * slowest lane; one thread per domain: at L_d = 8 the sum over threads,
+ * at 16, 32 and 64 the sum over warps of their poll rounds; lane groups: the
+ * sum over warps of their poll rounds).  With instructions per poll iteration this separates
  * busy-waiting from the visits' own instructions.  *polls is a host int64;
  * reading synchronises the context's stream and clears the count.  0 when
  * profiling was never enabled.  KMC_EINVAL for null arguments.  No

@@ -387,7 +387,7 @@ class Lattice:
 
     def set_launch(self, mode: int = KMC_LAUNCH_AUTO, size: int = 0, warps_per_cta: int = 16):
         """Launch plan (kmc_set_launch): size is the cluster size, the grid's
-        CTA count, or for the thread plans of L_d = 16, 32, 64 the domain
+        CTA count, or for KMC_LAUNCH_THREADS at L_d = 16, 32, 64 the domain
         order over the warps (0 or 1 replica after replica, 2 round-robin)."""
         kmc_set_launch(self.ctx, mode, size, warps_per_cta)
 

@@ -7,9 +7,28 @@
 // setting): one warp owns one trajectory for the whole launch and runs its
 // domain processes in schedule order, so the halo of a visit is the live
 // state -- no other domain of the trajectory moves meanwhile.  The lattice
-// lives in shared memory as bit rows (row y: two 64-bit words, bit x =
-// column x, 1 = up).  Lane l holds domain rows l*RPL .. l*RPL+RPL-1
-// (RPL = ceil(H/32)), so a warp scan over lanes runs in row-major order.
+// lives in shared memory as bit rows (PART_ROW32 words each), beside the
+// class counts of every domain and, where they fit, of every domain row; a
+// flip updates the counts of the five sites it touches, whichever domains
+// they lie in, so a visit starts from its counts without a recount.
+//
+// What bounds it is one warp's chain of real events (the paper's 50
+// trajectories leave two SMs of three idle, and a trajectory has no work for
+// a second warp): ncu counts 1.0 warps per scheduler that has any, issue
+// 24 % of its cycles, the stalls led by fixed-latency dependencies.  So the
+// steps of a trajectory are drawn 32 at a time across visits and schedules
+// (a window: one lane per step, whole visits of up to 32 steps each or 32
+// steps of a longer one), null runs cost nothing (the next event of the
+// window is one vote away), and the event's chain is kept short: the class
+// from the cumulative rates in every lane alike, the member's row from
+// 16 domain rows per lane of the rows' counts, its column from a
+// lane-parallel bit count, the five sites' classes from five lanes side by
+// side, the counts by shared-memory atomics.  About 1600 cycles an event
+// remain (rates 240, class 245, row 190-320, column 268, neighbours 143,
+// counts 295).  Measured at the start, after the windows and now: 50
+// trajectories of 100^2 in four stripes, k = 5, random order, 800 schedules
+// 3.22, 1.89, 1.34 ms; 500 of 12^2 in four blocks, k = 1, 4000 schedules
+// 11.1, 5.81, 3.54 ms.
 //
 // Step target (n_d not a power of two): P = 63 - ceil(log2 n_d),
 // M = n_d 2^P, target = floor(X M / 2^64) for X = w0 | w1<<32; with n_d a

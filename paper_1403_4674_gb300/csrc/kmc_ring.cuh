@@ -13,6 +13,17 @@
 // (integers, so their order does not matter) are reduced per warp with
 // ballots and warp reductions and added to global memory with one atomic per
 // warp and quantity.
+//
+// What bounds it: integer issue and the fixed latency between dependent
+// instructions.  48000 trajectories of 8 spins are 2.4 warps per scheduler;
+// ncu counts 49 % of the issue slots used, the ALU pipe 46 % and the multiply
+// pipe 40 % busy, stalls led by fixed-latency waits.  A warp runs the event
+// path whenever one of its 32 trajectories has an event, so a step is kept
+// short rather than skipped: the visit works on a 32-bit window of its domain
+// (below), and the next step's Philox block, which depends on nothing, is
+// drawn in line with the event so that its multiplies fill the event's waits.
+// Measured: 48000 x 8 spins, k = 5, 40 sweeps with ensemble sums 1031 -> 769 us;
+// 6000 x 64 spins, k = 10, 10 sweeps with records 931 -> 736 us.
 #pragma once
 
 #include <cstdint>
