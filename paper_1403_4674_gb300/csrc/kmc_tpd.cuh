@@ -34,9 +34,12 @@ namespace kmcdev {
 
 constexpr uint64_t TPD_COL0 = 0x0101010101010101ull; // column 0 of every row
 constexpr int TPD_CACHE = 2;  // rounds of a phase whose domains a thread keeps in shared memory
+constexpr int TPD_CHUNK = 32; // steps drawn at a time
+constexpr int TPD_LOOK = 3;   // steps looked at in a round of events
 // shared memory of a thread: 0 and the cumulative class rates, domain and
-// replica of its visits
-constexpr int TPD_THREAD_BYTES = 80 + 4 * TPD_CACHE * 8;
+// replica of its visits, the targets of a chunk and past its end ~0 (a target
+// no rate sum reaches), so that a look never reads past them
+constexpr int TPD_THREAD_BYTES = 80 + 4 * TPD_CACHE * 8 + (TPD_CHUNK + TPD_LOOK) * 8;
 constexpr int TPD_OBS_WORDS = 4; // open record per domain: record | steps << 32, bonds | mag << 32, mantissa, exponent
 
 // Bit y of an 8-bit column mask to bit 8y (column 0 of row y).
@@ -143,17 +146,23 @@ __device__ __forceinline__ void tpd_flush(const RunParams &P, bool on, const ulo
 // P.cta_col_off holds the five offsets of the colour-sorted domain list
 // P.slot_g; P.obs_dom the open records (TPD_OBS_WORDS per domain).
 //
-// What bounds it: with the 166 registers of a visit three 4-warp CTAs fit an
-// SM, and three warps per scheduler issue on about half of the cycles, so a
-// visit's latency counts as much as its instructions.  Hence the order of a
-// visit (the domain's words asked for first, then the first draw, then the
-// halo), the next step's draw in one straight line with this step's event,
-// counters added without reading them, and C_{c-1} through shared memory
-// (the integer pipe is the busiest one, 60 %).  512 uneven replicas, 60
-// schedules, records every 10, on 456 CTAs: k = 1 6.1 -> 5.2 ms, k = 4 8.0 ->
-// 7.4, k = 16 19.7 -> 18.4, k = 32 36.2 -> 33.3.  Threads that jump between
-// their own events (targets in shared memory) took 8.5 / 19.3 / 33.7 ms at k
-// = 4 / 16 / 32, four CTAs per SM at 128 registers 7.9 / 19.9 / 36.4.
+// What bounds it: with the registers of a visit three 4-warp CTAs fit an SM,
+// and three warps per scheduler issue on about half of the cycles, so a
+// visit's instructions and its latency both count.  An event is some 320
+// instructions and a draw 95, and one lane of 32 has an event at nearly every
+// step.  So a visit first draws its steps (four at a time side by side, targets
+// to shared memory), before its halo is there, and every round of events lets
+// each lane look once at its own next three targets: a lane with an event takes
+// it, one without sits out the round, and the warp needs about half as many
+// rounds as steps.  Before that the domain's words are asked for; counters are
+// added without reading them, and C_{c-1} is kept in shared memory.  512
+// uneven replicas, 60 schedules, records every 10, on 456 CTAs: at k = 4 5.93
+// -> 5.89 ms, k = 16 16.85 -> 14.41, k = 32 31.65 -> 26.27 against one step per
+// round with the next step's draw in line with the event; k = 1 3.64 -> 3.76.
+// Looks at two targets 5.80 / 14.79 / 27.31 (k = 4 / 16 / 32), at four 6.03 /
+// 14.65 / 26.64, lanes that look on until they find their next event no faster
+// than one step per round; four CTAs per SM at 128 registers 7.72 / 18.55 /
+// 33.68.
 template <bool EXPO>
 __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
 {
@@ -162,6 +171,7 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
     cum[0] = 0;
     const int bd = blockDim.x;
     uint2 *cache = reinterpret_cast<uint2 *>(cum + 10 * bd); // element (colour TPD_CACHE + round) bd: {domain, replica}
+    uint64_t *tg = cum + (10 + 4 * TPD_CACHE) * bd; // targets of the chunk
     const int tid = blockIdx.x * blockDim.x + threadIdx.x;
     const int nthreads = gridDim.x * blockDim.x;
     const uint32_t *col_off = P.cta_col_off;
@@ -284,7 +294,23 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
                 }
                 return act ? (((uint64_t)w.y << 32) | w.x) >> 1 : ~0ull;
             };
-            uint64_t tgt = draw(0);
+            // the targets of steps base .. base + 31 of the visit to shared memory
+            auto draw_chunk = [&](int base) {
+                const int n = min(TPD_CHUNK, smax - base);
+#pragma unroll 1
+                for (int i = 0; i + 4 <= n; i += 4) {
+                    uint64_t t[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) t[u] = draw(base + i + u);
+#pragma unroll
+                    for (int u = 0; u < 4; ++u) tg[(i + u) * bd] = t[u];
+                }
+#pragma unroll 1
+                for (int i = n & ~3; i < n; ++i) tg[i * bd] = draw(base + i);
+#pragma unroll
+                for (int u = 0; u < TPD_LOOK; ++u) tg[(n + u) * bd] = ~0ull;
+            };
+            draw_chunk(0);
             // halo: the N neighbour's S row, the S neighbour's N row, the W
             // neighbour's E column, the E neighbour's W column (half 0 of
             // each), stamped with the neighbour's completed visits; the warp
@@ -338,50 +364,62 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
             uint64_t R = tpd_rates(T, pl, A, Ch, cum, bd);
             uint32_t flips = 0;
             int dbonds = 0, dmag = 0;
-            // All lanes step together.  The next step's draw and the event of this
-            // one do not depend on each other: in one straight line they fill each
-            // other's latencies, so a lane without an event runs the event with
-            // no effect.  Only a step that is null in all 32 domains skips it.
-            for (int st = 0; st < smax; ++st) {
-                const bool ev = tgt < R; // else a null step (App. A: the diagonal 1 - R/n_d)
-                if (!__any_sync(FULL_WARP, ev)) {
-                    tgt = draw(st + 1);
-                    continue;
-                }
-                const uint64_t next = draw(st + 1);
-                // class: the first c with tgt < C_c; by the high words it may come
-                // out too high where those are equal
-                int c = 0;
-                const uint32_t th = (uint32_t)(tgt >> 32);
+            for (int base = 0; base < smax; base += TPD_CHUNK) {
+                if (base > 0) draw_chunk(base);
+                const int n = min(TPD_CHUNK, smax - base);
+                int pos = 0; // this lane's next step of the chunk
+                while (__any_sync(FULL_WARP, pos < n)) {
+                    // the first of the next steps that is no null step (App. A: the
+                    // diagonal 1 - R/n_d), else the last of them
+                    uint64_t t[TPD_LOOK];
 #pragma unroll
-                for (int cc = 0; cc < 9; ++cc) c += (th >= Ch[cc]) ? 1 : 0;
-                uint64_t Cprev = cum[c * bd];
-                while (tgt < Cprev) Cprev = cum[--c * bd];
-                const uint64_t Ac = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + c]);
-                // exact jj = floor((tgt - C_{c-1}) / A_c) < n_c <= 64: an FP32
-                // estimate rounded toward the lower side is jj or jj - 1, and
-                // one integer comparison decides which
-                const uint64_t x = tgt - Cprev;
-                const float inv = __frcp_rd(u64_to_float_ru(Ac));
-                uint32_t jj = (uint32_t)__fmul_rz(u64_to_float_rz(x), inv);
-                jj = (x - (uint64_t)jj * Ac >= Ac) ? jj + 1u : jj;
-                const int qc = (c >= 5) ? c - 5 : c;
-                const uint64_t mask = ((c >= 5) ? T : ~T) & pl.eq(qc);
-                const int site = select_bit(mask, jj) & 63;
-                T ^= ev ? 1ull << site : 0ull;
-                const int f = st >= k ? 1 : 0;
-                const uint64_t np = np0 + (uint64_t)f;
-                const uint64_t h = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)site)) * HASH_PRIME;
-                H = ev ? h : H;
-                flips += ev ? 1u : 0u;
-                // flipping spin s with neighbour sum 2 qc - 4 changes the bond
-                // sum by -2 s (2 qc - 4) and the magnetisation by -2 s
-                const int g2 = ev ? (c >= 5 ? -2 : 2) : 0;
-                dbonds += g2 * (2 * qc - 4);
-                dmag += g2;
-                pl.build(T, hN, hS, hW, hE);
-                R = tpd_rates(T, pl, A, Ch, cum, bd);
-                tgt = next;
+                    for (int u = 0; u < TPD_LOOK; ++u) t[u] = tg[(pos + u) * bd];
+                    uint64_t tgt = t[TPD_LOOK - 1];
+                    int off = TPD_LOOK - 1;
+#pragma unroll
+                    for (int u = TPD_LOOK - 2; u >= 0; --u) {
+                        const bool e = t[u] < R;
+                        tgt = e ? t[u] : tgt;
+                        off = e ? u : off;
+                    }
+                    const bool ev = tgt < R;
+                    const int st = base + pos + off;
+                    pos = min(pos + off + 1, n);
+                    // a lane without an event runs the event with no effect
+                    if (!__any_sync(FULL_WARP, ev)) continue;
+                    // class: the first c with tgt < C_c; by the high words it may come
+                    // out too high where those are equal
+                    int c = 0;
+                    const uint32_t th = (uint32_t)(tgt >> 32);
+#pragma unroll
+                    for (int cc = 0; cc < 9; ++cc) c += (th >= Ch[cc]) ? 1 : 0;
+                    uint64_t Cprev = cum[c * bd];
+                    while (tgt < Cprev) Cprev = cum[--c * bd];
+                    const uint64_t Ac = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + c]);
+                    // exact jj = floor((tgt - C_{c-1}) / A_c) < n_c <= 64: an FP32
+                    // estimate rounded toward the lower side is jj or jj - 1, and
+                    // one integer comparison decides which
+                    const uint64_t x = tgt - Cprev;
+                    const float inv = __frcp_rd(u64_to_float_ru(Ac));
+                    uint32_t jj = (uint32_t)__fmul_rz(u64_to_float_rz(x), inv);
+                    jj = (x - (uint64_t)jj * Ac >= Ac) ? jj + 1u : jj;
+                    const int qc = (c >= 5) ? c - 5 : c;
+                    const uint64_t mask = ((c >= 5) ? T : ~T) & pl.eq(qc);
+                    const int site = select_bit(mask, jj) & 63;
+                    T ^= ev ? 1ull << site : 0ull;
+                    const int f = st >= k ? 1 : 0;
+                    const uint64_t np = np0 + (uint64_t)f;
+                    const uint64_t h = (H ^ ((np << 32) | ((uint64_t)(st - (f ? k : 0)) << 16) | (uint64_t)site)) * HASH_PRIME;
+                    H = ev ? h : H;
+                    flips += ev ? 1u : 0u;
+                    // flipping spin s with neighbour sum 2 qc - 4 changes the bond
+                    // sum by -2 s (2 qc - 4) and the magnetisation by -2 s
+                    const int g2 = ev ? (c >= 5 ? -2 : 2) : 0;
+                    dbonds += g2 * (2 * qc - 4);
+                    dmag += g2;
+                    pl.build(T, hN, hS, hW, hE);
+                    R = tpd_rates(T, pl, A, Ch, cum, bd);
+                }
             }
             // edges first (neighbours wait for them), then tile, counters and record
             if (has) {

@@ -16,7 +16,7 @@ def _cuda():
         pytest.skip("no CUDA device")
 
 
-def _run(L, Ld, shift=0, plan=None, init=None):
+def _run(L, Ld, shift=0, plan=None, init=None, ks=None, schedule=0, time_mode=0):
     import torch
     import paper_1403_4674_gb300 as kmc
     n = sum(x * x for x in L)
@@ -27,11 +27,14 @@ def _run(L, Ld, shift=0, plan=None, init=None):
     if init is not None:
         sp.copy_(init)
         lat.reset(kmc.KMC_INIT_KEEP)
+    if ks is not None:
+        lat.set_replica_params(k=ks)
+        lat.reset(0)
     start = sp.cpu().numpy()
     if plan is not None:
         lat.set_launch(*plan)
     lat.set_rates([0.35 + 0.1 * i for i in range(len(L))], [0.05] * len(L))
-    obs = lat.run(6, obs_every=2).cpu().numpy()
+    obs = lat.run(6, schedule=schedule, time_mode=time_mode, obs_every=2).cpu().numpy()
     lat.sync()
     out = (start, sp.cpu().numpy(), *lat.domain_state(), obs, buf.cpu().numpy(), at, n)
     lat.close()
@@ -65,3 +68,13 @@ def test_rounds_of_the_8x8_kernel(ctas):
     """64 + 100 domains per colour on grids of 32 to 256 threads: one round to six."""
     L = [128, 160]
     _same(_run(L, 8, plan=(3, ctas, 1)), _run(L, 8, plan=(2, 8, 8)))
+
+
+@pytest.mark.parametrize("ks", [[1, 2], [3, 4], [15, 16], [17, 5], [32, 33], [1, 40]])
+@pytest.mark.parametrize("schedule,time_mode", [(0, 0), (1, 1)])
+def test_chunks_of_the_8x8_kernel(ks, schedule, time_mode):
+    """Visits that end inside, at and past a chunk of 32 drawn steps, replicas
+    of both lengths side by side in one warp."""
+    L = [48, 32]
+    a = _run(L, 8, plan=(3, 1, 2), ks=ks, schedule=schedule, time_mode=time_mode)
+    _same(a, _run(L, 8, plan=(2, 4, 8), ks=ks, schedule=schedule, time_mode=time_mode))
