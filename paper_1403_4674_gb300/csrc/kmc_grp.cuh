@@ -232,15 +232,19 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
     __syncthreads(); // the edge words of the CTA's domains are in place
 
     // The group's clock product since the record began, joined over its lanes
-    // (each lane multiplies the variates of its own steps).
-    auto joined_clock = [&](uint8_t *b, uint64_t &m, int &e) {
+    // (each lane multiplies the variates of its own steps).  A step takes 1.44
+    // off the exponent on average, and without records a launch's steps are
+    // one product: past 1.49e9 steps of a domain it leaves 32 bits.
+    auto joined_clock = [&](uint8_t *b, uint64_t &m, int64_t &e) {
         m = u64(b, Q::CLK + 16 * gl);
-        e = (int)(int64_t)u64(b, Q::CLK + 16 * gl + 8);
+        e = (int64_t)u64(b, Q::CLK + 16 * gl + 8);
 #pragma unroll
         for (int off = 1; off < G; off <<= 1) {
             const uint64_t m2 = __shfl_xor_sync(FULL_WARP, m, off);
-            const int e2 = __shfl_xor_sync(FULL_WARP, e, off);
-            mant_mul32(m, e, m2, e2);
+            const int64_t e2 = __shfl_xor_sync(FULL_WARP, (long long)e, off);
+            int up = 0;
+            mant_mul32(m, up, m2, 0);
+            e += e2 + up;
         }
         u64(b, Q::CLK + 16 * gl) = 1ull << 63;
         u64(b, Q::CLK + 16 * gl + 8) = 0;
@@ -250,7 +254,7 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
     // product into the domain's clock.  Called by the whole warp.
     auto flush = [&](uint8_t *b) {
         uint64_t m = 1ull << 63;
-        int e = 0;
+        int64_t e = 0;
         if (EXPO) joined_clock(b, m, e);
         const bool mine = gl == 0 && u32(b, Q::META) != 0xFFFFFFFFu;
         const uint64_t o0 = u64(b, Q::OBS), o1 = u64(b, Q::OBS + 8);
@@ -260,12 +264,12 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
         if (mine && EXPO) {
             uint64_t cm = u64(b, Q::CTR + 24);
             int64_t ce = (int64_t)u64(b, Q::CTR + 32);
-            mant_mul(cm, ce, m, (int64_t)e);
+            mant_mul(cm, ce, m, e);
             u64(b, Q::CTR + 24) = cm;
             u64(b, Q::CTR + 32) = (uint64_t)ce;
         }
         if (on)
-            dt = EXPO ? domain_time(true, m, (int64_t)e, 0, P.lambda) : __ddiv_rn((double)(uint32_t)(o0 >> 32), P.lambda);
+            dt = EXPO ? domain_time(true, m, e, 0, P.lambda) : __ddiv_rn((double)(uint32_t)(o0 >> 32), P.lambda);
         // the set's domains are one replica's and share the record: one sum
         int bonds = on ? (int)(uint32_t)o1 : 0, mag = on ? (int)(uint32_t)(o1 >> 32) : 0;
 #pragma unroll
@@ -693,12 +697,10 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
             __syncwarp();
         }
         if (EXPO) {
-            ulonglong2 &cl = *reinterpret_cast<ulonglong2 *>(b + Q::CLK + 16 * gl);
-            const ulonglong2 me = cl;
-            uint64_t m = me.x;
-            int e = (int)(int64_t)me.y;
-            mant_mul32(m, e, vM, vE);
-            cl = make_ulonglong2(m, (uint64_t)(int64_t)e);
+            uint64_t m = u64(b, Q::CLK + 16 * gl);
+            mant_mul32(m, vE, vM, 0);
+            u64(b, Q::CLK + 16 * gl) = m;
+            u64(b, Q::CLK + 16 * gl + 8) += (uint64_t)(int64_t)vE;
         }
         const uint64_t fl = u64(b, Q::CTR + 8), nst = u64(b, Q::CTR + 16), o0 = u64(b, Q::OBS), o1 = u64(b, Q::OBS + 8);
         __syncwarp();
