@@ -606,9 +606,9 @@ size_t grp_domain_bytes_for(int LD, int G)
     if (LD == 32) return G == 8 ? grp_domain_bytes<32, 8>() : G == 16 ? grp_domain_bytes<32, 16>() : grp_domain_bytes<32, 32>();
     return G == 16 ? grp_domain_bytes<64, 16>() : grp_domain_bytes<64, 32>();
 }
-TpdKernel thread_plan_kernel(const kmc_ctx *c, const Plan &pl, bool expo)
+TpdKernel thread_plan_kernel(const kmc_ctx *c, const Plan &pl, bool expo, int scores)
 {
-    return pl.groups ? grp_kernel_for(c->LD, pl.groups, expo) : tpd_kernel_for(c->LD, expo, scores_of(c));
+    return pl.groups ? grp_kernel_for(c->LD, pl.groups, expo) : tpd_kernel_for(c->LD, expo, scores);
 }
 size_t tpdr_warp_bytes_for(int LD)
 {
@@ -820,7 +820,8 @@ int balanced_thread_ctas(const kmc_ctx *c, int wpb)
 }
 
 // Can this plan run?  Shared memory, cluster support and (GRID) co-residency.
-// Only the kernels this context can launch are checked: both clock modes,
+// Only the kernels this context can launch are checked: both clock modes
+// without scores (they can be turned off at any time, also while capturing),
 // and the score-carrying variant only while scores are on (it holds more
 // registers, so fewer of its CTAs fit an SM; kmc_enable_grad re-checks).
 kmc_status check_plan(kmc_ctx *c, const Plan &pl)
@@ -829,8 +830,8 @@ kmc_status check_plan(kmc_ctx *c, const Plan &pl)
         if (c->grad && (c->LD == 8 || c->LD == 64))
             return fail(c, KMC_EINVAL, "the thread-per-domain plan of L_d = %d has no score kernel", c->LD);
         if (c->grad && pl.groups) return fail(c, KMC_EINVAL, "the lane-group kernel carries no scores");
-        for (int e = 0; e < 2; ++e) {
-            const void *kern = (const void *)thread_plan_kernel(c, pl, e == 0);
+        for (int v = 0; v < (c->grad ? 4 : 2); ++v) {
+            const void *kern = (const void *)thread_plan_kernel(c, pl, (v & 1) == 0, v < 2 ? NO_SCORES : scores_of(c));
             if (pl.smem > 0) {
                 if (pl.smem > (size_t)c->smem_optin)
                     return fail(c, KMC_EINVAL, "thread plan needs %zu bytes of shared memory per CTA (%d available)",
@@ -1783,7 +1784,7 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     const Plan &pl = c->plan;
     const bool cluster = pl.mode == KMC_LAUNCH_CLUSTER;
     const bool threads = pl.mode == KMC_LAUNCH_THREADS || pl.groups;
-    RunKernel kern = threads ? thread_plan_kernel(c, pl, time_mode == KMC_TIME_EXPONENTIAL)
+    RunKernel kern = threads ? thread_plan_kernel(c, pl, time_mode == KMC_TIME_EXPONENTIAL, scores_of(c))
                              : run_kernel_for(c->LD, time_mode == KMC_TIME_EXPONENTIAL, c->grad, cluster);
     cudaEvent_t ev0 = nullptr, ev1 = nullptr;
     const bool prof = c->prof && !cap;
