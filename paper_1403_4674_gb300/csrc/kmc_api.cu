@@ -43,6 +43,8 @@ struct Plan {
     int groups = 0;   // lanes per domain (grp_kernel; THREADS mode of L_d = 16, 32, 64, or GRID), 0: the mode's own kernel
     size_t smem = 0;
     bool checked = false; // check_plan has passed for the kernels of now
+    uint32_t *dev = nullptr; // device copy of the tables below (of an installed plan; the context's)
+    bool captured = false;   // a captured graph may read dev
     std::vector<uint32_t> cta_slot_off, cta_col_off, cta_rt_off, rt_rep, slot_g, slot_rt, slot_nb;
 };
 
@@ -79,15 +81,6 @@ struct kmc_ctx {
     unsigned long long *d_obs_acc = nullptr;
     size_t obs_acc_words = 0;
     void *d_tmp = nullptr; // n_dom * 32 + n_rep * 64 bytes, host-facing staging
-    // device copy of the launch plan
-    uint32_t *d_plan = nullptr;
-    size_t plan_words = 0;
-    // beside a random-order run's lane groups: the warp plan that such a run
-    // installs otherwise, ready for a fixed-time run (also while capturing)
-    uint32_t *d_alt = nullptr;
-    size_t alt_words = 0;
-    Plan alt;
-
     double J = 1.0, nu = 1.0;
     std::vector<double> beta, h, a, gb, gh;
     std::vector<uint64_t> A;
@@ -104,7 +97,11 @@ struct kmc_ctx {
     bool grad = false;
 
     int sm_count = 0, smem_optin = 0;
-    Plan plan;
+    // the launch plan, and beside a random-order run's lane groups the warp
+    // plan that such a run installs otherwise, ready for a fixed-time run
+    // (also while capturing)
+    Plan plan, alt;
+    std::vector<uint32_t *> kept; // tables of replaced plans that captured graphs read, until destroy
     int req_mode = KMC_LAUNCH_AUTO, req_size = 0, req_wpb = 16; // last requested plan
     int64_t launches = 0;
     int debug_extra = 0;
@@ -305,7 +302,7 @@ RunParams run_params(kmc_ctx *c)
     P.rep_gfix = c->d_gfix;
     P.rep_grad = c->d_grad;
     const Plan &pl = c->plan;
-    uint32_t *base = c->d_plan;
+    uint32_t *base = pl.dev;
     size_t off = 0;
     auto take = [&](size_t n) { uint32_t *p = base + off; off += n; return p; };
     P.cta_slot_off = take(pl.cta_slot_off.size());
@@ -895,24 +892,37 @@ kmc_status check_plan(kmc_ctx *c, const Plan &pl)
     return KMC_OK;
 }
 
+// The device tables of a plan that is replaced: a captured graph may be
+// replayed at any time, so what it reads stays until the context ends.  No
+// launch is in flight (install_plan has drained the stream).
+void release_plan(kmc_ctx *c, Plan &pl)
+{
+    if (pl.dev && pl.captured) c->kept.push_back(pl.dev);
+    else if (pl.dev) cudaFree(pl.dev);
+    pl = Plan();
+}
+
+// Make pl the context's plan, with device tables of its own: launches still
+// queued, and captured graphs, read those of the plan they were made with.
 kmc_status install_plan(kmc_ctx *c, Plan &pl)
 {
     kmc_status s = pl.checked ? KMC_OK : check_plan(c, pl);
     if (s != KMC_OK) return s;
     pl.checked = false;
-    if (c->d_alt) cudaFree(c->d_alt);
-    c->d_alt = nullptr;
     std::vector<uint32_t> flat;
     for (auto *v : {&pl.cta_slot_off, &pl.cta_col_off, &pl.cta_rt_off, &pl.rt_rep, &pl.slot_g, &pl.slot_rt, &pl.slot_nb})
         flat.insert(flat.end(), v->begin(), v->end());
-    if (flat.size() > c->plan_words) {
-        if (c->d_plan) cudaFree(c->d_plan);
-        c->d_plan = nullptr;
-        c->plan_words = 0;
-        if ((s = dev_alloc(c, &c->d_plan, flat.size())) != KMC_OK) return s;
-        c->plan_words = flat.size();
+    uint32_t *dev = nullptr;
+    if ((s = dev_alloc(c, &dev, flat.size())) != KMC_OK) return s;
+    cudaError_t ce = cudaMemcpy(dev, flat.data(), flat.size() * 4, cudaMemcpyHostToDevice);
+    if (ce == cudaSuccess && (c->plan.dev || c->alt.dev)) ce = cudaStreamSynchronize(c->stream);
+    if (ce != cudaSuccess) {
+        cudaFree(dev);
+        return fail(c, KMC_ECUDA, "launch plan: %s", cudaGetErrorString(ce));
     }
-    CUDA_TRY(c, cudaMemcpy(c->d_plan, flat.data(), flat.size() * 4, cudaMemcpyHostToDevice));
+    release_plan(c, c->plan);
+    release_plan(c, c->alt);
+    pl.dev = dev;
     c->plan = std::move(pl);
     return KMC_OK;
 }
@@ -1213,17 +1223,18 @@ kmc_status sync_ctx(kmc_ctx *c)
 void free_all(kmc_ctx *c)
 {
     void **ptrs[] = {(void **)&c->d_L, (void **)&c->d_Dx, (void **)&c->d_k, (void **)&c->d_init, (void **)&c->d_dom_off, (void **)&c->d_dom_rep,
-                     (void **)&c->d_alt, (void **)&c->d_site_off, (void **)&c->d_blk_off, (void **)&c->d_seed, (void **)&c->d_A,
+                     (void **)&c->d_site_off, (void **)&c->d_blk_off, (void **)&c->d_seed, (void **)&c->d_A,
                      (void **)&c->d_gfix, (void **)&c->d_grad, (void **)&c->d_h, (void **)&c->d_tiles,
                      (void **)&c->d_edges, (void **)&c->d_dctr, (void **)&c->d_err,
-                     (void **)&c->d_obs_acc, (void **)&c->d_tmp, (void **)&c->d_plan, (void **)&c->d_htab,
-                     (void **)&c->d_polls, (void **)&c->d_obs_dom};
+                     (void **)&c->d_obs_acc, (void **)&c->d_tmp, (void **)&c->d_htab,
+                     (void **)&c->d_polls, (void **)&c->d_obs_dom, (void **)&c->plan.dev, (void **)&c->alt.dev};
     for (void **p : ptrs) {
         if (*p) cudaFree(*p);
         *p = nullptr;
     }
+    for (uint32_t *p : c->kept) cudaFree(p);
+    c->kept.clear();
     c->obs_acc_words = 0;
-    c->plan_words = 0;
 }
 
 } // namespace
@@ -1712,40 +1723,26 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     const bool cap = capturing(c);
     const bool random_order = schedule == KMC_SCHEDULE_RANDOM_PERM, fixed_time = time_mode == KMC_TIME_HORIZON;
     const bool scores8_64 = c->grad && (c->LD == 8 || c->LD == 64);
-    if (c->plan.groups && c->plan.mode == KMC_LAUNCH_GRID && fixed_time && c->d_alt) {
-        // back to the warp plan (earlier launches keep reading the other buffer)
-        std::swap(c->plan, c->alt);
-        std::swap(c->d_plan, c->d_alt);
-        std::swap(c->plan_words, c->alt_words);
-    }
+    // back to the warp plan
+    if (c->plan.groups && c->plan.mode == KMC_LAUNCH_GRID && fixed_time && c->alt.dev) std::swap(c->plan, c->alt);
     if ((c->plan.mode == KMC_LAUNCH_THREADS && (scores8_64 || fixed_time || random_order)) ||
         (c->plan.groups && (c->grad || fixed_time))) {
         // the thread kernels cover fixed-length visits of the palindromic
         // and fixed schedules (with scores at L_d = 16, 32), and lane groups
         // random orders too: this run takes a warp plan, or a grid of lane
-        // groups with the warp plan kept beside it (installed once the stream
-        // has drained: earlier launches read the plan buffer)
+        // groups with the warp plan kept beside it
         if (cap) return fail(c, KMC_EINVAL, "this run needs a warp launch plan; set one before capturing");
-        CUDA_TRY(c, cudaStreamSynchronize(s));
         if ((st = default_warp_plan(c)) != KMC_OK) return st;
         Plan pl;
         if (random_order && !fixed_time && !c->grad && plan_few_domains(c, 0, pl, false) == KMC_OK) {
             pl.mode = KMC_LAUNCH_GRID;
-            Plan warp = c->plan;
-            uint32_t *d_warp = c->d_plan;
-            const size_t words = c->plan_words;
-            c->d_plan = nullptr;
-            c->plan_words = 0;
+            Plan warp;
+            std::swap(warp, c->plan);
             if (install_plan(c, pl) == KMC_OK) {
                 c->alt = std::move(warp);
-                c->d_alt = d_warp;
-                c->alt_words = words;
             } else {
                 cudaGetLastError();
-                if (c->d_plan) cudaFree(c->d_plan);
                 c->plan = std::move(warp);
-                c->d_plan = d_warp;
-                c->plan_words = words;
             }
         }
     }
@@ -1766,6 +1763,7 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     if ((st = n_obs > 0 ? launch_pack(c, s, base, c->d_obs_acc, (size_t)n_obs * c->n_rep * OBS_WORDS) : launch_pack(c, s)) != KMC_OK)
         return st;
     if (n_obs > 0 && (st = launch_observe(c, s, time_mode, base)) != KMC_OK) return st;
+    if (cap) c->plan.captured = true;
     RunParams P = run_params(c);
     P.schedule = schedule;
     P.obs_every = want_obs ? obs_every : 0;
@@ -1991,7 +1989,7 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
         c.d_edges = cv.take<uint64_t>((size_t)c.n_dom * EDGE_WORDS);
         c.d_dctr = cv.take<uint64_t>((size_t)c.n_dom * DCTR_WORDS);
         c.d_dom_rep = cv.take<uint32_t>((size_t)c.n_dom);
-        c.d_plan = cv.take<uint32_t>(flat.size());
+        pl.dev = cv.take<uint32_t>(flat.size());
         c.d_obs_acc = cv.take<unsigned long long>((size_t)std::max<int64_t>(n_obs, 1) * OBS_WORDS);
         c.d_L = cv.take<int32_t>(1);
         c.d_Dx = cv.take<int32_t>(1);
@@ -2031,7 +2029,6 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
     }
     Carver cv{base};
     carve(cv);
-    c.plan_words = flat.size();
 
     // inputs of this call; the array keeps the previous call's contents, so
     // everything the kernels read is written (or cleared) here first
@@ -2050,7 +2047,7 @@ kmc_status kmc_run_schedule_noalloc(int32_t L, int32_t L_d, int32_t k_steps, uin
         {c.d_L, c.L.data(), 4}, {c.d_Dx, c.Dx.data(), 4}, {c.d_k, c.kr.data(), 4}, {c.d_dom_off, c.dom_off.data(), 8},
         {c.d_site_off, c.site_off.data(), 8}, {c.d_blk_off, c.blk_off.data(), 16}, {c.d_seed, c.seed.data(), 8},
         {c.d_A, A16.data(), RATE_WORDS * 8}, {c.d_gfix, gfix.data(), GFIX_WORDS * 8}, {c.d_grad, g32.data(), 256}, {c.d_h, c.h.data(), 8},
-        {c.d_dom_rep, c.dom_rep.data(), (size_t)c.n_dom * 4}, {c.d_plan, flat.data(), flat.size() * 4},
+        {c.d_dom_rep, c.dom_rep.data(), (size_t)c.n_dom * 4}, {pl.dev, flat.data(), flat.size() * 4},
     };
     for (const Up &u : ups) {
         // pageable host source: the copy has completed when the call returns

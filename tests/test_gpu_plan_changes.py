@@ -72,3 +72,66 @@ def test_scores_turned_off_again(args):
     res = subprocess.run([sys.executable, "-c", OFF_AGAIN % ROOT, *map(str, args)], capture_output=True, text=True,
                          timeout=300)
     assert res.returncode == 0, res.stderr[-2000:]
+
+
+def _queued(plan):
+    """Runs queued on a non-blocking stream while the plan changes twice."""
+    import torch
+    import paper_1403_4674_gb300 as kmc
+    side = torch.cuda.Stream()
+    with torch.cuda.stream(side):
+        lat = kmc.Lattice([256], 32, 8, [11])
+        if plan:
+            lat.set_launch(*plan)
+        lat.set_rates([0.42], [0.01])
+        for _ in range(4):
+            lat.run(500)
+        lat.enable_grad(True)
+        for _ in range(4):
+            lat.run(500)
+        if not plan:
+            lat.set_launch(THREADS, 2, 2)
+        for _ in range(2):
+            lat.run(500)
+        lat.enable_grad(False)
+        lat.run(100)
+        return _state(lat)
+
+
+def test_plans_change_while_runs_are_queued():
+    _same(_queued(None), _queued(WARP))
+
+
+def _graphs(plan):
+    """Graphs captured with a plan that is then replaced."""
+    import torch
+    import paper_1403_4674_gb300 as kmc
+    side = torch.cuda.Stream()
+    lat = kmc.Lattice([256], 32, 8, [11])
+    if plan:
+        lat.set_launch(*plan)
+    lat.set_rates([0.42], [0.01])
+    torch.cuda.synchronize()
+    a = _captured(side, lat, 20)
+    lat.enable_grad(True)
+    lat.run(5)
+    torch.cuda.synchronize()
+    b = _captured(side, lat, 7)
+    if not plan:
+        lat.set_launch(GRID, 76, 4)
+    lat.run(3)
+    lat.enable_grad(False)
+    if not plan:
+        lat.set_launch()
+    lat.run(3)
+    torch.cuda.synchronize()
+    fill = [torch.full((1 << 16,), -1, dtype=torch.int32, device="cuda") for _ in range(8)]  # (into freed memory)
+    for g in (a, b, a):
+        g.replay()
+        torch.cuda.synchronize()
+    del fill
+    return _state(lat)
+
+
+def test_graphs_outlive_their_plan():
+    _same(_graphs(None), _graphs(WARP))
