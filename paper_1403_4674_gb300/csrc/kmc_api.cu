@@ -97,9 +97,9 @@ struct kmc_ctx {
     bool grad = false;
 
     int sm_count = 0, smem_optin = 0;
-    // the launch plan, and beside a random-order run's lane groups the warp
-    // plan that such a run installs otherwise, ready for a fixed-time run
-    // (also while capturing)
+    // the launch plan, and beside lane groups the plan for the runs that they
+    // do not serve (fixed-time visits, scores), each ready for a run that
+    // takes it again, also while capturing
     Plan plan, alt;
     std::vector<uint32_t *> kept; // tables of replaced plans that captured graphs read, until destroy
     int req_mode = KMC_LAUNCH_AUTO, req_size = 0, req_wpb = 16; // last requested plan
@@ -927,6 +927,26 @@ kmc_status install_plan(kmc_ctx *c, Plan &pl)
     return KMC_OK;
 }
 
+// Does plan pl serve such runs?  The thread kernels cover fixed-length visits
+// of the palindromic and fixed schedules (with scores at L_d = 16, 32); lane
+// groups carry no scores, and take random orders only with a warp plan beside
+// them (`other`), so that every run after one has a plan also while capturing.
+bool plan_serves(const kmc_ctx *c, const Plan &pl, const Plan &other, bool random_order, bool fixed_time)
+{
+    if (pl.groups) return !c->grad && !fixed_time && (!random_order || (other.dev && other.mode != KMC_LAUNCH_THREADS));
+    if (pl.mode == KMC_LAUNCH_THREADS)
+        return !fixed_time && !random_order && !(c->grad && (c->LD == 8 || c->LD == 64));
+    return true;
+}
+
+// Of the context's two plans the one for such runs: lane groups where they serve.
+void choose_plan(kmc_ctx *c, bool random_order, bool fixed_time)
+{
+    if (c->alt.dev && plan_serves(c, c->alt, c->plan, random_order, fixed_time) &&
+        (c->alt.groups || !plan_serves(c, c->plan, c->alt, random_order, fixed_time)))
+        std::swap(c->plan, c->alt);
+}
+
 kmc_status default_warp_plan(kmc_ctx *c);
 
 // The library's plan: one thread per domain (a warp then runs 32 domain
@@ -1685,15 +1705,23 @@ kmc_status kmc_enable_grad(kmc_ctx *c, int32_t enable)
             c->grad = was;
             return KMC_EINVAL;
         }
-        // the score kernels may not fit the current plan's shape: re-plan
-        Plan pl = c->plan;
-        if (check_plan(c, pl) != KMC_OK &&
-            kmc_set_launch(c, c->req_mode, c->req_size, c->req_wpb) != KMC_OK && default_plan(c) != KMC_OK) {
-            const std::string why = c->err;
-            c->grad = was;
-            return fail(c, KMC_EINVAL, "no launch plan fits the score kernels: %s", why.c_str());
+        // the score kernels may not fit the current plan's shape: re-plan (lane
+        // groups stay beside the new plan for when scores go off again)
+        choose_plan(c, false, false);
+        if (check_plan(c, c->plan) != KMC_OK) {
+            Plan groups;
+            std::swap(groups, c->plan.groups ? c->plan : c->alt);
+            if (kmc_set_launch(c, c->req_mode, c->req_size, c->req_wpb) != KMC_OK && default_plan(c) != KMC_OK) {
+                const std::string why = c->err;
+                std::swap(groups, c->plan.dev ? c->alt : c->plan);
+                c->grad = was;
+                choose_plan(c, false, false);
+                return fail(c, KMC_EINVAL, "no launch plan fits the score kernels: %s", why.c_str());
+            }
+            c->alt = std::move(groups);
         }
     }
+    choose_plan(c, false, false);
     return KMC_OK;
 }
 
@@ -1722,15 +1750,10 @@ kmc_status kmc_run_schedule(kmc_ctx *c, int64_t n_schedules, int32_t schedule, i
     const int64_t n_obs = want_obs ? units / obs_every : 0;
     const bool cap = capturing(c);
     const bool random_order = schedule == KMC_SCHEDULE_RANDOM_PERM, fixed_time = time_mode == KMC_TIME_HORIZON;
-    const bool scores8_64 = c->grad && (c->LD == 8 || c->LD == 64);
-    // back to the warp plan
-    if (c->plan.groups && c->plan.mode == KMC_LAUNCH_GRID && fixed_time && c->alt.dev) std::swap(c->plan, c->alt);
-    if ((c->plan.mode == KMC_LAUNCH_THREADS && (scores8_64 || fixed_time || random_order)) ||
-        (c->plan.groups && (c->grad || fixed_time))) {
-        // the thread kernels cover fixed-length visits of the palindromic
-        // and fixed schedules (with scores at L_d = 16, 32), and lane groups
-        // random orders too: this run takes a warp plan, or a grid of lane
-        // groups with the warp plan kept beside it
+    choose_plan(c, random_order, fixed_time);
+    if (!plan_serves(c, c->plan, c->alt, random_order, fixed_time)) {
+        // this run takes a warp plan, or a grid of lane groups with the warp
+        // plan kept beside it
         if (cap) return fail(c, KMC_EINVAL, "this run needs a warp launch plan; set one before capturing");
         if ((st = default_warp_plan(c)) != KMC_OK) return st;
         Plan pl;

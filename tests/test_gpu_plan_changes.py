@@ -135,3 +135,47 @@ def _graphs(plan):
 
 def test_graphs_outlive_their_plan():
     _same(_graphs(None), _graphs(WARP))
+
+
+@pytest.mark.parametrize("Ld", [16, 32, 64])
+def test_random_orders_with_scores_captured(Ld):
+    """After a random-order run every run has its plan at hand, also while capturing."""
+    import torch
+    import paper_1403_4674_gb300 as kmc
+    out, RANDOM = [], kmc.KMC_SCHEDULE_RANDOM_PERM
+    for plan in (None, WARP):
+        side = torch.cuda.Stream()
+        lat = kmc.Lattice([4 * Ld, 2 * Ld], Ld, 4, [3, 4])
+        if plan:
+            lat.set_launch(*plan)
+        lat.set_rates([0.42, 0.3], [0.01, 0.0])
+        lat.set_horizon(0.02)
+        lat.run(2, schedule=RANDOM)
+        lat.enable_grad(True)
+        torch.cuda.synchronize()
+        graphs = [_captured(side, lat, 3, schedule=RANDOM), _captured(side, lat, 2)]
+        lat.enable_grad(False)
+        graphs += [_captured(side, lat, 3, schedule=RANDOM), _captured(side, lat, 2, time_mode=kmc.KMC_TIME_HORIZON),
+                   _captured(side, lat, 1)]
+        for g in graphs:
+            g.replay()
+            torch.cuda.synchronize()
+        lat.run(2, schedule=RANDOM)
+        lat.sync()
+        out.append((lat.spins.cpu().numpy(), *lat.domain_state()[:2], lat.score().cpu().numpy()))
+        lat.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("Ld", [16, 32])
+def test_lane_groups_again_after_scores(Ld):
+    import paper_1403_4674_gb300 as kmc
+    lat = kmc.Lattice([8 * Ld], Ld, 4, [3])
+    before = lat.launch()
+    lat.enable_grad(True)
+    assert lat.launch() != before
+    lat.run(1)
+    lat.enable_grad(False)
+    assert lat.launch() == before
+    lat.close()
