@@ -775,7 +775,7 @@ __global__ void __launch_bounds__(512, 1) grp_kernel(const RunParams P)
     }
     if (P.polls && lane == 0 && polls != 0) atomicAdd(P.polls, polls);
     __syncthreads();
-    if (*(volatile int *)P.err != 0) return;
+    if (__any_sync(FULL_WARP, *(volatile int *)P.err != 0)) return; // (whole warps: records are closed by the warp)
     // write the domains back: tile, counters, open record
     for (int s = 0; s < ns; ++s) {
         uint8_t *b = dom(s);

@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
         gp += (uint64_t)nf;
     }
     if (P.polls && spins != 0) atomicAdd(P.polls, (unsigned long long)spins);
-    if (!ok || *(volatile int *)P.err != 0) return;
+    if (__any_sync(FULL_WARP, !ok || *(volatile int *)P.err != 0)) return; // (whole warps: records are closed by the warp)
     // every owned domain's open record
     if (P.n_obs > 0) {
         for (int c = 0; c < 4; ++c) {

@@ -893,7 +893,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
         gp += (uint64_t)nf;
     }
     if (P.polls && lane == 0 && polls != 0) atomicAdd(P.polls, polls);
-    if (!ok || *(volatile int *)P.err != 0) return;
+    if (__any_sync(FULL_WARP, !ok || *(volatile int *)P.err != 0)) return; // (whole warps: records are closed by the warp)
     // write the domain back: tile, counters, open record
     if (has) {
         for (int y = 0; y < LD; ++y) {

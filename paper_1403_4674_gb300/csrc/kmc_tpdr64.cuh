@@ -722,7 +722,7 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
         gp += (uint64_t)nf;
     }
     if (P.polls && lane == 0 && polls != 0) atomicAdd(P.polls, polls);
-    if (!ok || *(volatile int *)P.err != 0) return;
+    if (__any_sync(FULL_WARP, !ok || *(volatile int *)P.err != 0)) return; // (whole warps: records are closed by the warp)
     // write the domain back: tile, counters, open record
     if (has) {
         uint64_t *tile = reinterpret_cast<uint64_t *>(P.tiles + (size_t)g * (LD * LD / 8));
