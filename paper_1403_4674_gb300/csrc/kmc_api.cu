@@ -679,8 +679,16 @@ kmc_status check_plan(kmc_ctx *c, const Plan &pl);
 // has a warp of its own, the warps of set i of the four colours next to each
 // other in the grid; otherwise a warp takes ns / 2 sets of colours 0 and 1 or
 // of colours 3 and 2, so that colours 1 and 2, which do not wait for each
-// other, still run side by side.  wpb 0: a whole replica per CTA where 16
-// warps hold it (all its halos then stay in shared memory), else 4 warps.
+// other, still run side by side.  wpb 0: 4 warps per CTA, so that the warps
+// spread over the SMs; 8 for small replicas whose visits are so short that
+// halos in the CTA's own shared memory are worth more, while the SMs hold more
+// than 4 warps anyway.  Measured, us per schedule with a whole replica per CTA
+// (16 warps), 8 and 4 warps: 64 lattices of 256^2 in domains of 32x32 (4096
+// domains) at k = 1 9.5, 7.0, 6.9, at k = 4 20.8, 14.1, 13.4, at k = 16 63.1,
+// 40.4, 31.7 (one thread per domain: 54.1); 100 lattices of 64^2 in domains of
+// 16x16, 8 and 4 warps: at k = 1 4.84, 5.22, at k = 2 6.6, 6.8, at k = 4 9.8, 9.5;
+// 140 lattices of 128^2 so (two sets per warp for want of room) at k = 1 8.8,
+// 9.2, at k = 4 15.35, 15.43, at k = 16 35.8, 35.3.
 kmc_status plan_groups(kmc_ctx *c, int G, int ns, int wpb, Plan &pl, bool interleave)
 {
     if (!grp_kernel_for(c->LD, G, true)) return fail(c, KMC_EINVAL, "no lane-group kernel for L_d = %d, G = %d", c->LD, G);
@@ -689,8 +697,10 @@ kmc_status plan_groups(kmc_ctx *c, int G, int ns, int wpb, Plan &pl, bool interl
     struct Set { int r, first, n; };
     std::vector<Set> sets;
     int most = 0;
+    int64_t steps = 0;
     for (int r = 0; r < c->n_rep; ++r) {
         const int per = c->Dx[r] * c->Dx[r] / 4;
+        steps += 4ll * per * c->kr[r];
         most = std::max(most, (per + dpw - 1) / dpw);
         for (int i = 0; i < per && !interleave; i += dpw) sets.push_back({r, i, std::min(dpw, per - i)});
     }
@@ -699,17 +709,17 @@ kmc_status plan_groups(kmc_ctx *c, int G, int ns, int wpb, Plan &pl, bool interl
             const int per = c->Dx[r] * c->Dx[r] / 4;
             if (i * dpw < per) sets.push_back({r, i * dpw, std::min(dpw, per - i * dpw)});
         }
+    const size_t half = ns / 2;
+    const size_t warps = (ns == 1) ? 4 * sets.size() : 2 * ((sets.size() + half - 1) / half);
     if (wpb == 0) {
-        wpb = 4;
-        while (4 * most <= MAX_WPB && wpb < 4 * most) wpb *= 2;
+        const bool brief = steps < (ns == 1 ? 3ll : 8ll) * c->n_dom;
+        wpb = (brief && most > 1 && 4 * most <= MAX_WPB && warps > (size_t)4 * c->sm_count) ? 8 : 4;
     }
     pl = Plan();
     pl.mode = KMC_LAUNCH_THREADS;
     pl.groups = G;
     pl.wpb = wpb;
     pl.max_rt = ns;
-    const size_t half = ns / 2;
-    const size_t warps = (ns == 1) ? 4 * sets.size() : 2 * ((sets.size() + half - 1) / half);
     pl.n_cta = (int)((warps + wpb - 1) / wpb);
     const size_t n_warps = (size_t)pl.n_cta * wpb;
     pl.smem = GRP_TABLE_BYTES + (size_t)wpb * ns * dpw * grp_domain_bytes_for(c->LD, G);
