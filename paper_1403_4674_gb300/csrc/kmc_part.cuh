@@ -56,7 +56,10 @@ constexpr uint32_t PART_TAG_PERM = 2u;
 constexpr int PART_ROW32 = 6;
 // The class counts of domain rows are kept (u8 [N_D][10][rows], the rows
 // padded to a multiple of 16: one 128-bit load each 16 rows) when the
-// lattice has at most PART_RC_ROWS padded domain rows.
+// lattice has at most PART_RC_ROWS padded domain rows.  Otherwise an event
+// counts its domain's rows, four a lane over the whole warp (16 a lane on the
+// few lanes that would load them took 2.4 times as long: 1000 trajectories of
+// 100^2 in ten stripes, k = 5, 79 and 32 us a schedule).
 constexpr int PART_RC_ROWS = 1024;
 constexpr int PART_ORDER_BYTES = 1024;
 // shared memory of a trajectory in bytes: the class counts of the domain
@@ -246,6 +249,7 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
     const int nbx = stripes ? ND : P.Dx, nby = stripes ? 1 : P.Dx; // domains per row and column
 
     const bool use_rc = ND * Hp <= PART_RC_ROWS;
+    const int rpl = use_rc ? 16 : 4; // rows per lane in an event
     if (lane < 10) {
         const uint64_t Al = P.A[(size_t)tr * 10 + lane];
         atab[lane] = make_ulonglong2(Al, Al ? ~0ull / Al : 0ull);
@@ -481,25 +485,22 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
             const uint32_t ejj = pick >> 10;
             const int x0 = org[2 * ed], y0 = org[2 * ed + 1];
             // the row of the jj-th member of class c in row-major order: lane l
-            // holds the counts of domain rows 16 l .. 16 l + 15, a byte each
+            // holds the counts of domain rows rpl l .. rpl l + rpl - 1, a byte each
             uint4 rw = make_uint4(0u, 0u, 0u, 0u);
             if (use_rc) {
                 if (16 * lane < Hd) rw = *reinterpret_cast<const uint4 *>(rc + (ed * 10 + ec) * Hp + 16 * lane);
-            } else if (16 * lane < Hd) {
+            } else {
                 const u128 DM = DM0 << x0;
-                uint32_t wq[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-                for (int t = 0; t < 16; ++t) {
-                    const int yy = 16 * lane + t;
+                for (int t = 0; t < 4; ++t) {
+                    const int yy = 4 * lane + t;
                     if (yy < Hd)
-                        wq[t >> 2] |= (uint32_t)popc128(class_mask(row_planes(rows, y0 + yy, L, Lm, DM), ec)) << (8 * (t & 3));
+                        rw.x |= (uint32_t)popc128(class_mask(row_planes(rows, y0 + yy, L, Lm, DM), ec)) << (8 * t);
                 }
-                rw = make_uint4(wq[0], wq[1], wq[2], wq[3]);
             }
             const uint32_t q0 = __dp4a(rw.x, 0x01010101u, 0u), q1 = __dp4a(rw.y, 0x01010101u, q0),
                            q2 = __dp4a(rw.z, 0x01010101u, q1), cl = __dp4a(rw.w, 0x01010101u, q2);
             uint32_t incl = cl;
-            for (int off = 1; 16 * off < Hd; off <<= 1) {
+            for (int off = 1; rpl * off < Hd; off <<= 1) {
                 const uint32_t u = __shfl_up_sync(FULL_WARP, incl, off);
                 if (lane >= off) incl += u;
             }
@@ -519,7 +520,7 @@ __global__ void __launch_bounds__(PART_WARPS * 32) part_kernel(const PartParams 
                 const bool h0 = rr >= b0, h1 = rr >= b1, h2 = rr >= b2;
                 rr -= h2 ? b2 : h1 ? b1 : h0 ? b0 : 0u;
                 const int t = 4 * ((g0 ? 1 : 0) + (g1 ? 1 : 0) + (g2 ? 1 : 0)) + (h0 ? 1 : 0) + (h1 ? 1 : 0) + (h2 ? 1 : 0);
-                yr = __shfl_sync(FULL_WARP, (uint32_t)(16 * lane + t) | (rr << 8), __ffs(win) - 1);
+                yr = __shfl_sync(FULL_WARP, (uint32_t)(rpl * lane + t) | (rr << 8), __ffs(win) - 1);
             }
             const int yy = (int)(yr & 255u), y = y0 + yy;
             rr = yr >> 8;
