@@ -147,15 +147,14 @@ __device__ __forceinline__ void ring_visit(uint64_t &S, uint64_t &H, int64_t &fl
     uint64_t C[RING_CLASSES];
     word lw, rw;
     ring_cumulative(C, lw, rw, s, hl, hr, Ld, DM, A);
-    for (int j = 0; j < k; ++j) {
+    auto step = [&](int j, auto draw_next) {
         const uint64_t tgt = cur.tgt;
         const bool ev = tgt < C[RING_CLASSES - 1]; // else a null step
         if (EXPO) {
             const int z = __clzll((long long)cur.V);
             kmcdev::mant_mul(clkM, clkE, cur.V << z, (int64_t)(10 - z));
         }
-        const bool last = j + 1 == k;
-        if (!last || more) cur = ring_draw(last ? 0u : (uint32_t)(j + 1), (uint32_t)(last ? d2 : d), last ? np2 : np, key);
+        draw_next();
         if (__any_sync(lanes, ev)) {
             uint64_t lo = 0, Ac = A[0];
             float inv = invA[0];
@@ -184,7 +183,11 @@ __device__ __forceinline__ void ring_visit(uint64_t &S, uint64_t &H, int64_t &fl
             H = ev ? h : H;
             ring_cumulative(C, lw, rw, s, hl, hr, Ld, DM, A);
         }
-    }
+    };
+    // (the last step stands by itself: the draws of the others are all of this
+    // visit's domain and phase)
+    for (int j = 0; j + 1 < k; ++j) step(j, [&]() { cur = ring_draw((uint32_t)(j + 1), (uint32_t)d, np, key); });
+    step(k - 1, [&]() { if (more) cur = ring_draw(0u, (uint32_t)d2, np2, key); });
     S ^= (uint64_t)(s ^ s0) << first;
 }
 
