@@ -208,8 +208,6 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
         at(Lay::AT + c) = A[c];
         at(Lay::MR + c) = __ldg(&P.rep_A[(size_t)r * RATE_WORDS + RATE_RECIP + c]);
     }
-#pragma unroll
-    for (int i = CHUNK; i < CHUNK + 8; ++i) at(Lay::TG + i) = ~0ull;
     at(Lay::CC) = 0;
     // Score constants of the lane's replica (scores only; registers): the
     // two fixed-point words X_c (2^-Q) and Y_c (2^-(Q+18)) of a_c dlog a_c /
@@ -342,34 +340,50 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
             const int total = has ? nf * k : 0;
             const int smax = (int)__reduce_max_sync(FULL_WARP, (unsigned)total);
 
-            // The draws of the next CHUNK steps (they depend only on the
-            // seed, the domain and the step counters): targets and step
-            // counters to shared memory, clock variates into the visit's
-            // product.  Step s = f k + j of the visit is step j of global
-            // phase np0 + f.
+            // The draws of the next CHUNK steps, or of the visit's last ones (they
+            // depend only on the seed, the domain and the step): targets to
+            // shared memory, clock variates into the visit's product.  Step s =
+            // f k + j of the visit is step j of global phase np0 + f.  Targets
+            // past the last step are ~0, and LOOK more so that a look never
+            // reads an earlier chunk's.
+            constexpr int LOOK = SCORES == SCORES_INLINE ? 8 : 4;
             uint64_t vM = 1ull << 63;
             int vE = 0;
+            // (step and phase are counted along where scores are formed in the event:
+            // 4 % faster there at k = 20 to 64 than from st; without scores st is
+            // the faster by 3 %)
+            constexpr bool COUNTED = SCORES == SCORES_INLINE;
+            uint32_t jcur = 0, fcur = 0;
+            auto chunk = [&](int base) { return min(CHUNK, (smax - base + 3) & ~3); };
             auto draw = [&](int base) {
+                const int n = chunk(base);
 #pragma unroll 4
-                for (int i = 0; i < CHUNK; ++i) {
-                    uint64_t t = ~0ull;
-                    const int st = base + i;
-                    if (st < total) {
-                        const int f = st >= k ? 1 : 0; // at most two phases fuse
-                        const uint64_t np = np0 + (uint64_t)f;
-                        const uint4 w = philox4x32_10(make_uint4((uint32_t)(st - (f ? k : 0)), d, (uint32_t)np,
-                                                                 (uint32_t)(np >> 32) & 0xFFFFFFu), key);
-                        t = (((uint64_t)w.y << 32) | w.x) >> 1;
-                        if (EXPO) {
-                            // clock variate v = V 2^-53 as a normalised mantissa
-                            // m / 2^63 times 2^(10 - z)
-                            const uint64_t V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
-                            const int z = __clzll((long long)V);
-                            mant_mul32(vM, vE, V << z, 10 - z);
+                for (int i = 0; i < n; ++i) {
+                        uint64_t t = ~0ull;
+                        const int st = base + i;
+                        if (st < total) {
+                            // (at most two phases fuse)
+                            const uint32_t f = COUNTED ? fcur : st >= k ? 1u : 0u;
+                            const uint32_t j = COUNTED ? jcur : (uint32_t)(st - (f ? k : 0));
+                            if (COUNTED && ++jcur == (uint32_t)k) {
+                                jcur = 0;
+                                ++fcur;
+                            }
+                            const uint64_t np = np0 + (uint64_t)f;
+                            const uint4 w = philox4x32_10(make_uint4(j, d, (uint32_t)np, (uint32_t)(np >> 32) & 0xFFFFFFu), key);
+                            t = (((uint64_t)w.y << 32) | w.x) >> 1;
+                            if (EXPO) {
+                                // clock variate v = V 2^-53 as a normalised mantissa
+                                // m / 2^63 times 2^(10 - z)
+                                const uint64_t V = ((((uint64_t)w.w << 32) | w.z) >> 11) + 1ull;
+                                const int z = __clzll((long long)V);
+                                mant_mul32(vM, vE, V << z, 10 - z);
+                            }
                         }
+                        at(Lay::TG + i) = t;
                     }
-                    at(Lay::TG + i) = t;
-                }
+#pragma unroll
+                for (int u = 0; u < LOOK; ++u) at(Lay::TG + n + u) = ~0ull;
             };
             draw(0); // before the halo wait
 
@@ -589,6 +603,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                         if (SCORES != SCORES_INLINE) work_off(base - CHUNK);
                         draw(base);
                     }
+                    const int n = chunk(base);
                     // Each lane jumps from real event to real event of its own
                     // domain (the steps between are null: App. A, the diagonal
                     // 1 - R/n_d); the warp runs as many rounds as its busiest lane.
@@ -603,7 +618,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                         if (SCORES == SCORES_INLINE) {
                             // every round in which some lane's state is scored costs
                             // FP64 time, so the lanes look on until each has an event
-                            while (i < CHUNK) {
+                            while (i < n) {
                                 uint64_t t[8];
                                 unsigned m = 0;
 #pragma unroll
@@ -625,7 +640,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                                 }
                                 i += 8;
                             }
-                            ev = i < CHUNK;
+                            ev = i < n;
                             // the null steps before this event, or up to the chunk's
                             // (or the visit's) end, all in the current state
                             const int end = ev ? i : min(CHUNK, total - base);
@@ -635,7 +650,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                                 null_steps(end - pos);
                             }
                             pos = ev ? i + 1 : CHUNK;
-                        } else if (i < CHUNK) {
+                        } else if (i < n) {
                             // One look at four steps per round: a lane that finds none
                             // in them sits out this round's events, as the lane with
                             // the most events sets the number of rounds.  Looking on,
@@ -656,7 +671,7 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                             const uint64_t q0 = (f & 1) ? t[1] : t[0], q1 = (f & 1) ? t[3] : t[2];
                             tgt = (f & 2) ? q1 : q0;
                         }
-                        if (!__any_sync(FULL_WARP, ev || i < CHUNK)) break;
+                        if (!__any_sync(FULL_WARP, ev || i < n)) break;
                         if (!ev) continue;
                         const int ist = i; // the event's step in the chunk
                         ++i;
@@ -818,7 +833,9 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                             at32(Lay::EV + (int)ne) = (uint32_t)ist | ((uint32_t)c << 5) | ((uint32_t)(y * LD + col) << 9);
                             ++ne;
                         }
-                        rates();
+                        // (with scores after the visit no rates after the lane's last step: 2 %
+                        // faster there at k = 16; without scores the branch costs 1 to 3 %)
+                        if (SCORES != SCORES_AFTER || i < total - base) rates();
                         corrupt |= bad;
                     }
                 }

@@ -179,3 +179,30 @@ def test_lane_groups_again_after_scores(Ld):
     lat.enable_grad(False)
     assert lat.launch() == before
     lat.close()
+
+
+@pytest.mark.parametrize("Ld", [16, 32])
+@pytest.mark.parametrize("ks", [[1, 2], [3, 5], [7, 8], [15, 16], [17, 33], [32, 40]])
+@pytest.mark.parametrize("scores", [False, True])
+def test_one_thread_per_domain_chunks(Ld, ks, scores):
+    """Visits that end inside, at and past a chunk of drawn steps, replicas of
+    both lengths in one warp, on the kernel of one thread per domain (a plan
+    made while scores are on keeps it when they go off)."""
+    import paper_1403_4674_gb300 as kmc
+    out = []
+    for plan in ((THREADS, 2, 2), WARP):
+        lat = kmc.Lattice([4 * Ld, 2 * Ld], Ld, 1, [8, 9])
+        lat.set_replica_params(k=ks)
+        lat.enable_grad(True)
+        lat.set_launch(*plan)
+        lat.enable_grad(scores)
+        assert lat.launch()[3] == plan[2]
+        lat.set_rates([0.25, 0.4], [0.02, -0.01])
+        obs = [lat.run(5, obs_every=2), lat.run(4, obs_every=2, schedule=kmc.KMC_SCHEDULE_FIXED,
+                                                time_mode=kmc.KMC_TIME_EXPECTED)]
+        lat.sync()
+        out.append((lat.spins.cpu().numpy(), *lat.domain_state()[:2], lat.score().cpu().numpy(),
+                    *[o[..., :3].cpu().numpy() for o in obs]))
+        lat.close()
+    for a, b in zip(*out):
+        assert np.array_equal(a, b)
