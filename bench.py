@@ -274,22 +274,22 @@ KERNEL_SOURCES = {"run_kernel": ("kmc_kernels.cuh",), "tpd_kernel": ("kmc_kernel
                   "tpdr_kernel": ("kmc_kernels.cuh", "kmc_tpdr.cuh"),
                   "tpdr64_kernel": ("kmc_kernels.cuh", "kmc_tpdr.cuh", "kmc_tpdr64.cuh")}
 NCU_KERNEL_SHA256 = {
-    "run_kernel": "90af89946413baa798ef8f01d0c7ce7e5b89bd1e0fd3acf67e20162380c30ad6",
-    "tpd_kernel": "5ab1c616b84c8ddd0b73b5d36543cc05ac331f4a3fd1470c4adebfb01c54cb6b",
-    "tpdr_kernel": "1c3f3576cd4a8b8ff68d0f0762f1031a3aaaa29eaceace994b1a14a8ede61ed8",
-    "tpdr64_kernel": "6b404b82601f0094f4f12fc6fe54ed1788cea73a5585c71dbbe6715c588f5699",
+    "run_kernel": "902a57337bf29bd8e150f87074669409eb47a1c7026088220d44e729ced6d7f7",
+    "tpd_kernel": "efbb6a42bacee890fdbf1ca90ec57187767bdee1136284fafc01fbf49ed0a20c",
+    "tpdr_kernel": "5f6d174a0b10e46dfa3a23d70381b5a996c74ce673decebaf4d9342d7c62934b",
+    "tpdr64_kernel": "ba3bbdd21d21a1a2e3d4ab179f02efbefbf0440b8883b3226eaa2d9811acc92e",
 }
 # instructions of one poll iteration: per warp iteration for the warp kernels
 # and the shared-memory thread kernel, per thread re-read for the 8x8 one
-INST_PER_POLL = {"run_kernel": 22.24, "tpd_kernel": 0.85, "tpdr_kernel": 28.38, "tpdr64_kernel": 32.44}
+INST_PER_POLL = {"run_kernel": 22.24, "tpd_kernel": 0.85, "tpdr_kernel": 35.33, "tpdr64_kernel": 38.54}
 NCU_COUNTS = {
     # (workload, kernel): (warp instructions, steps, poll iterations or None, DRAM bytes) of one launch
-    ("ising1024", "tpdr_kernel/rr"): (105701953345, 2580480000, 359845347, 6919936),
-    ("ising1024", "run_kernel"): (424586232478, 2580480000, 1572988655, 6585856),
-    ("grad", "tpdr_kernel"): (38819166107, 1310720000, 238780472, 5571840),
-    ("lattice8192", "tpdr64_kernel"): (18400662534, 524288000, 59494537, 11306240),
-    ("batched", "tpd_kernel/k16"): (37003135232, 2636876800, 160081004, 7619467264),
-    ("batched", "tpd_kernel/k32"): (73589388272, 5273753600, 637452521, 6709346304),
+    ("ising1024", "tpdr_kernel/rr"): (97103291436, 2580480000, 283359134, 7126272),
+    ("ising1024", "run_kernel"): (422455880649, 2580480000, 1580671157, 6534400),
+    ("grad", "tpdr_kernel"): (30952072445, 1310720000, 42958501, 5539328),
+    ("lattice8192", "tpdr64_kernel"): (16542301603, 524288000, 46415157, 11485952),
+    ("batched", "tpd_kernel/k16"): (28671384527, 2636876800, 230995487, 6310492928),
+    ("batched", "tpd_kernel/k32"): (53409055992, 5273753600, 496135401, 6166425600),
 }
 ISSUE_PER_SM_CYCLE = 4  # one warp instruction per scheduler per cycle, four schedulers
 

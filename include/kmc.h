@@ -265,9 +265,12 @@ kmc_status kmc_lr_observable(kmc_ctx *ctx, const double *rec_dev, int32_t stride
  * likelihood-ratio score of kmc_grad; the paper has no gradients, the score
  * is that of its uniformised chain, App. A).  The score-carrying kernels use
  * more registers; if they do not fit the current launch plan's shape, the
- * plan is rebuilt (requested plan first, else the default).  KMC_EINVAL
- * when turning scores on while the stream is capturing or when no plan fits
- * the score kernels; the setting then stays. */
+ * plan is rebuilt (requested plan first, else the default).  Lane groups
+ * carry no scores: they stay beside the plan that takes their place and are
+ * taken again when scores go off.  Runs already queued, and graphs captured
+ * before, keep their plan.  KMC_EINVAL when turning scores on while the stream
+ * is capturing or when no plan fits the score kernels; the setting then
+ * stays. */
 kmc_status kmc_enable_grad(kmc_ctx *ctx, int32_t enable);
 
 /* Re-initialise spins from the seeds (init as in kmc_create_lattice, or
@@ -355,12 +358,13 @@ kmc_status kmc_rate_table_error(const kmc_ctx *ctx, double *max_rel_err);
  *     grid's threads); an 8x8 domain is one 64-bit word, so the domain
  *     process runs in registers, with state, edge words and counters in
  *     global memory (L2).
- *     L_d = 16, 32, 64 with few domains (about two warps per scheduler at 8
- *     or more lanes per domain: 128 to 8192 domains on 152 SMs; scores off):
- *     8, 16 or 32 lanes per domain, by how many fill the SMs, the domain in
- *     the CTA's shared memory (0.8 to 2.3 KB); warps_per_cta as given, under
- *     KMC_LAUNCH_AUTO a whole replica per CTA where 16 warps hold it, else 4.
- *     `size` as below.
+ *     L_d = 16, 32, 64 with few domains (at most two warps per scheduler with
+ *     8, at L_d = 64 16, lanes per domain and two sets of domains per warp: up
+ *     to 9728 domains of L_d = 16, 32 and 4864 of L_d = 64 on 152 SMs; scores
+ *     off): 8, 16 or 32 lanes per domain, by how many fill the SMs, the domain
+ *     in the CTA's shared memory (0.8 to 2.3 KB); warps_per_cta as given, under
+ *     KMC_LAUNCH_AUTO 4, or 8 for small replicas with short visits.  `size` as
+ *     below.
  *     L_d = 16, 32, 64 otherwise: one domain per thread for the whole launch,
  *     with no warp collective on the step path, a warp
  *     holding 32 domains of one colour; the domain's rows, the class counts
@@ -385,12 +389,16 @@ kmc_status kmc_rate_table_error(const kmc_ctx *ctx, double *max_rel_err);
  *     (KMC_EINVAL while the stream is capturing).  For random colour orders
  *     of L_d = 16, 32, 64 without scores that is a GRID of lane groups where
  *     the domains are few, as above; the one-warp-per-domain plan stays
- *     beside it and is taken again by a run with fixed-time visits, also
- *     while the stream is capturing.
+ *     beside it.  Of two plans side by side a run takes the one that serves
+ *     it, also while the stream is capturing: the warp plan for fixed-time
+ *     visits and scores, the lane groups for the others.
  * In all plans a visit starts as soon as its four neighbours have finished
  * their visits of earlier colour phases (per-domain dataflow instead of a
  * barrier per phase; Sec. 2.2 lets non-interacting domains run at once); observation records are built from per-visit changes,
  * so no point of a launch synchronises a whole replica.
+ * Replacing a plan waits for the context's stream; a CUDA graph captured
+ * before keeps the plan that it was captured with (its tables stay until
+ * kmc_destroy).
  * warps_per_cta: 1..16.  Returns KMC_EINVAL if the plan cannot be scheduled
  * or the state does not fit in shared memory; the previous plan then stays.
  * Results do not depend on the plan, except the last bits of the FP64 domain

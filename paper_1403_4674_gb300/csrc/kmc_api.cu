@@ -776,6 +776,13 @@ kmc_status plan_groups(kmc_ctx *c, int G, int ns, int wpb, Plan &pl, bool interl
 //   8192 domains of 32x32, k = 8:  (8,2) 37.5  thread 42.7; 12288: (8,2) 47.8 thread 43.8
 //   1024 domains of 64x64, k = 8:  (32,2) 26.9 (16,1) 36.7 thread 61.4
 //   4096 domains of 64x64, k = 8:  (16,2) 50.5 thread 65.0; 9216: (16,2) 81.4 thread 77.9
+// and, from a lattice that has relaxed, (8,2) against thread:
+//   6400 domains of 16x16: k = 1 9.3, 12.7, k = 4 16.2, 21.2, k = 16 39.2, 50.8, k = 33 76.8, 111
+//   6400 domains of 32x32: k = 1 9.7, 12.4, k = 4 17.9, 21.1, k = 16 45.1, 50.0, k = 33 90.6, 110
+//   9216 domains of 32x32: k = 1 9.7, 12.7, k = 4 18.1, 21.4, k = 16 46.0, 49.9, k = 33 91.8, 110
+// The limit is two warps per scheduler at the fewest lanes and two sets per
+// warp: 9728 domains of 16x16 or 32x32 and 4864 of 64x64 on 152 SMs, fewer
+// where a replica's domains of a colour do not fill their sets.
 kmc_status plan_few_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
 {
     if (c->LD == 8) return fail(c, KMC_EINVAL, "no lane-group kernel for L_d = 8");
@@ -814,7 +821,9 @@ kmc_status plan_thread_domains(kmc_ctx *c, int wpb, Plan &pl, bool interleave)
 // busiest thread has domains; while the last round of the full grid is at
 // least half full the full grid is faster (every SM equally loaded: the
 // 512-replica batch, 1.6 domains per thread, 19.1 -> 18.4 ms), else the
-// threads are the domains of a colour divided by the rounds.
+// threads are the domains of a colour divided by the rounds (replicas of 128^2,
+// 1.1 and 1.3 domains per thread, k = 1, 4, 16: 22 % faster than the full grid;
+// from 1.4 to 2.8 the two are within 1.5 % on such alike replicas).
 int balanced_thread_ctas(const kmc_ctx *c, int wpb)
 {
     const int64_t per_colour = (c->n_dom + 3) / 4;

@@ -23,12 +23,17 @@
 // from the cumulative rates in every lane alike, the member's row from
 // 16 domain rows per lane of the rows' counts, its column from a
 // lane-parallel bit count, the five sites' classes from five lanes side by
-// side, the counts by shared-memory atomics.  About 1600 cycles an event
-// remain (rates 240, class 245, row 190-320, column 268, neighbours 143,
-// counts 295).  Measured at the start, after the windows and now: 50
-// trajectories of 100^2 in four stripes, k = 5, random order, 800 schedules
-// 3.22, 1.89, 1.34 ms; 500 of 12^2 in four blocks, k = 1, 4000 schedules
-// 11.1, 5.81, 3.54 ms.
+// side, the counts by shared-memory atomics.  Measured one visit after the
+// other, with the windows and now: 50 trajectories of 100^2 in four stripes,
+// k = 5, random order, 800 schedules 3.22, 1.89, 1.20 ms; 500 of 12^2 in four
+// blocks, k = 1, 4000 schedules 11.1, 5.81, 3.11 ms.  Section clocks of one
+// trajectory of each, cycles: an event 1630 and 1500 (of it about: rates 240,
+// class 245, row 190-320, column 268, neighbours 143, counts 295), a window
+// 1030 and 2120 (its orders and draws 730 and 1350, the last look that finds
+// no event 240, records 70 and 520), staging and writing back 130,000 and
+// 21,000 once.  16,000 steps are 500 windows with about 1000 events (one step
+// in 16, the stripes) or 2400 (one in 6.6, the blocks), so events are 0.8 of
+// 1.2 ms and 1.8 of 3.1 ms.
 //
 // Step target (n_d not a power of two): P = 63 - ceil(log2 n_d),
 // M = n_d 2^P, target = floor(X M / 2^64) for X = w0 | w1<<32; with n_d a
@@ -190,8 +195,8 @@ __device__ __forceinline__ int site_class(const uint32_t *rows, int x, int y, in
 // event of the whole window, in whichever visit it falls; every lane has
 // formed its own step's class and member index by then, and after the event
 // each lane forms its domain's rates again from the class counts in shared
-// memory.  What a trajectory costs is thus one chain per real event (about
-// one step in eight at T = 2.4) and a fixed part per 32 steps, where a loop
+// memory.  What a trajectory costs is thus one chain per real event (at T =
+// 2.4 one step in 6 to 16) and a fixed part per 32 steps, where a loop
 // over visits paid a fixed part per visit.  Records between the window's
 // steps come from per-lane copies of the bond sum and the magnetisation and
 // from the inclusive products of the clock variates; the lanes at whose

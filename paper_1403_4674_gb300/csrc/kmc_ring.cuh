@@ -22,8 +22,9 @@
 // short rather than skipped: the visit works on a 32-bit window of its domain
 // (below), and the next step's Philox block, which depends on nothing, is
 // drawn in line with the event so that its multiplies fill the event's waits.
-// Measured: 48000 x 8 spins, k = 5, 40 sweeps with ensemble sums 1031 -> 769 us;
-// 6000 x 64 spins, k = 10, 10 sweeps with records 931 -> 736 us.
+// Measured against a step of draw, then event, on 64-bit words: 48000 x 8
+// spins, k = 5, 40 sweeps with ensemble sums 1031 -> 732 us; 6000 x 64 spins,
+// k = 10, 10 sweeps with records 931 -> 651 us.
 #pragma once
 
 #include <cstdint>
@@ -185,7 +186,8 @@ __device__ __forceinline__ void ring_visit(uint64_t &S, uint64_t &H, int64_t &fl
         }
     };
     // (the last step stands by itself: the draws of the others are all of this
-    // visit's domain and phase)
+    // visit's domain and phase, whose share of the first Philox round then is
+    // formed once; with one loop that chose per step 770 and 737 us)
     for (int j = 0; j + 1 < k; ++j) step(j, [&]() { cur = ring_draw((uint32_t)(j + 1), (uint32_t)d, np, key); });
     step(k - 1, [&]() { if (more) cur = ring_draw(0u, (uint32_t)d2, np2, key); });
     S ^= (uint64_t)(s ^ s0) << first;

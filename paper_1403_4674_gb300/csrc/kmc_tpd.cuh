@@ -154,15 +154,18 @@ __device__ __forceinline__ void tpd_flush(const RunParams &P, bool on, const ulo
 // to shared memory), before its halo is there, and every round of events lets
 // each lane look once at its own next three targets: a lane with an event takes
 // it, one without sits out the round, and the warp needs about half as many
-// rounds as steps.  Before that the domain's words are asked for; counters are
-// added without reading them, and C_{c-1} is kept in shared memory.  512
-// uneven replicas, 60 schedules, records every 10, on 456 CTAs: at k = 4 5.93
-// -> 5.89 ms, k = 16 16.85 -> 14.41, k = 32 31.65 -> 26.27 against one step per
-// round with the next step's draw in line with the event; k = 1 3.64 -> 3.76.
-// Looks at two targets 5.80 / 14.79 / 27.31 (k = 4 / 16 / 32), at four 6.03 /
-// 14.65 / 26.64, lanes that look on until they find their next event no faster
-// than one step per round; four CTAs per SM at 128 registers 7.72 / 18.55 /
-// 33.68.
+// rounds as steps.  Before that the domain's words and the halo are asked for;
+// counters are added without reading them, and C_{c-1} is kept in shared
+// memory.  512 uneven replicas, 60 schedules, records every 10, on 456 CTAs, at
+// k = 1 / 4 / 16 / 32: 3.64 / 5.93 / 16.85 / 31.65 ms with one step per round
+// and the next step's draw in line with the event, 3.77 / 5.89 / 14.37 / 26.25
+// drawn first and three looked at, 3.61 / 5.59 / 14.01 / 25.71 with the halo
+// asked for before the draws and no rates after a visit's last step (one 128^2
+// lattice at k = 1, where every warp runs the phases in step: 13.4, 16.1, 12.9
+// us a schedule).  Of drawn first: looks at two targets 5.80 / 14.79 / 27.31
+// (k = 4 / 16 / 32), at four 6.03 / 14.65 / 26.64, lanes that look on until they
+// find their next event no faster than one step per round; four CTAs per SM at
+// 128 registers 7.72 / 18.55 / 33.68.
 template <bool EXPO>
 __global__ void __launch_bounds__(128, 3) tpd_kernel(const RunParams P)
 {

@@ -40,7 +40,9 @@
 // scan for the next event in every round, 6.84 with the list, 5.75 with one
 // look at four targets per round (at eight 6.05, at two 5.96).  256 lattices
 // of 256^2 with scores, k = 8, 100 schedules: 7.43 ms with the scores in the
-// event, 4.06 with them worked off after it (4.07 without scores).
+// event, 4.06 with them worked off after it (4.07 without scores).  Chunks of
+// drawn steps that end with the visit: 12 lattices of 1024^2 at k = 1 16.1 ->
+// 13.2 us a schedule, at k = 4 24.7 -> 22.0, at k = 16 50.6 -> 49.4.
 //
 // Scope: palindromic and fixed colour schedules, exponential and expected
 // clocks, per-replica k, records at schedule endpoints or every colour pass,
@@ -550,9 +552,9 @@ __global__ void __launch_bounds__(128) tpdr_kernel(const RunParams P)
                 // magnetisation and the scores is worked off from the list of the
                 // chunk's events (with scores also the counts before each), after
                 // the visit's edges are published: the neighbours do not wait for
-                // it.  With scores this is most of a visit's work: 256 x 256^2,
-                // 100 schedules, k = 8 7.43 -> 4.11 ms, k = 2 6.09 -> 3.89, k = 16
-                // 12.1 -> 9.7.  Visits of more than 32 steps (k = 33: 24 % slower
+                // it.  With scores this is most of a visit's work: 256 x 256^2 in
+                // us a schedule, formed in the event -> after it, k = 1 20.2 -> 12.6,
+                // k = 4 37.8 -> 20.1, k = 8 54.0 -> 28.9, k = 16 78 -> 65.  Visits of more than 32 steps (k = 33: 24 % slower
                 // with lists of 16 steps, and longer ones do not fit) form their
                 // scores event by event.
                 auto work_off = [&](int base) {

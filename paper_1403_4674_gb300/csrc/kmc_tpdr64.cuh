@@ -288,10 +288,9 @@ __global__ void __launch_bounds__(128) tpdr64_kernel(const RunParams P)
             const int smax = (int)__reduce_max_sync(FULL_WARP, (unsigned)total);
 
             // The draws of the next CHUNK steps (they depend only on the
-            // seed, the domain and the step counters): targets and step
-            // counters to shared memory, clock variates into the visit's
-            // product.  Step s = f k + j of the visit is step j of global
-            // phase np0 + f.
+            // seed, the domain and the step): targets to shared memory, clock
+            // variates into the visit's product.  Step s = f k + j of the visit
+            // is step j of global phase np0 + f.
             uint64_t vM = 1ull << 63;
             int vE = 0;
             auto draw = [&](int base) {
