@@ -25,7 +25,7 @@
 //
 // Measured, whole calls: 1024^2 at L_d = 32, k = 4, 200 schedules 3.26 -> 1.07
 // ms (before: one lane per domain); 64^2 at L_d = 16, k = 1, 1000 schedules
-// 9.58 -> 5.09 ms; 16 lattices of 256^2 at L_d = 16 in random colour order, 40
+// 9.58 -> 5.1 to 5.5 ms; 16 lattices of 256^2 at L_d = 16 in random colour order, 40
 // schedules 1.25 -> 0.64 ms (before: one warp per domain).  ncu, 1024 domains
 // of 32x32 at G = 32: 0.9 warps per scheduler, 28 % of the issue slots, 31 of
 // 32 threads active, stalls led by fixed-latency waits (1.2 cycles per
